@@ -59,7 +59,8 @@ bool alloc_sim(Sim &S, DevMem &mem, int n, int nsub) {
   S.rc = mem.get<double>(np); S.A = mem.get<double>(np);
   S.T = mem.get<u64>(np); S.rcsq = mem.get<u64>(np);
   S.afar = mem.get<double>(3 * np);
-  S.part = mem.get<double>(nt * nt * 2 * 96);
+  kick_split(S.npad, num_sms(), &S.kch, &S.kchunk);
+  S.part = mem.get<double>(nt * std::max(2 * nt, (size_t)S.kch) * 96);
   S.pkick = mem.get<double>(nt * 3); S.pfin = mem.get<double>(nt * 3);
   S.cbm = mem.get<unsigned>(np * W); S.rowany = mem.get<unsigned>(W);
   S.ccnt = mem.get<int>(np); S.clist = mem.get<int>(np * CCAP);
@@ -69,7 +70,7 @@ bool alloc_sim(Sim &S, DevMem &mem, int n, int nsub) {
   S.fail = mem.get<int>(np); S.nfail = mem.get<int>(1);
   S.gstart = mem.get<int>(np + 1); S.gmem = mem.get<int>(np); S.ngroups = mem.get<int>(1);
   S.big = mem.get<int>(np); S.nbig = mem.get<int>(1);
-  // kick work list: for each tile I, the diagonal tile, then both halves of every J > I
+  // precise kick work list: for each tile I, the diagonal tile, then both halves of every J > I
   std::vector<int> items;
   for (int I = 0; I < S.nt; ++I) {
     items.push_back(I | (I << 10));
@@ -80,8 +81,7 @@ bool alloc_sim(Sim &S, DevMem &mem, int n, int nsub) {
   }
   S.nitems = (int)items.size();
   S.items = mem.get<int>(items.size());
-  // two warps per sub-partition: the second hides the first's FP64 dependency waits (measured at
-  // N = 2048: one warp 102.6 us, two 88.3 us, three 89.8 us, four 90.2 us per kick)
+  // two warps per sub-partition: the second hides the first's FP64 dependency waits
   const int target = 8 * num_sms();
   S.nwarps = S.nitems < target ? S.nitems : target;
   S.flags = mem.get<int>(4); S.status = mem.get<int>(1);
@@ -241,7 +241,7 @@ int first_kick(genga_ctx *c) {
     return GENGA_OK;
   }
   launch_kick(S, c->P, false, c->prm.precise_div != 0, st);
-  launch_fin(S, c->P, FIN_INIT, 0.0, 0.0, nullptr, st);
+  launch_fin(S, c->P, FIN_INIT, c->prm.precise_div != 0, 0.0, 0.0, nullptr, st);
   if (c->tpmode) {
     CK(cudaMemsetAsync(c->T.npairs, 0, sizeof(unsigned), st));
     CK(cudaMemsetAsync(c->T.bsnext, 0, (4 + 4 * TP_BS_MAXBLOCKS) * sizeof(unsigned), st));
@@ -311,7 +311,7 @@ void enqueue_step(genga_ctx *c, cudaStream_t st) {
   const TPSet &T = c->T;
   launch_rcrit(S, P, std::fabs(dt), 1, st);
   launch_kick(S, P, true, precise, st);  // runs only if the critical radii grew too much
-  launch_fin(S, P, FIN_OPEN, 0.5 * c->w[0] * dt, 0.0, nullptr, st);
+  launch_fin(S, P, FIN_OPEN, precise, 0.5 * c->w[0] * dt, 0.0, nullptr, st);
   for (int j = 0; j < c->nsub; ++j) {
     const double tau = c->w[j] * dt;
     const double hcm2 = j > 0 ? 0.5 * c->w[j - 1] * dt * inv_m0 : 0.0;
@@ -357,7 +357,7 @@ void enqueue_step(genga_ctx *c, cudaStream_t st) {
     launch_kick(S, P, inner, precise, st, inner);
     if (c->profiling) cudaEventRecordWithFlags(c->kev[2 * j + 1], st, cudaEventRecordExternal);
     const double h2 = (j + 1 < c->nsub) ? 0.5 * c->w[j + 1] * dt : 0.0;
-    launch_fin(S, P, inner ? FIN_CLOSE_ALL : FIN_CLOSE, 0.5 * tau, h2, nullptr, st);
+    launch_fin(S, P, inner ? FIN_CLOSE_ALL : FIN_CLOSE, precise, 0.5 * tau, h2, nullptr, st);
     if (tp) {  // join; the particles' BS and every particle's closing kick (after the last substep
                // with their last Sun drift, from the massive momentum before the closing kick)
       cudaStreamWaitEvent(st, c->ev_join, 0);
@@ -1500,7 +1500,7 @@ int genga_phase_kick(int n, double G, double pc, int kmode, int precise_div, con
   if (mem.err != cudaSuccess) { mem.release(); return GENGA_ENOMEM; }
   launch_soa_setup(S, P, m, alive, x, nullptr, rc, n, st);
   launch_kick(S, P, false, precise_div != 0, st);
-  launch_fin(S, P, FIN_INIT, 0.0, 0.0, aout, st);
+  launch_fin(S, P, FIN_INIT, precise_div != 0, 0.0, 0.0, aout, st);
   soa_copy(a, n, aout, S.npad, n, st);
   launch_bitmap_pairs(S.cbm, S.npad, S.W, tmp, S.npad * (S.npad - 1) / 2 + 1, dcnt, st);
   int cnt = 0;

@@ -80,7 +80,7 @@ struct Sim {
   double *rc, *A;                // [npad]; A = 1/(0.9 rc)
   u64 *T, *rcsq;                 // [npad]; bits of (pc rc)^2 and rc^2
   double *afar;                  // [3 npad] far-field accelerations of the last kick
-  double *part;                  // [nt * nt * 2 * 3 * 32] kick partial sums
+  double *part;                  // [nt * max(2 nt, kch) * 3 * 32] kick partial sums
   double *pkick, *pfin;          // [nt * 3] per-tile momentum partials
   unsigned *cbm, *rowany;        // candidate bitmap [npad * W], row-nonempty bits [W]
   int *ccnt, *clist;             // per-body candidate count [npad] and partners [npad * CCAP]
@@ -89,7 +89,8 @@ struct Sim {
   int *fail, *nfail;             // Kepler-fallback bodies [npad] and count
   int *gstart, *gmem, *ngroups;  // groups
   int *big, *nbig;               // groups with gbig or more members (the cluster kernel's work list)
-  int *items, nitems, nwarps;    // kick work list
+  int *items, nitems, nwarps;    // work list of the precise kick
+  int kch, kchunk;               // fixed-point kick: chunks of partners per tile, partners per chunk
   // batched mode (independent systems; null in the single-system mode)
   int nsys;
   int *sys_of, *sys_start;       // system of each body [npad]; body range of each system [nsys+1]

@@ -14,10 +14,12 @@ void launch_rcrit(const Sim &S, const DevParams &P, double tau_abs, int check_re
 // full: every pair with its changeover weight, no candidates recorded; runs only when the opening
 // kick must be recomputed, unless force (then always, also recording the momentum for the Sun drift)
 void launch_kick(const Sim &S, const DevParams &P, bool full, bool precise, cudaStream_t st, bool force = false);
-void launch_fin(const Sim &S, const DevParams &P, FinMode mode, double h1, double h2, double *aout,
+// precise: which pair kernel wrote the partial sums
+void launch_fin(const Sim &S, const DevParams &P, FinMode mode, bool precise, double h1, double h2, double *aout,
                 cudaStream_t st);
 void launch_hc(const Sim &S, double hcm, cudaStream_t st);
-int kick_grid(const Sim &S);
+// the fixed-point pair kernel's chunks of partners per tile, partners per chunk
+void kick_split(int npad, int sms, int *chunks, int *chunk);
 
 // step.cu
 void launch_drift(const Sim &S, const DevParams &P, double tau, double hcm1, double hcm2,

@@ -1,12 +1,12 @@
 // kick.cu -- critical radii (Eq. rcrit), the K-weighted pairwise kick with the prechecker
 // (Eq. Hb, Sect. 2.2 and 3.2 "Kick"), and its per-body finalisation (KickA/KickB reuse).
 //
-// The pair kernel evaluates every unordered pair once (Newton's third law) on 32x32 body tiles:
-// each lane holds one body i of tile I, the 32 bodies of tile J rotate through the lanes by warp
-// shuffles, and the j-side accumulators rotate with them. A work item is half of a tile pair
-// (16 ring steps), which balances ~6.7 items per sub-partition at N = 2048. Partial sums go to a
-// per-(tile, partner tile, half) buffer that the finalisation sums in a fixed order, so results
-// are bitwise reproducible. Per unordered pair the kernel issues 20 FP64 instructions.
+// Two pair kernels. k_kick_fx (the default) evaluates each body's pull from every partner in 64-bit
+// fixed point on the integer and FP32 pipes (fxpair.cuh). k_kick_precise (precise_div = 1: IEEE square
+// root and division) evaluates every unordered pair once in FP64. Both leave partial sums per body
+// tile in a fixed layout that the finalisation sums in a fixed order, so results are bitwise
+// reproducible.
+#include "fxpair.cuh"
 #include "genga_launch.h"
 
 namespace genga {
@@ -50,11 +50,15 @@ __global__ void k_rcrit(Sim S, DevParams P, double tau_abs, int check_reuse) {
 }
 
 // ---------------------------------------------------------------------------------------------
-// Pair kernel. FULL: all pairs with inline changeover weights (used only when the critical
-// radii grew too much for reuse); otherwise far pairs only, candidates recorded in the bitmap.
+// Pair kernel with IEEE square root and division (precise_div = 1). FULL: all pairs with inline
+// changeover weights (used only when the critical radii grew too much for reuse); otherwise far
+// pairs only, candidates recorded in the bitmap. Every unordered pair once (Newton's third law) on
+// 32x32 body tiles: each lane holds one body i of tile I, the 32 bodies of tile J rotate through the
+// lanes by warp shuffles, and the j-side sums rotate with them. A work item is half of a tile pair
+// (16 ring steps); its partial sums go to a slot per (tile, partner tile, half).
 // ---------------------------------------------------------------------------------------------
-template <bool FULL, bool PRECISE>
-__global__ void __launch_bounds__(128) k_kick(Sim S, DevParams P, int force) {
+template <bool FULL>
+__global__ void __launch_bounds__(128) k_kick_precise(Sim S, DevParams P, int force) {
   if (FULL && !force && S.flags[0] == 0) return;
   // a full opening kick after a new state also records the precheck candidates (flag 3)
   const bool record = FULL && !force && S.flags[3] != 0;
@@ -109,9 +113,7 @@ __global__ void __launch_bounds__(128) k_kick(Sim S, DevParams P, int force) {
       const bool act = !diag || s < 15 || lane < 16;
       const double dx = xj - xi, dy = yj - yi, dz = zj - zi;
       const double r2 = __fma_rn(dz, dz, __fma_rn(dy, dy, __dmul_rn(dx, dx)));
-      double w3;
-      if (PRECISE) w3 = 1.0 / (r2 * sqrt(r2));
-      else w3 = rcube_refined(r2);
+      const double w3 = 1.0 / (r2 * sqrt(r2));
       double gj = act ? gmj : 0.0, gi = act ? gmi : 0.0;
       const u64 rb = dbits(r2);
       if (FULL) {
@@ -160,6 +162,262 @@ __global__ void __launch_bounds__(128) k_kick(Sim S, DevParams P, int force) {
       pj[0] = ajx; pj[32] = ajy; pj[64] = ajz;
     }
   }
+}
+
+// ---------------------------------------------------------------------------------------------
+// Fixed-point pair kernel. A CTA holds TW tiles of 32 bodies, a warp each, one body a lane, and CW
+// chunks of at most 64 partners in shared memory (TW CW = 8 warps); a warp sums one tile's pulls
+// from one chunk into that (tile, chunk)'s slot. FULL and the candidates as in k_kick_precise; every
+// body records its own row of the bitmap.
+//
+// Pass 1 separates the near partners -- inside the precheck radius, or closer than the fixed-point
+// grid resolves, or the body itself -- into a bit mask and bounds the sum of the others. Pass 2 sums
+// the far pulls. The near pairs of the warp are then listed and taken one a lane in FP64 with the
+// exact decision arithmetic. A CTA with a number the fixed-point form cannot hold (not finite, a
+// negative mass) takes every pair as near.
+//
+// No Newton's third law: the sums of the j side would rotate through the lanes with 24 more
+// shuffled words a pair (4 cycles each), as much as evaluating the pair once more.
+// ---------------------------------------------------------------------------------------------
+constexpr int KX_WARPS = 8;
+constexpr int KX_CTAS = 3;  // CTAs per SM (80 registers; measured at N = 2048: two 33.9 us, three 33.7 us a kick)
+constexpr int KX_LIST = 96;  // near pairs of a warp taken together; more: each lane takes its own in turn
+constexpr int KX_SMALL = 8;  // partners a chunk for fewer than 8 tiles
+template <int CAP>
+struct KxShared {
+  float4 h[CAP], m[CAP];  // position in single precision (h + m); .w: mass, its exponent
+  longlong2 xy[CAP], zM[CAP];
+  float lim[CAP];
+};
+struct KxList {  // near pairs: body lane << 8 | partner, and their pulls
+  int e[KX_LIST];
+  double f[3][KX_LIST];
+};
+
+// max(T, grid limit) as the first pass's limit on rough r^2 (units of 2^(2E - 60)), rounded up by
+// 2^-10 (rough r^2 is within 2^-12).
+__device__ __forceinline__ float kx_limit(u64 T, int E) {
+  const float t = scalbnf(d2f_safe(__longlong_as_double((long long)T)), 60 - 2 * E);
+  return fmaxf(t, fx::FX_RMIN2) * 1.001f;
+}
+__device__ __forceinline__ float kx_norm2(double x, double y, double z) {  // |x|^2, rounded up
+  const float a = d2f_safe(x), b = d2f_safe(y), c = d2f_safe(z);
+  return fmaf(c, c, fmaf(b, b, a * a)) * 1.000002f;
+}
+__device__ __forceinline__ bool kx_odd(double x) { return fx::expo(x) == 0x7ff; }
+
+// The pair (i, j) in FP64: records a candidate, returns the pull's factor (0: nothing to add here).
+template <bool FULL>
+__device__ __forceinline__ double kx_near(const Sim &S, const DevParams &P, int i, int j, bool record, double &dx,
+                                          double &dy, double &dz) {
+  const int np = S.npad;
+  if (j == i || !S.alive[j]) return 0.0;
+  dx = S.x[j] - S.x[i]; dy = S.x[np + j] - S.x[np + i]; dz = S.x[2 * np + j] - S.x[2 * np + i];
+  const double r2 = __fma_rn(dz, dz, __fma_rn(dy, dy, __dmul_rn(dx, dx)));
+  const u64 rb = dbits(r2);
+  const bool cand = rb < umax64(S.T[i], S.T[j]);
+  if (record && cand) {
+    const int ki = atomicAdd(&S.ccnt[i], 1);
+    atomicOr(&S.cbm[(size_t)i * S.W + (j >> 5)], 1u << (j & 31));
+    atomicOr(&S.rowany[i >> 5], 1u << (i & 31));
+    if (ki < CCAP) S.clist[i * CCAP + ki] = j;
+    if (i < j) atomicAdd((unsigned long long *)&S.counters[C_CAND], 1ULL);
+  }
+  if (!FULL && cand) return 0.0;  // handled by the near pass
+  double g = S.gm[j] * rcube_refined(r2);
+  if (FULL && rb < umax64(S.rcsq[i], S.rcsq[j])) {  // inside the changeover zone: weight K
+    double wB, wA;
+    changeover_w(r2 * rsqrt_refined(r2), pmin(S.A[i], S.A[j]), P.kmode, wB, wA);
+    g *= wB;
+  }
+  return g;
+}
+
+template <bool FULL, int TW>
+__global__ void __launch_bounds__(32 * KX_WARPS, KX_CTAS) k_kick_fx(Sim S, DevParams P, int force) {
+  if (FULL && !force && S.flags[0] == 0) return;
+  const bool record = FULL ? (!force && S.flags[3] != 0) : true;
+  constexpr int CW = KX_WARPS / TW, CAP = TW == 8 ? fx::FX_CHUNK : KX_SMALL;
+  __shared__ KxShared<CAP> smem[CW];
+  __shared__ KxList slist[KX_WARPS];
+  __shared__ int s_n2, s_me[CW];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int np = S.npad, C = S.kch, nt = S.nt;
+  const double *__restrict__ X = S.x;
+  const int gwarp = blockIdx.x * KX_WARPS + wid;
+  if ((!FULL || force) && gwarp < nt) {  // per-tile momentum before the closing kick (second Sun drift)
+    const int i = gwarp * 32 + lane;
+    const double mi = S.m[i];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const double p = warp_sum(mi * S.v[c * np + i]);
+      if (lane == 0) S.pkick[gwarp * 3 + c] = p;
+    }
+  }
+  const int tgroups = (nt + TW - 1) / TW;
+  const int I = (blockIdx.x % tgroups) * TW + wid % TW, cw = wid / TW, c0 = (blockIdx.x / tgroups) * CW + cw;
+  const bool on = I < nt && c0 < C;
+  if (tid == 0) s_n2 = 0;
+  if (tid < CW) s_me[tid] = -2000;
+  // own body; partners (one a thread, twice over when the CTA holds more than four chunks)
+  const int i = min(I, nt - 1) * 32 + lane;
+  const bool ali = on && S.alive[i] != 0;
+  const double xi = ali ? X[i] : 0.0, yi = ali ? X[np + i] : 0.0, zi = ali ? X[2 * np + i] : 0.0;
+  const u64 Ti = ali ? S.T[i] : 0ULL;
+  constexpr int NB = CW * CAP, PB = (NB + 32 * KX_WARPS - 1) / (32 * KX_WARPS);
+  double bx[PB], by[PB], bz[PB], bg[PB];
+  u64 bT[PB];
+  float n2 = kx_norm2(xi, yi, zi);
+  bool odd = kx_odd(xi) || kx_odd(yi) || kx_odd(zi);
+#pragma unroll
+  for (int k = 0; k < PB; ++k) {
+    const int q = tid + 32 * KX_WARPS * k, ch = (blockIdx.x / tgroups) * CW + q / CAP, u = q % CAP;
+    const int j = ch * S.kchunk + u;
+    const bool al = q < NB && ch < C && u < S.kchunk && j < np && S.alive[j] != 0;
+    bx[k] = al ? X[j] : 0.0; by[k] = al ? X[np + j] : 0.0; bz[k] = al ? X[2 * np + j] : 0.0;
+    bg[k] = al ? S.gm[j] : 0.0;
+    bT[k] = al ? S.T[j] : 0ULL;
+    n2 = fmaxf(n2, kx_norm2(bx[k], by[k], bz[k]));
+    odd |= kx_odd(bx[k]) || kx_odd(by[k]) || kx_odd(bz[k]) || kx_odd(bg[k]) || (long long)dbits(bg[k]) < 0;
+  }
+  __syncthreads();
+  // common scale: |x| < 2^E; per chunk the largest mass exponent
+  const int wn2 = __reduce_max_sync(0xffffffffu, __float_as_int(n2));
+  if (lane == 0) atomicMax(&s_n2, wn2);
+#pragma unroll
+  for (int k = 0; k < PB; ++k) {
+    const int q = tid + 32 * KX_WARPS * k;
+    if (q >= NB) continue;
+    u64 M;
+    int me;
+    fx::set_mass(bg[k], M, me);
+    if (M) atomicMax(&s_me[q / CAP], me);
+  }
+  odd = __syncthreads_or(odd) || s_n2 >= 0x7f000000;
+  const int E = odd ? 0 : ((s_n2 >> 23) - 127 + 2) >> 1;
+#pragma unroll
+  for (int k = 0; k < PB; ++k) {
+    const int q = tid + 32 * KX_WARPS * k;
+    if (q >= NB) continue;
+    KxShared<CAP> &sm = smem[q / CAP];
+    const int u = q % CAP;
+    fx::Pos p;
+    u64 M;
+    int me;
+    fx::set_pos(p, odd ? 0.0 : bx[k], odd ? 0.0 : by[k], odd ? 0.0 : bz[k], E);
+    fx::set_mass(odd ? 0.0 : bg[k], M, me);
+    sm.h[u] = make_float4(p.hx, p.hy, p.hz, fx::mass_f(M, me, s_me[q / CAP]));
+    sm.m[u] = make_float4(p.mx, p.my, p.mz, __int_as_float(me));
+    sm.xy[u] = make_longlong2(p.X, p.Y);
+    sm.zM[u] = make_longlong2(p.Z, (long long)M);
+    sm.lim[u] = kx_limit(bT[k], E);
+  }
+  fx::Pos pi;
+  fx::set_pos(pi, odd ? 0.0 : xi, odd ? 0.0 : yi, odd ? 0.0 : zi, E);
+  const float limi = odd ? __int_as_float(0x7f800000) : kx_limit(Ti, E);
+  __syncthreads();
+  if (!on) return;
+  const KxShared<CAP> &sm = smem[cw];
+  const int j0 = c0 * S.kchunk, cnt = min(S.kchunk, np - j0);  // at least one partner
+  // pass 1: near partners, bound of the far sum
+  unsigned near[2] = {0u, 0u};
+  float B = 0.0f;
+#pragma unroll
+  for (int w = 0; w < 2; ++w) {
+    const int n = min(cnt - 32 * w, 32);
+#pragma unroll 4
+    for (int k = 0; k < n; ++k) {
+      const float4 h = sm.h[32 * w + k];
+      const float r2 = fx::rough_r2(pi, h.x, h.y, h.z);
+      if (r2 >= fmaxf(limi, sm.lim[32 * w + k])) B = fmaf(h.w, fx::frcp(r2), B);
+      else near[w] |= 1u << k;
+    }
+  }
+  // pass 2: the far pulls
+  const int A = fx::units(B, s_me[cw]);
+  fx::Acc acc;
+  fx::clear(acc);
+#pragma unroll
+  for (int w = 0; w < 2; ++w) {
+    const int n = min(cnt - 32 * w, 32);
+    for (int k0 = 0; k0 < n; k0 += fx::FX_FLUSH) {
+      const int k1 = min(n, k0 + fx::FX_FLUSH);
+#pragma unroll 2
+      for (int k = k0; k < k1; ++k) {
+        const float4 h = sm.h[32 * w + k], m = sm.m[32 * w + k];
+        const longlong2 a = sm.xy[32 * w + k], b = sm.zM[32 * w + k];
+        const fx::Pos pj = {a.x, a.y, b.x, h.x, h.y, h.z, m.x, m.y, m.z};
+        fx::pull(pi, pj, (u64)b.y, __float_as_int(m.w), A, !((near[w] >> k) & 1u), acc);
+      }
+      fx::flush(acc);
+    }
+  }
+  double ax = fx::value(acc.h[0], acc.l[0], A, E), ay = fx::value(acc.h[1], acc.l[1], A, E),
+         az = fx::value(acc.h[2], acc.l[2], A, E);
+  // the near pairs in FP64: listed by (body, partner), one a lane, added per body in partner order
+  {
+    const unsigned self = I * 32 + lane - j0;  // the body itself is not a pair
+    if (self < 32u) near[0] &= ~(1u << self);
+    else if (self < 64u) near[1] &= ~(1u << (self - 32u));
+    if (!ali) { near[0] = 0u; near[1] = 0u; }
+  }
+  const int nn = __popc(near[0]) + __popc(near[1]);
+  int incl = nn;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += t;
+  }
+  const int total = __shfl_sync(0xffffffffu, incl, 31);
+  if (total > 0 && total <= KX_LIST) {
+    KxList &L = slist[wid];
+    int at = incl - nn;
+#pragma unroll
+    for (int w = 0; w < 2; ++w)
+      for (unsigned bits = near[w]; bits; bits &= bits - 1) L.e[at++] = lane << 8 | (32 * w + __ffs(bits) - 1);
+    __syncwarp();
+    for (int k = lane; k < total; k += 32) {
+      double dx = 0.0, dy = 0.0, dz = 0.0;
+      const double g = kx_near<FULL>(S, P, I * 32 + (L.e[k] >> 8), j0 + (L.e[k] & 255), record, dx, dy, dz);
+      L.f[0][k] = g * dx; L.f[1][k] = g * dy; L.f[2][k] = g * dz;
+    }
+    __syncwarp();
+    for (int k = incl - nn; k < incl; ++k) { ax += L.f[0][k]; ay += L.f[1][k]; az += L.f[2][k]; }
+  } else if (total > 0) {
+#pragma unroll
+    for (int w = 0; w < 2; ++w)
+      for (unsigned bits = near[w]; bits; bits &= bits - 1) {
+        double dx = 0.0, dy = 0.0, dz = 0.0;
+        const double g = kx_near<FULL>(S, P, i, j0 + 32 * w + __ffs(bits) - 1, record, dx, dy, dz);
+        ax += g * dx; ay += g * dy; az += g * dz;
+      }
+  }
+  double *p = S.part + ((size_t)I * C + c0) * 96 + lane;
+  p[0] = ali ? ax : 0.0; p[32] = ali ? ay : 0.0; p[64] = ali ? az : 0.0;
+}
+
+// The fixed-point kernel's split of a tile's partners: chunks per tile, partners per chunk. About 8
+// KX_CTAS warps per SM, at least 8 partners a chunk (below that the set-up of a warp outweighs its
+// loop), at most 64 (the bit masks). Up to 1024 bodies at most 2048 chunks in all (the partial-sum
+// slots of the static scratch).
+void kick_split(int npad, int sms, int *chunks, int *chunk) {
+  const int nt = npad / 32, lo = (npad + fx::FX_CHUNK - 1) / fx::FX_CHUNK, hi = npad / KX_SMALL;
+  int C = KX_WARPS * KX_CTAS * sms / nt;
+  if (nt <= 32 && C > 2048 / nt) C = 2048 / nt;
+  if (C > hi || nt < 8) C = hi;  // chunks of KX_SMALL
+  if (C < lo) C = lo;
+  *chunk = (npad + C - 1) / C;
+  *chunks = (npad + *chunk - 1) / *chunk;
+}
+
+template <bool FULL>
+static void launch_kick_fx(const Sim &S, const DevParams &P, int force, cudaStream_t st) {
+  const int tw = S.nt >= 8 ? 8 : (S.nt >= 4 ? 4 : (S.nt >= 2 ? 2 : 1)), cw = KX_WARPS / tw;
+  const int grid = ((S.nt + tw - 1) / tw) * ((S.kch + cw - 1) / cw);
+  if (tw == 8) k_kick_fx<FULL, 8><<<grid, 32 * KX_WARPS, 0, st>>>(S, P, force);
+  else if (tw == 4) k_kick_fx<FULL, 4><<<grid, 32 * KX_WARPS, 0, st>>>(S, P, force);
+  else if (tw == 2) k_kick_fx<FULL, 2><<<grid, 32 * KX_WARPS, 0, st>>>(S, P, force);
+  else k_kick_fx<FULL, 1><<<grid, 32 * KX_WARPS, 0, st>>>(S, P, force);
 }
 
 // Component c of the near-pair acceleration of body i: the precheck candidates recorded in row i
@@ -217,10 +475,10 @@ __device__ __forceinline__ double near_term(const Sim &S, const DevParams &P, in
 // Also writes the per-tile momentum of the new velocities for the next Sun drift.
 // ---------------------------------------------------------------------------------------------
 template <int MODE>
-__global__ void __launch_bounds__(128) k_fin(Sim S, DevParams P, double h1, double h2, double *aout) {
+__global__ void __launch_bounds__(128) k_fin(Sim S, DevParams P, double h1, double h2, double *aout, int nslot) {
   constexpr bool ALL = MODE == FIN_CLOSE_ALL;  // the pair kernel weighed every pair: no near pass
   const int B = blockIdx.x, c = blockIdx.y, wi = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int np = S.npad, nt = S.nt, i = B * 32 + lane;
+  const int np = S.npad, i = B * 32 + lane;
   __shared__ double red[4][32];
   __shared__ int ent[32 * CCAP], raw[32 * CCAP];
   __shared__ double contrib[32 * CCAP];
@@ -252,8 +510,8 @@ __global__ void __launch_bounds__(128) k_fin(Sim S, DevParams P, double h1, doub
     if (lane == 0) off[0] = 0;
   }
   if (use_part) {  // far-field partial sums: each warp a quarter of the slots, two chains of alternate slots
-    const int nslot = 2 * nt, s0 = wi * nslot / 4, s1 = (wi + 1) * nslot / 4;
-    const double *base = S.part + (size_t)B * nt * 2 * 96 + c * 32 + lane;
+    const int s0 = wi * nslot / 4, s1 = (wi + 1) * nslot / 4;
+    const double *base = S.part + (size_t)B * nslot * 96 + c * 32 + lane;
     double acc0 = 0.0, acc1 = 0.0;
     int s = s0;
     for (; s + 1 < s1; s += 2) { acc0 += base[(size_t)s * 96]; acc1 += base[(size_t)(s + 1) * 96]; }
@@ -301,34 +559,30 @@ __global__ void __launch_bounds__(128) k_fin(Sim S, DevParams P, double h1, doub
 }
 
 // ---------------------------------------------------------------------------------------------
-int kick_grid(const Sim &S) {
-  int warps = S.nwarps > S.nt ? S.nwarps : S.nt;
-  return (warps * 32 + 127) / 128;
-}
-
 void launch_rcrit(const Sim &S, const DevParams &P, double tau_abs, int check_reuse, cudaStream_t st) {
   k_rcrit<<<(S.npad + 127) / 128, 128, 0, st>>>(S, P, tau_abs, check_reuse);
 }
 
 void launch_kick(const Sim &S, const DevParams &P, bool full, bool precise, cudaStream_t st, bool force) {
-  const int grid = kick_grid(S);
   const int f = force ? 1 : 0;
-  if (full) {
-    if (precise) k_kick<true, true><<<grid, 128, 0, st>>>(S, P, f);
-    else k_kick<true, false><<<grid, 128, 0, st>>>(S, P, f);
+  if (precise) {
+    const int grid = ((S.nwarps > S.nt ? S.nwarps : S.nt) * 32 + 127) / 128;
+    if (full) k_kick_precise<true><<<grid, 128, 0, st>>>(S, P, f);
+    else k_kick_precise<false><<<grid, 128, 0, st>>>(S, P, 0);
   } else {
-    if (precise) k_kick<false, true><<<grid, 128, 0, st>>>(S, P, 0);
-    else k_kick<false, false><<<grid, 128, 0, st>>>(S, P, 0);
+    if (full) launch_kick_fx<true>(S, P, f, st);
+    else launch_kick_fx<false>(S, P, 0, st);
   }
 }
 
-void launch_fin(const Sim &S, const DevParams &P, FinMode mode, double h1, double h2, double *aout,
+void launch_fin(const Sim &S, const DevParams &P, FinMode mode, bool precise, double h1, double h2, double *aout,
                 cudaStream_t st) {
   dim3 grid(S.nt, 3);
-  if (mode == FIN_CLOSE) k_fin<FIN_CLOSE><<<grid, 128, 0, st>>>(S, P, h1, h2, aout);
-  else if (mode == FIN_CLOSE_ALL) k_fin<FIN_CLOSE_ALL><<<grid, 128, 0, st>>>(S, P, h1, h2, aout);
-  else if (mode == FIN_OPEN) k_fin<FIN_OPEN><<<grid, 128, 0, st>>>(S, P, h1, h2, aout);
-  else k_fin<FIN_INIT><<<grid, 128, 0, st>>>(S, P, h1, h2, aout);
+  const int nslot = precise ? 2 * S.nt : S.kch;  // partial-sum slots per tile of the pair kernel used
+  if (mode == FIN_CLOSE) k_fin<FIN_CLOSE><<<grid, 128, 0, st>>>(S, P, h1, h2, aout, nslot);
+  else if (mode == FIN_CLOSE_ALL) k_fin<FIN_CLOSE_ALL><<<grid, 128, 0, st>>>(S, P, h1, h2, aout, nslot);
+  else if (mode == FIN_OPEN) k_fin<FIN_OPEN><<<grid, 128, 0, st>>>(S, P, h1, h2, aout, nslot);
+  else k_fin<FIN_INIT><<<grid, 128, 0, st>>>(S, P, h1, h2, aout, nslot);
 }
 
 // Second Sun drift after the last substep: x += hcm * P, P the momentum before the closing kick.

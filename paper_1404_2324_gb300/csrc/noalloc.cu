@@ -123,6 +123,7 @@ extern "C" int genga_kick_noalloc(int n, double G, double pc, int kmode, int pre
   S.items = (int *)(base + O_ITEMS);
   S.nitems = S.nt * S.nt;
   S.nwarps = S.nitems < 8 * sms ? S.nitems : 8 * sms;  // the allocating kick's configuration
+  kick_split(S.npad, sms, &S.kch, &S.kchunk);
   S.flags = (int *)(base + O_FLAGS); S.status = (int *)(base + O_STATUS);
   S.counters = (long long *)(base + O_COUNTERS);
   double *aout = (double *)(base + O_AOUT);
@@ -146,10 +147,10 @@ extern "C" int genga_kick_noalloc(int n, double G, double pc, int kmode, int pre
       cudaMemsetAsync(S.status, 0, sizeof(int), st) != cudaSuccess ||
       cudaMemsetAsync(S.counters, 0, NCOUNTERS * sizeof(long long), st) != cudaSuccess)
     return GENGA_ECUDA;
-  k_items<<<1, 32, 0, st>>>(S.items, S.nt);
+  if (precise_div) k_items<<<1, 32, 0, st>>>(S.items, S.nt);
   launch_soa_setup(S, P, m, alive, x, nullptr, rc, n, st);
   launch_kick(S, P, false, precise_div != 0, st);
-  launch_fin(S, P, FIN_INIT, 0.0, 0.0, aout, st);
+  launch_fin(S, P, FIN_INIT, precise_div != 0, 0.0, 0.0, aout, st);
   if (cudaMemcpy2DAsync(a, n * sizeof(double), aout, S.npad * sizeof(double), n * sizeof(double), 3,
                         cudaMemcpyDeviceToDevice, st) != cudaSuccess)
     return GENGA_ECUDA;
