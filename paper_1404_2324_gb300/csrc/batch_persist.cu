@@ -73,11 +73,8 @@ __device__ __forceinline__ void bp_big_force(BpBig &sh, const DevParams &P, doub
       const bool cen = p == q;
       const double dx = (cen ? 0.0 : z[p][0]) - xq, dy = (cen ? 0.0 : z[p][1]) - yq, dz = (cen ? 0.0 : z[p][2]) - zq;
       const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-      const double yr = rsqrt_refined(r2);
       const bool inside = sh.alive[p] && dbits(r2) < umax64(sh.rcsq[q], sh.rcsq[p]);
-      const double wA = changeover_wA_clamped(r2 * yr, pmin(sh.A[q], sh.A[p]), P.kmode);
-      const double w = cen ? 1.0 : (inside ? wA : 0.0);
-      const double f = (cen ? Gm0 : sh.gm[p]) * w * (yr * yr * yr);
+      const double f = bs_factor(r2, cen ? Gm0 : sh.gm[p], pmin(sh.A[q], sh.A[p]), cen, inside, P.kmode);
       ax = fma(f, dx, ax); ay = fma(f, dy, ay); az = fma(f, dz, az);
     }
   }

@@ -139,11 +139,8 @@ __device__ __forceinline__ void pair_terms(const PairTerm &t, const DevParams &P
     const bool cen = t.cen;
     const double dx = (cen ? 0.0 : pos[p][0]) - xq, dy = (cen ? 0.0 : pos[p][1]) - yq, dz = (cen ? 0.0 : pos[p][2]) - zq;
     const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-    const double yr = rsqrt_refined(r2);
     const bool inside = t.palive && dbits(r2) < t.thr;
-    const double wA = changeover_wA_clamped(r2 * yr, t.Amin, P.kmode);
-    const double w = cen ? 1.0 : (inside ? wA : 0.0);
-    const double f = t.pref * w * (yr * yr * yr);
+    const double f = bs_factor(r2, t.pref, t.Amin, cen, inside, P.kmode);
     ax = f * dx; ay = f * dy; az = f * dz;
   }
   ax += __shfl_xor_sync(0xffffffffu, ax, 1);

@@ -14,6 +14,7 @@
 // the large-group list that the grouping kernel writes.
 #include <cooperative_groups.h>
 
+#include "fxforce.cuh"
 #include "genga_launch.h"
 
 namespace cg = cooperative_groups;
@@ -67,11 +68,8 @@ __device__ __forceinline__ void cl_terms(const BsClShared &sh, const DevParams &
       const double dx = (cen ? 0.0 : pos[p][0]) - xq, dy = (cen ? 0.0 : pos[p][1]) - yq,
                    dz = (cen ? 0.0 : pos[p][2]) - zq;
       const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-      const double yr = rsqrt_refined(r2);
       const bool inside = sh.alive[p] && dbits(r2) < umax64(sh.rcsq[q], sh.rcsq[p]);
-      const double wA = changeover_wA_clamped(r2 * yr, pmin(sh.A[q], sh.A[p]), P.kmode);
-      const double w = cen ? 1.0 : (inside ? wA : 0.0);
-      const double f = (cen ? Gm0 : sh.gm[p]) * w * (yr * yr * yr);
+      const double f = bs_factor(r2, cen ? Gm0 : sh.gm[p], pmin(sh.A[q], sh.A[p]), cen, inside, P.kmode);
       ax = fma(f, dx, ax); ay = fma(f, dy, ay); az = fma(f, dz, az);
     }
   }
@@ -102,11 +100,8 @@ __device__ __forceinline__ void cl_eval(BsClShared &sh, const DevParams &P, doub
     const double dx = (cen ? 0.0 : pos[b][0]) - pos[a][0], dy = (cen ? 0.0 : pos[b][1]) - pos[a][1],
                  dz = (cen ? 0.0 : pos[b][2]) - pos[a][2];
     const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-    const double yr = rsqrt_refined(r2);
-    const bool inside = sh.alive[a] && sh.alive[b] && dbits(r2) < umax64(sh.rcsq[a], sh.rcsq[b]);
-    const double wA = changeover_wA_clamped(r2 * yr, pmin(sh.A[a], sh.A[b]), P.kmode);
-    const double w = cen ? (sh.alive[a] ? Gm0 : 0.0) : (inside ? wA : 0.0);
-    const double f = w * (yr * yr * yr);
+    const bool inside = !cen && sh.alive[a] && sh.alive[b] && dbits(r2) < umax64(sh.rcsq[a], sh.rcsq[b]);
+    const double f = bs_factor(r2, cen ? Gm0 : 1.0, pmin(sh.A[a], sh.A[b]), cen && sh.alive[a], inside, P.kmode);
     sh.term[t][0] = f * dx; sh.term[t][1] = f * dy; sh.term[t][2] = f * dz;
   }
   __syncthreads();

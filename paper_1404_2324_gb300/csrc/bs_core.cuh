@@ -2,6 +2,7 @@
 // kernels of bs.cu and the persistent batched kernel (batch_persist.cu). Every translation unit
 // that includes it holds its own copy of the Neville factors (bs_core_set_factors fills it).
 #pragma once
+#include "fxforce.cuh"
 #include "genga_launch.h"
 
 namespace genga {
@@ -59,11 +60,8 @@ __device__ __forceinline__ void bs_terms(const SH &sh, const DevParams &P, doubl
       const double dx = (cen ? 0.0 : pos[p][0]) - xq, dy = (cen ? 0.0 : pos[p][1]) - yq,
                    dz = (cen ? 0.0 : pos[p][2]) - zq;
       const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-      const double yr = rsqrt_refined(r2);
       const bool inside = sh.alive[p] && dbits(r2) < umax64(sh.rcsq[q], sh.rcsq[p]);
-      const double wA = changeover_wA_clamped(r2 * yr, pmin(sh.A[q], sh.A[p]), P.kmode);
-      const double w = cen ? 1.0 : (inside ? wA : 0.0);
-      const double f = (cen ? Gm0 : sh.gm[p]) * w * (yr * yr * yr);
+      const double f = bs_factor(r2, cen ? Gm0 : sh.gm[p], pmin(sh.A[q], sh.A[p]), cen, inside, P.kmode);
       ax = fma(f, dx, ax); ay = fma(f, dy, ay); az = fma(f, dz, az);
     }
   }

@@ -24,6 +24,7 @@
 // become resident once the kernels beside it on other graph branches finish, none of which waits on
 // this one. Every wait is bounded: after GR_SPIN_LIMIT polls a CTA sets the abort flag and the
 // status bit ST_GRID_TIMEOUT, and every CTA leaves.
+#include "fxforce.cuh"
 #include "genga_launch.h"
 
 namespace genga {
@@ -111,11 +112,9 @@ __device__ void gr_accel(GrShared &sh, const BsGridBuf &B, const DevParams &P, d
         const double dx = (cen ? 0.0 : sh.pos[t][0]) - xq, dy = (cen ? 0.0 : sh.pos[t][1]) - yq,
                      dz = (cen ? 0.0 : sh.pos[t][2]) - zq;
         const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-        const double yr = rsqrt_refined(r2);
         const bool inside = sh.al[t] && dbits(r2) < umax64(rqq, sh.rq[t]);
-        const double wA = changeover_wA_clamped(r2 * yr, pmin(Aq, sh.A[t]), P.kmode);
-        const double w = cen ? 1.0 : (inside ? wA : 0.0);
-        const double f = (cen ? Gm0 : sh.gm[t]) * w * (yr * yr * yr);
+        if (!cen && !inside) continue;
+        const double f = bs_factor(r2, cen ? Gm0 : sh.gm[t], pmin(Aq, sh.A[t]), cen, inside, P.kmode);
         ax = fma(f, dx, ax); ay = fma(f, dy, ay); az = fma(f, dz, az);
       }
     }

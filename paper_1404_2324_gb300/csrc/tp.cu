@@ -16,6 +16,7 @@
 #include <cmath>
 #include <cstring>
 
+#include "fxforce.cuh"
 #include "genga_launch.h"
 
 namespace genga {
@@ -502,7 +503,7 @@ __device__ __forceinline__ void tp_force(const Sim &S, const TPSet &T, const Dev
   for (int p = 0;; ++p) {
     // this lane's body: the Sun (level lane, first round) or planet p (upper lane)
     double bx = 0.0, by = 0.0, bz = 0.0, gm = P.Gm0, A = 0.0;
-    u64 cut = ~0ULL;
+    u64 cut = 0ULL;
     const bool body = up && bits;
     if (body) {
       const int j = __ffs(bits) - 1;
@@ -521,11 +522,7 @@ __device__ __forceinline__ void tp_force(const Sim &S, const TPSet &T, const Dev
     if (body || (!up && p == 0)) {
       dx = bx - sx; dy = by - sy; dz = bz - sz;
       const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-      const double yr = rsqrt_refined(r2);
-      const double r3 = up ? yr * yr * yr : rcube_refined(r2);
-      double wB, wA;
-      changeover_w(r2 * yr, A, P.kmode, wB, wA);  // 1 for the Sun (A = 0)
-      g = dbits(r2) >= cut ? 0.0 : gm * wA * r3;
+      g = bs_factor(r2, gm, A, !up, dbits(r2) < cut, P.kmode);
     }
     if (p == 0 && !up) { ax = g * dx; ay = g * dy; az = g * dz; }  // the Sun: -G m0 y / |y|^3
     const double gp = __shfl_xor_sync(act, g, 8), px = __shfl_xor_sync(act, dx, 8),
