@@ -110,44 +110,6 @@ struct BsPairShared {
 // the two warps of a unit (named barrier 1 + unit, 64 threads)
 __device__ __forceinline__ void unit_sync(int bar) { asm volatile("bar.sync %0, 64;" ::"r"(bar) : "memory"); }
 
-// One lane's term (the central mass if p == q, else partner p) with what stays fixed over an
-// attempt: the source's G m, the smaller A = 1/(0.9 rc), the larger rc^2 (bits) and the partner's
-// live flag; only the positions change between evaluations.
-struct PairTerm {
-  double pref, Amin;
-  u64 thr;
-  bool cen, palive, has;
-};
-
-__device__ __forceinline__ PairTerm pair_term(const BsPairShared &sh, double Gm0, int g, int q, int p) {
-  PairTerm t;
-  t.has = p < g;
-  const int pp = t.has ? p : q;
-  t.cen = p == q;
-  t.pref = t.cen ? Gm0 : sh.gm[pp];
-  t.Amin = pmin(sh.A[q], sh.A[pp]);
-  t.thr = umax64(sh.rcsq[q], sh.rcsq[pp]);
-  t.palive = sh.alive[pp] != 0;
-  return t;
-}
-
-__device__ __forceinline__ void pair_terms(const PairTerm &t, const DevParams &P, int q, int p, const double (*pos)[3],
-                                           bool q_alive, double &ax, double &ay, double &az) {
-  ax = ay = az = 0.0;
-  if (q_alive && t.has) {
-    const double xq = pos[q][0], yq = pos[q][1], zq = pos[q][2];
-    const bool cen = t.cen;
-    const double dx = (cen ? 0.0 : pos[p][0]) - xq, dy = (cen ? 0.0 : pos[p][1]) - yq, dz = (cen ? 0.0 : pos[p][2]) - zq;
-    const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-    const bool inside = t.palive && dbits(r2) < t.thr;
-    const double f = bs_factor(r2, t.pref, t.Amin, cen, inside, P.kmode);
-    ax = f * dx; ay = f * dy; az = f * dz;
-  }
-  ax += __shfl_xor_sync(0xffffffffu, ax, 1);
-  ay += __shfl_xor_sync(0xffffffffu, ay, 1);
-  az += __shfl_xor_sync(0xffffffffu, az, 1);
-}
-
 // One attempt of length H from sh.y by one warp, with the warp's own buffers (index w). Returns the
 // accepted level (0: no level converged) and leaves the extrapolated state in sh.yn[w].
 __device__ int pair_attempt(BsPairShared &sh, int w, const DevParams &P, double Gm0, int g, double H, int lane) {
@@ -156,9 +118,14 @@ __device__ int pair_attempt(BsPairShared &sh, int w, const DevParams &P, double 
   const bool act = q < g;
   const double h = __ddiv_rn(H, (double)nk), h2 = 2.0 * h;
   const bool qa = act && sh.alive[q];
-  double zA[6], zB[6];
-  for (int c = 0; c < 6; ++c) zA[c] = act ? sh.y[q][c] : 0.0;
-  if (act && sub == 0) for (int c = 0; c < 3; ++c) sh.pos[w][0][lev][q][c] = zA[c];
+  const int qq = act ? q : 0, oc = 2 * sub, on = 2 - sub;  // own components: 0 and 1, or 2
+  double xA[2], vA[2], xB[2], vB[2];  // the two newest states of the level's chain
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    xA[k] = act && k < on ? sh.y[q][oc + k] : 0.0;
+    vA[k] = act && k < on ? sh.y[q][3 + oc + k] : 0.0;
+    if (act && k < on) sh.pos[w][0][lev][q][oc + k] = xA[k];
+  }
   const int qc = lane / 6, cc = lane % 6;
   const bool rowth = qc < g;
   double scale = 0.0;
@@ -169,15 +136,12 @@ __device__ int pair_attempt(BsPairShared &sh, int w, const DevParams &P, double 
   }
   if (lane < BS_LEVELS) sh.err[w][lane] = 0ULL;
   __syncwarp();
-  const int qq = act ? q : 0;
-  const PairTerm term = pair_term(sh, Gm0, g, qq, sub);
-  double ax, ay, az;
-  pair_terms(term, P, qq, sub, sh.pos[w][0][lev], qa, ax, ay, az);
-  if (qa) {
-    zB[0] = fma(h, zA[3], zA[0]); zB[1] = fma(h, zA[4], zA[1]); zB[2] = fma(h, zA[5], zA[2]);
-    zB[3] = fma(h, ax, zA[3]); zB[4] = fma(h, ay, zA[4]); zB[5] = fma(h, az, zA[5]);
-  } else {
-    for (int c = 0; c < 6; ++c) zB[c] = zA[c];
+  double ac[3];
+  bs_accel(sh, P, Gm0, g, qq, sub, 2, sh.pos[w][0][lev], qa, ac);
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    xB[k] = qa ? fma(h, vA[k], xA[k]) : xA[k];
+    vB[k] = qa ? fma(h, ac[k], vA[k]) : vA[k];
   }
   const int lmax = P.bs_kmax < BS_LEVELS ? P.bs_kmax : BS_LEVELS;
   const u64 eps = dbits(P.bs_eps);
@@ -185,22 +149,33 @@ __device__ int pair_attempt(BsPairShared &sh, int w, const DevParams &P, double 
   int acc = 0, b = 1;
   for (int e = 1; e <= 2 * lmax; ++e) {
     const bool lv = act && e <= nk;
-    if (lv && sub == 0) for (int c = 0; c < 3; ++c) sh.pos[w][b][lev][q][c] = zB[c];
-    __syncwarp();
-    pair_terms(term, P, qq, sub, sh.pos[w][b][lev], qa && e <= nk, ax, ay, az);
     if (lv) {
-      if (qa && e < nk) {
-        double zn[6];
-        zn[0] = fma(h2, zB[3], zA[0]); zn[1] = fma(h2, zB[4], zA[1]); zn[2] = fma(h2, zB[5], zA[2]);
-        zn[3] = fma(h2, ax, zA[3]); zn[4] = fma(h2, ay, zA[4]); zn[5] = fma(h2, az, zA[5]);
-        for (int c = 0; c < 6; ++c) { zA[c] = zB[c]; zB[c] = zn[c]; }
-      }
+#pragma unroll
+      for (int k = 0; k < 2; ++k)
+        if (k < on) sh.pos[w][b][lev][q][oc + k] = xB[k];
+    }
+    __syncwarp();
+    bs_accel(sh, P, Gm0, g, qq, sub, 2, sh.pos[w][b][lev], qa && e <= nk, ac);
+    if (lv) {
       // the level's chain is done: its tableau lanes form T_{L,1} = (z_{n-1} + z_n + h z'_n) / 2,
       // one component each, so the warp issues that arithmetic once instead of per level lane
-      if (e == nk && sub == 0) {
+      if (e == nk) {
         double *z = sh.zt[w][lev][q];
-        for (int c = 0; c < 6; ++c) { z[c] = zA[c]; z[6 + c] = zB[c]; }
-        z[12] = ax; z[13] = ay; z[14] = az; z[15] = h;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          if (k >= on) continue;
+          z[oc + k] = xA[k]; z[3 + oc + k] = vA[k];
+          z[6 + oc + k] = xB[k]; z[9 + oc + k] = vB[k];
+          z[12 + oc + k] = ac[k];
+        }
+        if (sub == 0) z[15] = h;
+      } else if (qa) {
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          const double xn = fma(h2, vB[k], xA[k]), vn = fma(h2, ac[k], vA[k]);
+          xA[k] = xB[k]; vA[k] = vB[k];
+          xB[k] = xn; vB[k] = vn;
+        }
       }
     }
     b ^= 1;

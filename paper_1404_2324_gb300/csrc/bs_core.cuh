@@ -42,33 +42,44 @@ struct BsSharedT {
 };
 using BsShared = BsSharedT<BS_GMAX>;
 
-// Acceleration terms of member q assigned to this thread: term p == q is the central mass, any
-// other p the (1 - K)-weighted pull of partner p (H_A, Eq. Ha). Summed over the slot's threads.
-// Every lane runs the same straight-line code (the central mass is a partner at the origin with
-// G m0 and weight 1; a partner outside rc gets weight 0): lanes of one warp that took different
-// branches would each pay for both, and an FP64 warp instruction costs its sub-partition 64
-// cycles whatever its active lanes.
+// Acceleration of member q at positions pos by the slot's ttps threads (4, 2 or 1): thread tsub sums
+// the terms p = tsub, tsub + ttps, ... (p == q: the central mass; any other p the (1 - K)-weighted pull
+// of partner p, H_A, Eq. Ha) and is given the components it owns: thread c of 4 component c, threads 0
+// and 1 of 2 the components 0, 1 and 2, one thread all three. Every lane runs the same straight-line
+// code (the central mass is a partner at the origin with G m0 and weight 1; a partner outside rc gets
+// weight 0): lanes of one warp that took different branches would each pay for both, and an FP64 warp
+// instruction costs its sub-partition 64 cycles whatever its active lanes. The threads exchange what
+// they do not own, so a slot of 4 issues 3 additions for the sum and 4 instructions for its chain
+// step, where every thread holding every component took 6 and 6.
 template <class SH>
-__device__ __forceinline__ void bs_terms(const SH &sh, const DevParams &P, double Gm0, int g, int q, int sub,
-                                         int tps, const double (*pos)[3], bool q_alive, double &ax, double &ay,
-                                         double &az) {
-  ax = ay = az = 0.0;
-  const double xq = pos[q][0], yq = pos[q][1], zq = pos[q][2];
+__device__ __forceinline__ void bs_accel(const SH &sh, const DevParams &P, double Gm0, int g, int q, int tsub, int ttps,
+                                         const double (*pos)[3], bool q_alive, double (&acc)[3]) {
+  double a0 = 0.0, a1 = 0.0, a2 = 0.0;
   if (q_alive) {
-    for (int p = sub; p < g; p += tps) {
+    const double xq = pos[q][0], yq = pos[q][1], zq = pos[q][2];
+    for (int p = tsub; p < g; p += ttps) {
       const bool cen = p == q;
       const double dx = (cen ? 0.0 : pos[p][0]) - xq, dy = (cen ? 0.0 : pos[p][1]) - yq,
                    dz = (cen ? 0.0 : pos[p][2]) - zq;
       const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
       const bool inside = sh.alive[p] && dbits(r2) < umax64(sh.rcsq[q], sh.rcsq[p]);
       const double f = bs_factor(r2, cen ? Gm0 : sh.gm[p], pmin(sh.A[q], sh.A[p]), cen, inside, P.kmode);
-      ax = fma(f, dx, ax); ay = fma(f, dy, ay); az = fma(f, dz, az);
+      a0 = fma(f, dx, a0); a1 = fma(f, dy, a1); a2 = fma(f, dz, a2);
     }
   }
-  for (int o = tps >> 1; o > 0; o >>= 1) {
-    ax += __shfl_xor_sync(0xffffffffu, ax, o);
-    ay += __shfl_xor_sync(0xffffffffu, ay, o);
-    az += __shfl_xor_sync(0xffffffffu, az, o);
+  acc[0] = a0; acc[1] = a1; acc[2] = a2;
+  if (ttps == 4) {
+    const bool hi = (tsub & 2) != 0, odd = (tsub & 1) != 0;
+    const double r0 = __shfl_xor_sync(0xffffffffu, hi ? a0 : a2, 2), r1 = __shfl_xor_sync(0xffffffffu, a1, 2);
+    // threads 0, 1 now sum components 0 and 1 of the pair (tsub, tsub + 2), threads 2, 3 component 2
+    const double s0 = (hi ? a2 : a0) + r0, s1 = a1 + r1;
+    const double r = __shfl_xor_sync(0xffffffffu, hi || odd ? s0 : s1, 1);
+    acc[0] = (hi || !odd ? s0 : s1) + r;
+  } else if (ttps == 2) {
+    const bool odd = (tsub & 1) != 0;
+    const double r0 = __shfl_xor_sync(0xffffffffu, odd ? a0 : a2, 1), r1 = __shfl_xor_sync(0xffffffffu, a1, 1);
+    acc[0] = (odd ? a2 : a0) + r0;
+    acc[1] = a1 + r1;
   }
 }
 
@@ -103,6 +114,8 @@ __device__ void bs_group(BsSharedT<GM> &sh, const Sim &S, const DevParams &P, do
   const bool spec = g <= 2 && tps == 4 && NT >= 128 && GM >= 18;  // uniform
   const int half = spec ? (sub >> 1) : 0, tsub = spec ? (sub & 1) : sub, ttps = spec ? 2 : tps;
   const int qm = q + 16 * half;  // this thread's member in its attempt's position and tableau arrays
+  const int oc = ttps == 4 ? tsub : 2 * tsub;  // this thread's components: oc .. oc + on - 1
+  const int on = ttps == 4 ? (tsub < 3 ? 1 : 0) : (ttps == 2 ? 2 - tsub : 3);
   const int trow = (spec && tid >= 64) ? tid - 64 : tid;  // tableau thread of attempt (spec && tid >= 64)
   const int thalf = (spec && tid >= 64) ? 1 : 0;
   if (tid < g) {
@@ -129,9 +142,13 @@ __device__ void bs_group(BsSharedT<GM> &sh, const Sim &S, const DevParams &P, do
     // tableau first, but attempts that converge at level 4-6 (almost all) skip the deeper chains.
     const double h = __ddiv_rn(half ? 0.5 * H : H, (double)nk), h2 = 2.0 * h;
     const bool qa = act && sh.alive[q];
-    double zA[6], zB[6], out[6];
-    for (int c = 0; c < 6; ++c) zA[c] = sh.y[q][c];
-    if (act && tsub == 0) for (int c = 0; c < 3; ++c) sh.pos[0][lev][qm][c] = zA[c];
+    double xA[3], vA[3], xB[3], vB[3];  // the two newest states of the level's chain, own components
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      xA[k] = k < on ? sh.y[q][oc + k] : 0.0;
+      vA[k] = k < on ? sh.y[q][3 + oc + k] : 0.0;
+      if (act && k < on) sh.pos[0][lev][qm][oc + k] = xA[k];
+    }
     const int qc = trow / 6, cc = trow % 6;
     const bool rowth = qc < g;
     double scale = 0.0;  // error scale of (qc, cc): 1/|x| or 1/|v| at the start of the attempt
@@ -142,15 +159,15 @@ __device__ void bs_group(BsSharedT<GM> &sh, const Sim &S, const DevParams &P, do
     }
     if (tid < BS_LEVELS) { sh.err[tid] = 0ULL; sh.err2[tid] = 0ULL; }
     __syncthreads();
-    double ax = 0.0, ay = 0.0, az = 0.0;
-    // every lane of a warp that holds any active slot takes part (the term sums shuffle across
-    // lanes); warps without active slots stay off the FP64 pipe
-    if (__any_sync(0xffffffffu, act)) bs_terms(sh, P, Gm0, g, q, tsub, ttps, sh.pos[0][lev] + 16 * half, qa, ax, ay, az);
-    if (qa) {
-      zB[0] = fma(h, zA[3], zA[0]); zB[1] = fma(h, zA[4], zA[1]); zB[2] = fma(h, zA[5], zA[2]);
-      zB[3] = fma(h, ax, zA[3]); zB[4] = fma(h, ay, zA[4]); zB[5] = fma(h, az, zA[5]);
-    } else {
-      for (int c = 0; c < 6; ++c) zB[c] = zA[c];
+    double ac[3] = {0.0, 0.0, 0.0};
+    // every lane of a warp that holds any active slot takes part (the sums shuffle across lanes);
+    // warps without active slots stay off the pipes
+    if (__any_sync(0xffffffffu, act)) bs_accel(sh, P, Gm0, g, q, tsub, ttps, sh.pos[0][lev] + 16 * half, qa, ac);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      if (k >= on) continue;
+      xB[k] = qa ? fma(h, vA[k], xA[k]) : xA[k];
+      vB[k] = qa ? fma(h, ac[k], vA[k]) : vA[k];
     }
     const int lmax = P.bs_kmax < BS_LEVELS ? P.bs_kmax : BS_LEVELS;
     const u64 eps = dbits(P.bs_eps);
@@ -159,28 +176,28 @@ __device__ void bs_group(BsSharedT<GM> &sh, const Sim &S, const DevParams &P, do
     int b = 1;
     for (int e = 1; e <= 2 * lmax; ++e) {
       const bool lv = act && e <= nk;
-      if (lv && tsub == 0) for (int c = 0; c < 3; ++c) sh.pos[b][lev][qm][c] = zB[c];
-      __syncthreads();
-      if (__any_sync(0xffffffffu, lv)) bs_terms(sh, P, Gm0, g, q, tsub, ttps, sh.pos[b][lev] + 16 * half, qa, ax, ay, az);
       if (lv) {
-        if (qa) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+          if (k < on) sh.pos[b][lev][qm][oc + k] = xB[k];
+      }
+      __syncthreads();
+      if (__any_sync(0xffffffffu, lv)) bs_accel(sh, P, Gm0, g, q, tsub, ttps, sh.pos[b][lev] + 16 * half, qa, ac);
+      if (lv) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          if (k >= on) continue;
           if (e < nk) {
-            double zn[6];
-            zn[0] = fma(h2, zB[3], zA[0]); zn[1] = fma(h2, zB[4], zA[1]); zn[2] = fma(h2, zB[5], zA[2]);
-            zn[3] = fma(h2, ax, zA[3]); zn[4] = fma(h2, ay, zA[4]); zn[5] = fma(h2, az, zA[5]);
-            for (int c = 0; c < 6; ++c) { zA[c] = zB[c]; zB[c] = zn[c]; }
-          } else {
-            out[0] = 0.5 * fma(h, zB[3], zB[0] + zA[0]);
-            out[1] = 0.5 * fma(h, zB[4], zB[1] + zA[1]);
-            out[2] = 0.5 * fma(h, zB[5], zB[2] + zA[2]);
-            out[3] = 0.5 * fma(h, ax, zB[3] + zA[3]);
-            out[4] = 0.5 * fma(h, ay, zB[4] + zA[4]);
-            out[5] = 0.5 * fma(h, az, zB[5] + zA[5]);
+            if (qa) {
+              const double xn = fma(h2, vB[k], xA[k]), vn = fma(h2, ac[k], vA[k]);
+              xA[k] = xB[k]; vA[k] = vB[k];
+              xB[k] = xn; vB[k] = vn;
+            }
+          } else {  // T_{L,1}
+            sh.tab[lev][qm][oc + k] = qa ? 0.5 * fma(h, vB[k], xB[k] + xA[k]) : xA[k];
+            sh.tab[lev][qm][3 + oc + k] = qa ? 0.5 * fma(h, ac[k], vB[k] + vA[k]) : vA[k];
           }
-        } else if (e == nk) {
-          for (int c = 0; c < 6; ++c) out[c] = zA[c];
         }
-        if (e == nk && tsub == 0) for (int c = 0; c < 6; ++c) sh.tab[lev][qm][c] = out[c];  // T_{L,1}
       }
       b ^= 1;
       if (e & 1) continue;

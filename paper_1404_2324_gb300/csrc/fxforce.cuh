@@ -56,45 +56,55 @@ FX_HD Num num(double x) {
   return n;
 }
 
-// pref w / r^3 for r2 > 0 (normal): w = 1 (full), W_A of the changeover zone with A = 1/(0.9 rc)
-// (zone), or 0 (neither).
-FX_HD double pull_factor(double r2, const Num &pref, const Num &A, bool full, bool zone) {
-  const u64 b = d2u(r2);
-  const int q = (int)(b >> 52) - 1022, odd = q & 1, k = (q - odd) >> 1;  // r2 = R 4^k, R in [0.5, 2)
-  const u64 R = (((b & 0xfffffffffffffULL) | 0x10000000000000ULL) << 9) << odd;  // 2^-62
-  const float u = frsqrt(i2f(((126 + odd) << 23) | (int)((u32)(b >> 29) & 0x7fffffu)));
-  const u32 U = (u32)f2i(u + 2.0f) << 9;                        // 2^-31
+// pref w rho^-3 in 2^-59 (times 2^pref.me) from rho^2 = R 2^-62 in [0.5, 2) and its single-precision
+// value; r = rho 2^k. w = 1 (full), W_A of the changeover zone with A = 1/(0.9 rc) (zone), or 0.
+FX_HD u64 factor(u64 R, float rho2, int k, const Num &pref, const Num &A, bool full, bool zone) {
+  const u32 U = (u32)f2i(frsqrt(rho2) + 2.0f) << 9;             // 2^-31
   const u64 W = mulu(U, U);                                     // 2^-62
   const u64 e = (1ULL << 60) - mulhi(R, W);                     // 2^-60, signed
   const int e1 = (int)((i64)e >> 11);                           // 2^-49
   const u32 ee = hi32((u64)muls(e1, e1));                       // 2^-66
   const u64 F = (1ULL << 63) + 12ULL * e + (ee * 15u >> 6);
-  const u64 Y3 = mulhi(mul32(W, U), F);                         // r^-3 8^k, 2^-60
+  const u64 Y3 = mulhi(mul32(W, U), F);                         // rho^-3, 2^-60
   u64 w = full ? (1ULL << 63) : 0ULL;                           // 2^-63
-  const u64 rho = mulhi(mul32(R, U), (1ULL << 63) + 4ULL * e + (ee * 3u >> 6));  // 2^-60
-  const int n = k + A.me;                                       // r A = rho M_A 2^n
-  i64 y = (i64)(mulhi(rho, A.M) << ((n + 3) & 63)) >> 1;        // r A in 2^-61 for -3 <= n <= 1
-  y -= 256204778801521550LL;                                    // 2^61 / 9
-  if (n < -3) y = 0;
-  if (n > 1) y = 1LL << 61;
-  y = y < 0 ? 0 : (y > (1LL << 61) ? (1LL << 61) : y);
-  const u64 yy = sqrhi((u64)y << 2), oo = sqrhi((1ULL << 63) - ((u64)y << 2));  // 2^-62
-  const u64 D = yy + oo;                                        // in [0.5, 1]
-  const float s = frcp((float)(int)hi32(D) * 9.313225746154785e-10f);  // 1 .. 2
-  const u32 S = (u32)f2i(s + 4.0f) << 9;                        // 2^-30
-  const u64 d = (1ULL << 60) - mul32(D, S);                     // 2^-60, signed
-  const int d1 = (int)((i64)d >> 11);
-  const u64 H = (1ULL << 63) + 8ULL * d + (hi32((u64)muls(d1, d1)) >> 3);
-  const u64 wA = mulhi(mul32(oo, S), H) << 4;                   // 2^-63
-  if (zone && !full) w = wA;
-  u64 z = mulhi(mulhi(Y3 << 1, w), pref.M);                     // 2^-59 (2^-61 Y3, 2^-63 w and M)
+  if (zone && !full) {
+    const u64 rho = mulhi(mul32(R, U), (1ULL << 63) + 4ULL * e + (ee * 3u >> 6));  // 2^-60
+    const int n = k + A.me;                                     // r A = rho M_A 2^n
+    i64 y = (i64)((mulhi(rho, A.M) << ((n + 3) & 63)) >> 1);    // r A in 2^-61 for -3 <= n <= 1
+    y -= 256204778801521550LL;                                  // 2^61 / 9
+    if (n < -3) y = 0;
+    if (n > 1) y = 1LL << 61;
+    y = y < 0 ? 0 : (y > (1LL << 61) ? (1LL << 61) : y);
+    const u64 yy = sqrhi((u64)y << 2), oo = sqrhi((1ULL << 63) - ((u64)y << 2));  // 2^-62
+    const u64 D = yy + oo;                                      // in [0.5, 1]
+    const float s = frcp((float)(int)hi32(D) * 9.313225746154785e-10f);  // 1 .. 2
+    const u32 S = (u32)f2i(s + 4.0f) << 9;                      // 2^-30
+    const u64 d = (1ULL << 60) - mul32(D, S);                   // 2^-60, signed
+    const int d1 = (int)((i64)d >> 11);
+    const u64 H = (1ULL << 63) + 8ULL * d + (hi32((u64)muls(d1, d1)) >> 3);
+    w = mulhi(mul32(oo, S), H) << 4;
+  }
+  return mulhi(mulhi(Y3 << 1, w), pref.M);
+}
+
+// z 2^ex as a double (round to nearest; z > 0 or 0).
+FX_HD double to_double(u64 z, int ex) {
   if (z == 0ULL) return 0.0;
   const int lz = clz64(z);
-  z <<= lz;                                                     // f = z 2^(-59 - lz) 2^me 8^-k
-  const u64 m = (z + 0x400ULL) >> 11;                           // 53 bits, rounded (2^53 carries into the exponent)
-  const int ex = 1023 + 63 - lz - 59 + pref.me - 3 * k;
-  if (ex <= 0 || ex >= 0x7fe || z + 0x400ULL < z) return ex <= 0 ? 0.0 : scalbn((double)(z >> 1), ex - 1023 - 62);
-  return u2d(m + ((u64)(ex - 1) << 52));
+  z <<= lz;
+  const u64 m = (z + 0x400ULL) >> 11;                           // 53 bits (2^53 carries into the exponent)
+  const int be = 1023 + 63 - lz + ex;
+  if (be <= 0 || be >= 0x7fe || z + 0x400ULL < z) return be <= 0 ? 0.0 : scalbn((double)(z >> 1), ex - lz + 1);
+  return u2d(m + ((u64)(be - 1) << 52));
+}
+
+// pref w / r^3 for r2 > 0 (normal); full, zone as in factor.
+FX_HD double pull_factor(double r2, const Num &pref, const Num &A, bool full, bool zone) {
+  const u64 b = d2u(r2);
+  const int q = (int)(b >> 52) - 1022, odd = q & 1, k = (q - odd) >> 1;  // r2 = R 4^k, R in [0.5, 2)
+  const u64 R = (((b & 0xfffffffffffffULL) | 0x10000000000000ULL) << 9) << odd;  // 2^-62
+  const float rho2 = i2f(((126 + odd) << 23) | (int)((u32)(b >> 29) & 0x7fffffu));
+  return to_double(factor(R, rho2, k, pref, A, full, zone), pref.me - 59 - 3 * k);
 }
 
 }  // namespace fx
