@@ -283,7 +283,7 @@ void enqueue_step_batch(genga_ctx *c, cudaStream_t st) {
       cudaStreamWaitEvent(c->side, c->ev_fork, 0);
       cudaStreamWaitEvent(c->side2, c->ev_fork, 0);
       launch_bs_pair(S, P, tau, c->pair_grid, c->side);
-      launch_bs(S, P, tau, c->bs_grid, c->side2, BS_GMAX + 1, BS_SMALL + 1);
+      launch_bs(S, P, tau, c->bs_grid, c->side2, BS_GMAX + 1, 3);  // and the groups of 3..BS_SMALL expected to be long
       launch_bs_wide(S, P, tau, c->wide_grid, c->side2);  // queue 3: groups above BS_GMAX members
       launch_bs_small(S, P, tau, c->small_grid, st);
       cudaEventRecord(c->ev_join, c->side);
@@ -890,7 +890,7 @@ int genga_init_batch(genga_ctx **out, int n_sys, const int *offsets, const doubl
     // the parts' BS kernels run side by side: each part a share of the grids one batch would use
     p->pair_grid = std::max(8, 2 * p->pair_grid / K);
     p->small_grid = std::max(16, 2 * p->small_grid / K);
-    p->bs_grid = std::max(4, 2 * p->bs_grid / K);
+    p->bs_grid = std::max(8, 2 * p->bs_grid / K);
     if (rc == GENGA_OK) rc = genga_batch_set_schedule(p, 0);
     if (rc == GENGA_OK) rc = genga_batch_set_kick(p, bsplit, bblock);
     // the counters as a batch of one part leaves them after init; then the first kick in this shape

@@ -468,9 +468,10 @@ __global__ void __launch_bounds__(32 * BG_WARPS) k_b_group(Sim S) {
         S.gsize[g] = cnt[r];
         // the queue of the kernel that integrates the group; groups whose members needed many
         // substeps last time start first (they set the BS time)
-        const int qi = cnt[r] <= 2 ? 0 : (cnt[r] <= BS_SMALL ? 1 : (cnt[r] <= BS_GMAX ? 2 : 3));
+        const bool heavy = hist[r] >= BS_HEAVY;
+        const int qi = cnt[r] <= 2 ? 0 : (cnt[r] <= BS_SMALL && !heavy ? 1 : (cnt[r] <= BS_GMAX ? 2 : 3));
         int *qo = S.gorder + (size_t)qi * S.npad;
-        if (hist[r] >= BS_HEAVY) qo[atomicAdd(&S.norder[2 * qi], 1)] = g;
+        if (heavy) qo[atomicAdd(&S.norder[2 * qi], 1)] = g;
         else qo[S.npad - 1 - atomicAdd(&S.norder[2 * qi + 1], 1)] = g;
         pos[r] = p;
         ng++;

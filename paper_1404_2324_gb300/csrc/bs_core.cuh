@@ -100,7 +100,12 @@ __device__ void bs_group(BsSharedT<GM> &sh, const Sim &S, const DevParams &P, do
     if (tid == 0) atomicOr(S.status, ST_GROUP_TOO_LARGE);
     return;
   }
-  const int slot = tid / tps, sub = tid % tps;
+  // Wide speculation (groups of three or four members on 256 threads): the second half of the CTA runs
+  // the attempt at H/2, as below, from the second attempt on (most groups accept the first). Measured
+  // on 300 systems, whose longest groups of three set the BS phase: 2.41 -> 2.20 ms for 4 steps.
+  const bool specw = (g == 3 || g == 4) && NT == 256 && GM >= 20;  // uniform
+  const int stid = specw ? (tid & 127) : tid;
+  const int slot = stid / tps, sub = stid % tps;
   const bool act = slot < BS_LEVELS * g;
   const int lev = act ? slot / g : 0;  // level k = lev + 1, n_k = 2k substeps
   const int q = act ? slot % g : 0;
@@ -112,12 +117,12 @@ __device__ void bs_group(BsSharedT<GM> &sh, const Sim &S, const DevParams &P, do
   // serial step control's next attempt would be that one (the attempt at H failed), so results and
   // decisions are the serial algorithm's, and a failed attempt no longer costs a round of its own.
   const bool spec = g <= 2 && tps == 4 && NT >= 128 && GM >= 18;  // uniform
-  const int half = spec ? (sub >> 1) : 0, tsub = spec ? (sub & 1) : sub, ttps = spec ? 2 : tps;
+  const int half = spec ? (sub >> 1) : (specw ? tid >> 7 : 0), tsub = spec ? (sub & 1) : sub, ttps = spec ? 2 : tps;
   const int qm = q + 16 * half;  // this thread's member in its attempt's position and tableau arrays
   const int oc = ttps == 4 ? tsub : 2 * tsub;  // this thread's components: oc .. oc + on - 1
   const int on = ttps == 4 ? (tsub < 3 ? 1 : 0) : (ttps == 2 ? 2 - tsub : 3);
-  const int trow = (spec && tid >= 64) ? tid - 64 : tid;  // tableau thread of attempt (spec && tid >= 64)
-  const int thalf = (spec && tid >= 64) ? 1 : 0;
+  const int tb = spec ? 64 : (specw ? 128 : NT);  // tableau threads from tb on: the attempt at H/2
+  const int thalf = tid >= tb ? 1 : 0, trow = thalf ? tid - tb : tid;
   if (tid < g) {
     const int i = S.gmem[g0 + tid];
     sh.idx[tid] = i;
@@ -141,16 +146,18 @@ __device__ void bs_group(BsSharedT<GM> &sh, const Sim &S, const DevParams &P, do
     // attempt stops at the first converged level: the same decision as building the whole
     // tableau first, but attempts that converge at level 4-6 (almost all) skip the deeper chains.
     const double h = __ddiv_rn(half ? 0.5 * H : H, (double)nk), h2 = 2.0 * h;
-    const bool qa = act && sh.alive[q];
+    const bool specn = spec || (specw && attempts > 1);  // uniform: this attempt has its twin at H/2
+    const bool acta = act && (half == 0 || specn);
+    const bool qa = acta && sh.alive[q];
     double xA[3], vA[3], xB[3], vB[3];  // the two newest states of the level's chain, own components
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       xA[k] = k < on ? sh.y[q][oc + k] : 0.0;
       vA[k] = k < on ? sh.y[q][3 + oc + k] : 0.0;
-      if (act && k < on) sh.pos[0][lev][qm][oc + k] = xA[k];
+      if (acta && k < on) sh.pos[0][lev][qm][oc + k] = xA[k];
     }
     const int qc = trow / 6, cc = trow % 6;
-    const bool rowth = qc < g;
+    const bool rowth = qc < g && (thalf == 0 || specn);
     double scale = 0.0;  // error scale of (qc, cc): 1/|x| or 1/|v| at the start of the attempt
     if (rowth) {
       const double *yq = sh.y[qc] + (cc < 3 ? 0 : 3);
@@ -162,7 +169,7 @@ __device__ void bs_group(BsSharedT<GM> &sh, const Sim &S, const DevParams &P, do
     double ac[3] = {0.0, 0.0, 0.0};
     // every lane of a warp that holds any active slot takes part (the sums shuffle across lanes);
     // warps without active slots stay off the pipes
-    if (__any_sync(0xffffffffu, act)) bs_accel(sh, P, Gm0, g, q, tsub, ttps, sh.pos[0][lev] + 16 * half, qa, ac);
+    if (__any_sync(0xffffffffu, acta)) bs_accel(sh, P, Gm0, g, q, tsub, ttps, sh.pos[0][lev] + 16 * half, qa, ac);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       if (k >= on) continue;
@@ -175,7 +182,7 @@ __device__ void bs_group(BsSharedT<GM> &sh, const Sim &S, const DevParams &P, do
     int acc = 0, accB = 0;
     int b = 1;
     for (int e = 1; e <= 2 * lmax; ++e) {
-      const bool lv = act && e <= nk;
+      const bool lv = acta && e <= nk;
       if (lv) {
 #pragma unroll
         for (int k = 0; k < 3; ++k)
@@ -212,7 +219,7 @@ __device__ void bs_group(BsSharedT<GM> &sh, const Sim &S, const DevParams &P, do
       }
       if (Lc >= 2) warp_max_to(thalf ? &sh.err2[Lc - 1] : &sh.err[Lc - 1], ev);  // thalf is uniform per warp
       __syncthreads();
-      if (spec && !accB && Lc >= 2 && sh.err2[Lc - 1] <= eps) {  // the attempt at H/2 converged (uniform)
+      if (specn && !accB && Lc >= 2 && sh.err2[Lc - 1] <= eps) {  // the attempt at H/2 converged (uniform)
         accB = Lc;
         if (thalf && rowth) sh.yn[qc + 16][cc] = tlast;
       }
@@ -220,7 +227,7 @@ __device__ void bs_group(BsSharedT<GM> &sh, const Sim &S, const DevParams &P, do
     }
     if (acc && rowth && !thalf) sh.yn[qc][cc] = tlast;  // the accepted row is the last one built
     double Hs = H;  // length of the accepted substep
-    if (!acc && spec) {  // the serial control halves H; its next attempt is the one at H/2
+    if (!acc && specn) {  // the serial control halves H; its next attempt is the one at H/2
       if (++halvings > P.bs_max_halvings) {
         if (tid == 0) atomicOr(S.status, ST_BS_FAILED);
         __syncthreads();

@@ -13,6 +13,7 @@ import pytest
 import oracle as O
 from paper_1404_2324_gb300 import genga, ics
 from tests.gpu_util import aos, dev, soa
+from tests.test_gpu_phases import _bs_phase_vs_oracle, _clumps
 
 pytestmark = pytest.mark.gpu
 
@@ -59,3 +60,14 @@ def test_pulls_across_the_changeover_zone_match_the_oracle(kmode, size, mass, rc
     for got, want in ((aos(X), rx), (aos(V), rv)):
         err = np.linalg.norm(got - want, axis=1) / np.linalg.norm(want, axis=1)
         assert err.max() <= 2e-12, (err.max(), int(err.argmax()))
+
+
+@pytest.mark.parametrize("seed,spread,R", [(1, 0.0002, None), (8, 0.0002, None), (4, 0.0003, 2e-5), (6, 0.0003, 2e-5)])
+def test_groups_of_three_and_four_with_failed_attempts_match_the_oracle(seed, spread, R):
+    """Tight groups of three and four members, up to nine substeps with failed attempts between them
+    and, with the larger radii, mergers: from the second attempt on the attempt at H/2 runs in the
+    other half of the CTA and is taken exactly when the serial control would try it next."""
+    x, v, m, Rr, groups = _clumps((3, 4) * 4, seed=seed, spread=spread, R=R)
+    ref, U = _bs_phase_vs_oracle(x, v, m, Rr, groups)
+    assert ref["steps"] > len(groups) and (ref["coll"] > 0) == (R is not None)
+    assert U == pytest.approx(ref["U"], rel=1e-9)
