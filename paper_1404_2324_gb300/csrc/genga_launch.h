@@ -19,7 +19,7 @@ void launch_fin(const Sim &S, const DevParams &P, FinMode mode, bool precise, do
                 cudaStream_t st);
 void launch_hc(const Sim &S, double hcm, cudaStream_t st);
 // the fixed-point pair kernel's chunks of partners per tile, partners per chunk
-void kick_split(int npad, int sms, int *chunks, int *chunk);
+void kick_split(int npad, int sms, int *chunks, int *chunk, int systems = 1);
 
 // step.cu
 void launch_drift(const Sim &S, const DevParams &P, double tau, double hcm1, double hcm2,

@@ -6,8 +6,7 @@
 // root and division) evaluates every unordered pair once in FP64. Both leave partial sums per body
 // tile in a fixed layout that the finalisation sums in a fixed order, so results are bitwise
 // reproducible.
-#include "fxpair.cuh"
-#include "genga_launch.h"
+#include "kick_fx.cuh"
 
 namespace genga {
 
@@ -165,47 +164,9 @@ __global__ void __launch_bounds__(128) k_kick_precise(Sim S, DevParams P, int fo
 }
 
 // ---------------------------------------------------------------------------------------------
-// Fixed-point pair kernel. A CTA holds TW tiles of 32 bodies, a warp each, one body a lane, and CW
-// chunks of at most 64 partners in shared memory (TW CW = 8 warps); a warp sums one tile's pulls
-// from one chunk into that (tile, chunk)'s slot. FULL and the candidates as in k_kick_precise; every
-// body records its own row of the bitmap.
-//
-// Pass 1 separates the near partners -- inside the precheck radius, or closer than the fixed-point
-// grid resolves, or the body itself -- into a bit mask and bounds the sum of the others. Pass 2 sums
-// the far pulls. The near pairs of the warp are then listed and taken one a lane in FP64 with the
-// exact decision arithmetic. A CTA with a number the fixed-point form cannot hold (not finite, a
-// negative mass) takes every pair as near.
-//
-// No Newton's third law: the sums of the j side would rotate through the lanes with 24 more
-// shuffled words a pair (4 cycles each), as much as evaluating the pair once more.
+// Fixed-point pair kernel (kick_fx.cuh): FULL and the candidates as in k_kick_precise; every body records
+// its own row of the bitmap. The sums of a (tile, chunk) go to its slot.
 // ---------------------------------------------------------------------------------------------
-constexpr int KX_WARPS = 8;
-constexpr int KX_CTAS = 3;  // CTAs per SM (80 registers; measured at N = 2048: two 33.9 us, three 33.7 us a kick)
-constexpr int KX_LIST = 96;  // near pairs of a warp taken together; more: each lane takes its own in turn
-constexpr int KX_SMALL = 8;  // partners a chunk for fewer than 8 tiles
-template <int CAP>
-struct KxShared {
-  float4 h[CAP], m[CAP];  // position in single precision (h + m); .w: mass, its exponent
-  longlong2 xy[CAP], zM[CAP];
-  float lim[CAP];
-};
-struct KxList {  // near pairs: body lane << 8 | partner, and their pulls
-  int e[KX_LIST];
-  double f[3][KX_LIST];
-};
-
-// max(T, grid limit) as the first pass's limit on rough r^2 (units of 2^(2E - 60)), rounded up by
-// 2^-10 (rough r^2 is within 2^-12).
-__device__ __forceinline__ float kx_limit(u64 T, int E) {
-  const float t = scalbnf(d2f_safe(__longlong_as_double((long long)T)), 60 - 2 * E);
-  return fmaxf(t, fx::FX_RMIN2) * 1.001f;
-}
-__device__ __forceinline__ float kx_norm2(double x, double y, double z) {  // |x|^2, rounded up
-  const float a = d2f_safe(x), b = d2f_safe(y), c = d2f_safe(z);
-  return fmaf(c, c, fmaf(b, b, a * a)) * 1.000002f;
-}
-__device__ __forceinline__ bool kx_odd(double x) { return fx::expo(x) == 0x7ff; }
-
 // The pair (i, j) in FP64: records a candidate, returns the pull's factor (0: nothing to add here).
 template <bool FULL>
 __device__ __forceinline__ double kx_near(const Sim &S, const DevParams &P, int i, int j, bool record, double &dx,
@@ -237,14 +198,8 @@ template <bool FULL, int TW>
 __global__ void __launch_bounds__(32 * KX_WARPS, KX_CTAS) k_kick_fx(Sim S, DevParams P, int force) {
   if (FULL && !force && S.flags[0] == 0) return;
   const bool record = FULL ? (!force && S.flags[3] != 0) : true;
-  constexpr int CW = KX_WARPS / TW, CAP = TW == 8 ? fx::FX_CHUNK : KX_SMALL;
-  __shared__ KxShared<CAP> smem[CW];
-  __shared__ KxList slist[KX_WARPS];
-  __shared__ int s_n2, s_me[CW];
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  const int np = S.npad, C = S.kch, nt = S.nt;
-  const double *__restrict__ X = S.x;
-  const int gwarp = blockIdx.x * KX_WARPS + wid;
+  const int lane = threadIdx.x & 31, np = S.npad, C = S.kch, nt = S.nt;
+  const int gwarp = blockIdx.x * KX_WARPS + (threadIdx.x >> 5);
   if ((!FULL || force) && gwarp < nt) {  // per-tile momentum before the closing kick (second Sun drift)
     const int i = gwarp * 32 + lane;
     const double mi = S.m[i];
@@ -255,143 +210,14 @@ __global__ void __launch_bounds__(32 * KX_WARPS, KX_CTAS) k_kick_fx(Sim S, DevPa
     }
   }
   const int tgroups = (nt + TW - 1) / TW;
-  const int I = (blockIdx.x % tgroups) * TW + wid % TW, cw = wid / TW, c0 = (blockIdx.x / tgroups) * CW + cw;
-  const bool on = I < nt && c0 < C;
-  if (tid == 0) s_n2 = 0;
-  if (tid < CW) s_me[tid] = -2000;
-  // own body; partners (one a thread, twice over when the CTA holds more than four chunks)
-  const int i = min(I, nt - 1) * 32 + lane;
-  const bool ali = on && S.alive[i] != 0;
-  const double xi = ali ? X[i] : 0.0, yi = ali ? X[np + i] : 0.0, zi = ali ? X[2 * np + i] : 0.0;
-  const u64 Ti = ali ? S.T[i] : 0ULL;
-  constexpr int NB = CW * CAP, PB = (NB + 32 * KX_WARPS - 1) / (32 * KX_WARPS);
-  double bx[PB], by[PB], bz[PB], bg[PB];
-  u64 bT[PB];
-  float n2 = kx_norm2(xi, yi, zi);
-  bool odd = kx_odd(xi) || kx_odd(yi) || kx_odd(zi);
-#pragma unroll
-  for (int k = 0; k < PB; ++k) {
-    const int q = tid + 32 * KX_WARPS * k, ch = (blockIdx.x / tgroups) * CW + q / CAP, u = q % CAP;
-    const int j = ch * S.kchunk + u;
-    const bool al = q < NB && ch < C && u < S.kchunk && j < np && S.alive[j] != 0;
-    bx[k] = al ? X[j] : 0.0; by[k] = al ? X[np + j] : 0.0; bz[k] = al ? X[2 * np + j] : 0.0;
-    bg[k] = al ? S.gm[j] : 0.0;
-    bT[k] = al ? S.T[j] : 0ULL;
-    n2 = fmaxf(n2, kx_norm2(bx[k], by[k], bz[k]));
-    odd |= kx_odd(bx[k]) || kx_odd(by[k]) || kx_odd(bz[k]) || kx_odd(bg[k]) || (long long)dbits(bg[k]) < 0;
-  }
-  __syncthreads();
-  // common scale: |x| < 2^E; per chunk the largest mass exponent
-  const int wn2 = __reduce_max_sync(0xffffffffu, __float_as_int(n2));
-  if (lane == 0) atomicMax(&s_n2, wn2);
-#pragma unroll
-  for (int k = 0; k < PB; ++k) {
-    const int q = tid + 32 * KX_WARPS * k;
-    if (q >= NB) continue;
-    u64 M;
-    int me;
-    fx::set_mass(bg[k], M, me);
-    if (M) atomicMax(&s_me[q / CAP], me);
-  }
-  odd = __syncthreads_or(odd) || s_n2 >= 0x7f000000;
-  const int E = odd ? 0 : ((s_n2 >> 23) - 127 + 2) >> 1;
-#pragma unroll
-  for (int k = 0; k < PB; ++k) {
-    const int q = tid + 32 * KX_WARPS * k;
-    if (q >= NB) continue;
-    KxShared<CAP> &sm = smem[q / CAP];
-    const int u = q % CAP;
-    fx::Pos p;
-    u64 M;
-    int me;
-    fx::set_pos(p, odd ? 0.0 : bx[k], odd ? 0.0 : by[k], odd ? 0.0 : bz[k], E);
-    fx::set_mass(odd ? 0.0 : bg[k], M, me);
-    sm.h[u] = make_float4(p.hx, p.hy, p.hz, fx::mass_f(M, me, s_me[q / CAP]));
-    sm.m[u] = make_float4(p.mx, p.my, p.mz, __int_as_float(me));
-    sm.xy[u] = make_longlong2(p.X, p.Y);
-    sm.zM[u] = make_longlong2(p.Z, (long long)M);
-    sm.lim[u] = kx_limit(bT[k], E);
-  }
-  fx::Pos pi;
-  fx::set_pos(pi, odd ? 0.0 : xi, odd ? 0.0 : yi, odd ? 0.0 : zi, E);
-  const float limi = odd ? __int_as_float(0x7f800000) : kx_limit(Ti, E);
-  __syncthreads();
+  int I, c0;
+  bool ali;
+  double ax, ay, az;
+  const bool on = kx_block<TW>(
+      S.x, np, S.gm, S.alive, S.T, 0, np, nt, C, S.kchunk, blockIdx.x % tgroups, blockIdx.x / tgroups,
+      [&](int i, int j, double &dx, double &dy, double &dz) { return kx_near<FULL>(S, P, i, j, record, dx, dy, dz); }, I, c0,
+      ali, ax, ay, az);
   if (!on) return;
-  const KxShared<CAP> &sm = smem[cw];
-  const int j0 = c0 * S.kchunk, cnt = min(S.kchunk, np - j0);  // at least one partner
-  // pass 1: near partners, bound of the far sum
-  unsigned near[2] = {0u, 0u};
-  float B = 0.0f;
-#pragma unroll
-  for (int w = 0; w < 2; ++w) {
-    const int n = min(cnt - 32 * w, 32);
-#pragma unroll 4
-    for (int k = 0; k < n; ++k) {
-      const float4 h = sm.h[32 * w + k];
-      const float r2 = fx::rough_r2(pi, h.x, h.y, h.z);
-      if (r2 >= fmaxf(limi, sm.lim[32 * w + k])) B = fmaf(h.w, fx::frcp(r2), B);
-      else near[w] |= 1u << k;
-    }
-  }
-  // pass 2: the far pulls
-  const int A = fx::units(B, s_me[cw]);
-  fx::Acc acc;
-  fx::clear(acc);
-#pragma unroll
-  for (int w = 0; w < 2; ++w) {
-    const int n = min(cnt - 32 * w, 32);
-    for (int k0 = 0; k0 < n; k0 += fx::FX_FLUSH) {
-      const int k1 = min(n, k0 + fx::FX_FLUSH);
-#pragma unroll 2
-      for (int k = k0; k < k1; ++k) {
-        const float4 h = sm.h[32 * w + k], m = sm.m[32 * w + k];
-        const longlong2 a = sm.xy[32 * w + k], b = sm.zM[32 * w + k];
-        const fx::Pos pj = {a.x, a.y, b.x, h.x, h.y, h.z, m.x, m.y, m.z};
-        fx::pull(pi, pj, (u64)b.y, __float_as_int(m.w), A, !((near[w] >> k) & 1u), acc);
-      }
-      fx::flush(acc);
-    }
-  }
-  double ax = fx::value(acc.h[0], acc.l[0], A, E), ay = fx::value(acc.h[1], acc.l[1], A, E),
-         az = fx::value(acc.h[2], acc.l[2], A, E);
-  // the near pairs in FP64: listed by (body, partner), one a lane, added per body in partner order
-  {
-    const unsigned self = I * 32 + lane - j0;  // the body itself is not a pair
-    if (self < 32u) near[0] &= ~(1u << self);
-    else if (self < 64u) near[1] &= ~(1u << (self - 32u));
-    if (!ali) { near[0] = 0u; near[1] = 0u; }
-  }
-  const int nn = __popc(near[0]) + __popc(near[1]);
-  int incl = nn;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int t = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += t;
-  }
-  const int total = __shfl_sync(0xffffffffu, incl, 31);
-  if (total > 0 && total <= KX_LIST) {
-    KxList &L = slist[wid];
-    int at = incl - nn;
-#pragma unroll
-    for (int w = 0; w < 2; ++w)
-      for (unsigned bits = near[w]; bits; bits &= bits - 1) L.e[at++] = lane << 8 | (32 * w + __ffs(bits) - 1);
-    __syncwarp();
-    for (int k = lane; k < total; k += 32) {
-      double dx = 0.0, dy = 0.0, dz = 0.0;
-      const double g = kx_near<FULL>(S, P, I * 32 + (L.e[k] >> 8), j0 + (L.e[k] & 255), record, dx, dy, dz);
-      L.f[0][k] = g * dx; L.f[1][k] = g * dy; L.f[2][k] = g * dz;
-    }
-    __syncwarp();
-    for (int k = incl - nn; k < incl; ++k) { ax += L.f[0][k]; ay += L.f[1][k]; az += L.f[2][k]; }
-  } else if (total > 0) {
-#pragma unroll
-    for (int w = 0; w < 2; ++w)
-      for (unsigned bits = near[w]; bits; bits &= bits - 1) {
-        double dx = 0.0, dy = 0.0, dz = 0.0;
-        const double g = kx_near<FULL>(S, P, i, j0 + 32 * w + __ffs(bits) - 1, record, dx, dy, dz);
-        ax += g * dx; ay += g * dy; az += g * dz;
-      }
-  }
   double *p = S.part + ((size_t)I * C + c0) * 96 + lane;
   p[0] = ali ? ax : 0.0; p[32] = ali ? ay : 0.0; p[64] = ali ? az : 0.0;
 }
@@ -399,10 +225,10 @@ __global__ void __launch_bounds__(32 * KX_WARPS, KX_CTAS) k_kick_fx(Sim S, DevPa
 // The fixed-point kernel's split of a tile's partners: chunks per tile, partners per chunk. About 8
 // KX_CTAS warps per SM, at least 8 partners a chunk (below that the set-up of a warp outweighs its
 // loop), at most 64 (the bit masks). Up to 1024 bodies at most 2048 chunks in all (the partial-sum
-// slots of the static scratch).
-void kick_split(int npad, int sms, int *chunks, int *chunk) {
+// slots of the static scratch). systems: equal systems summed by one launch.
+void kick_split(int npad, int sms, int *chunks, int *chunk, int systems) {
   const int nt = npad / 32, lo = (npad + fx::FX_CHUNK - 1) / fx::FX_CHUNK, hi = npad / KX_SMALL;
-  int C = KX_WARPS * KX_CTAS * sms / nt;
+  int C = (int)((long)KX_WARPS * KX_CTAS * sms / ((long)nt * systems));
   if (nt <= 32 && C > 2048 / nt) C = 2048 / nt;
   if (C > hi || nt < 8) C = hi;  // chunks of KX_SMALL
   if (C < lo) C = lo;

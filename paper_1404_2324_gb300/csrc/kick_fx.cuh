@@ -1,0 +1,211 @@
+// kick_fx.cuh -- the fixed-point sum of the pulls on tiles of bodies, shared by the main mode's pair
+// kernel (kick.cu) and the differentiable engine's (adjoint.cu).
+//
+// A CTA holds TW tiles of 32 bodies, a warp each, one body a lane, and CW chunks of at most 64
+// partners in shared memory (TW CW = 8 warps); a warp sums one tile's pulls from one chunk.
+//
+// Pass 1 separates the near partners -- inside the caller's limit radius, or closer than the
+// fixed-point grid resolves, or the body itself -- into a bit mask and bounds the sum of the others.
+// Pass 2 sums the far pulls (fxpair.cuh). The near pairs of the warp are then listed and handed to
+// the caller one a lane, in FP64 with its exact decisions. A CTA with a number the fixed-point form
+// cannot hold (not finite, a negative mass) takes every pair as near.
+//
+// What bounds it at N = 2048 (32.6 us, 33.6 with its event nodes; the FP64 tile ring it replaced 87):
+// the wide multiply-adds' pipe, 62 % busy, 30 of them a pull at 4 cycles; pass 1 about 6 us, set-up and
+// launch 8 us, the near pairs 3 us. Two CTAs per SM measured the same as three.
+//
+// No Newton's third law: the sums of the j side would rotate through the lanes with 24 more
+// shuffled words a pair (4 cycles each), as much as evaluating the pair once more.
+#pragma once
+#include "fxpair.cuh"
+#include "genga_launch.h"
+
+namespace genga {
+
+constexpr int KX_WARPS = 8;
+constexpr int KX_CTAS = 3;  // CTAs per SM (80 registers; measured at N = 2048: two 33.9 us, three 33.7 us a kick)
+constexpr int KX_LIST = 96;  // near pairs of a warp taken together; more: each lane takes its own in turn
+constexpr int KX_SMALL = 8;  // partners a chunk for fewer than 8 tiles
+template <int CAP>
+struct KxShared {
+  float4 h[CAP], m[CAP];  // position in single precision (h + m); .w: mass, its exponent
+  longlong2 xy[CAP], zM[CAP];
+  float lim[CAP];
+};
+struct KxList {  // near pairs: body lane << 8 | partner, and their pulls
+  int e[KX_LIST];
+  double f[3][KX_LIST];
+};
+
+// max(T, grid limit) as the first pass's limit on rough r^2 (units of 2^(2E - 60)), rounded up by
+// 2^-10 (rough r^2 is within 2^-12).
+__device__ __forceinline__ float kx_limit(u64 T, int E) {
+  const float t = scalbnf(d2f_safe(__longlong_as_double((long long)T)), 60 - 2 * E);
+  return fmaxf(t, fx::FX_RMIN2) * 1.001f;
+}
+__device__ __forceinline__ float kx_norm2(double x, double y, double z) {  // |x|^2, rounded up
+  const float a = d2f_safe(x), b = d2f_safe(y), c = d2f_safe(z);
+  return fmaf(c, c, fmaf(b, b, a * a)) * 1.000002f;
+}
+__device__ __forceinline__ bool kx_odd(double x) { return fx::expo(x) == 0x7ff; }
+
+// The pulls on body (base + I 32 + lane), I = tg TW + wid % TW, from the partners of chunk c0 = cg CW +
+// wid / TW (kchunk partners each, np bodies, nt tiles, C chunks) into (ax, ay, az); x: component-major
+// with leading dimension ld. lim: squared limit radii (bits); a pair inside max(lim_i, lim_j), or
+// closer than the grid resolves, is near(i, j, dx, dy, dz)'s, which returns the pull's factor.
+// Returns false for a warp without a tile and chunk. All threads of the CTA call it.
+template <int TW, class Near>
+__device__ __forceinline__ bool kx_block(const double *__restrict__ X, int ld, const double *__restrict__ gm,
+                                         const int *__restrict__ alive, const u64 *__restrict__ lim, int base, int np,
+                                         int nt, int C, int kchunk, int tg, int cg, Near near_pair, int &I, int &c0,
+                                         bool &ali, double &ax, double &ay, double &az) {
+  constexpr int CW = KX_WARPS / TW, CAP = TW == 8 ? fx::FX_CHUNK : KX_SMALL;
+  __shared__ KxShared<CAP> smem[CW];
+  __shared__ KxList slist[KX_WARPS];
+  __shared__ int s_n2, s_me[CW];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int cw = wid / TW;
+  I = tg * TW + wid % TW;
+  c0 = cg * CW + cw;
+  const bool on = I < nt && c0 < C;
+  if (tid == 0) s_n2 = 0;
+  if (tid < CW) s_me[tid] = -2000;
+  // own body; partners (one a thread, twice over when the CTA holds more than four chunks)
+  const int i = base + min(I, nt - 1) * 32 + lane;
+  ali = on && alive[i] != 0;
+  const double xi = ali ? X[i] : 0.0, yi = ali ? X[ld + i] : 0.0, zi = ali ? X[2 * ld + i] : 0.0;
+  const u64 Ti = ali ? lim[i] : 0ULL;
+  constexpr int NB = CW * CAP, PB = (NB + 32 * KX_WARPS - 1) / (32 * KX_WARPS);
+  double bx[PB], by[PB], bz[PB], bg[PB];
+  u64 bT[PB];
+  float n2 = kx_norm2(xi, yi, zi);
+  bool odd = kx_odd(xi) || kx_odd(yi) || kx_odd(zi);
+#pragma unroll
+  for (int k = 0; k < PB; ++k) {
+    const int q = tid + 32 * KX_WARPS * k, ch = cg * CW + q / CAP, u = q % CAP;
+    const int jl = ch * kchunk + u, j = base + jl;
+    const bool al = q < NB && ch < C && u < kchunk && jl < np && alive[j] != 0;
+    bx[k] = al ? X[j] : 0.0; by[k] = al ? X[ld + j] : 0.0; bz[k] = al ? X[2 * ld + j] : 0.0;
+    bg[k] = al ? gm[j] : 0.0;
+    bT[k] = al ? lim[j] : 0ULL;
+    n2 = fmaxf(n2, kx_norm2(bx[k], by[k], bz[k]));
+    odd |= kx_odd(bx[k]) || kx_odd(by[k]) || kx_odd(bz[k]) || kx_odd(bg[k]) || (long long)dbits(bg[k]) < 0;
+  }
+  __syncthreads();
+  // common scale: |x| < 2^E; per chunk the largest mass exponent
+  const int wn2 = __reduce_max_sync(0xffffffffu, __float_as_int(n2));
+  if (lane == 0) atomicMax(&s_n2, wn2);
+#pragma unroll
+  for (int k = 0; k < PB; ++k) {
+    const int q = tid + 32 * KX_WARPS * k;
+    if (q >= NB) continue;
+    u64 M;
+    int me;
+    fx::set_mass(bg[k], M, me);
+    if (M) atomicMax(&s_me[q / CAP], me);
+  }
+  odd = __syncthreads_or(odd) || s_n2 >= 0x7f000000;
+  const int E = odd ? 0 : ((s_n2 >> 23) - 127 + 2) >> 1;
+#pragma unroll
+  for (int k = 0; k < PB; ++k) {
+    const int q = tid + 32 * KX_WARPS * k;
+    if (q >= NB) continue;
+    KxShared<CAP> &sm = smem[q / CAP];
+    const int u = q % CAP;
+    fx::Pos p;
+    u64 M;
+    int me;
+    fx::set_pos(p, odd ? 0.0 : bx[k], odd ? 0.0 : by[k], odd ? 0.0 : bz[k], E);
+    fx::set_mass(odd ? 0.0 : bg[k], M, me);
+    sm.h[u] = make_float4(p.hx, p.hy, p.hz, fx::mass_f(M, me, s_me[q / CAP]));
+    sm.m[u] = make_float4(p.mx, p.my, p.mz, __int_as_float(me));
+    sm.xy[u] = make_longlong2(p.X, p.Y);
+    sm.zM[u] = make_longlong2(p.Z, (long long)M);
+    sm.lim[u] = kx_limit(bT[k], E);
+  }
+  fx::Pos pi;
+  fx::set_pos(pi, odd ? 0.0 : xi, odd ? 0.0 : yi, odd ? 0.0 : zi, E);
+  const float limi = odd ? __int_as_float(0x7f800000) : kx_limit(Ti, E);
+  __syncthreads();
+  ax = ay = az = 0.0;
+  if (!on) return false;
+  const KxShared<CAP> &sm = smem[cw];
+  const int j0 = c0 * kchunk, cnt = min(kchunk, np - j0);  // at least one partner
+  // pass 1: near partners, bound of the far sum
+  unsigned near[2] = {0u, 0u};
+  float B = 0.0f;
+#pragma unroll
+  for (int w = 0; w < 2; ++w) {
+    const int n = min(cnt - 32 * w, 32);
+#pragma unroll 4
+    for (int k = 0; k < n; ++k) {
+      const float4 h = sm.h[32 * w + k];
+      const float r2 = fx::rough_r2(pi, h.x, h.y, h.z);
+      if (r2 >= fmaxf(limi, sm.lim[32 * w + k])) B = fmaf(h.w, fx::frcp(r2), B);
+      else near[w] |= 1u << k;
+    }
+  }
+  // pass 2: the far pulls
+  const int A = fx::units(B, s_me[cw]);
+  fx::Acc acc;
+  fx::clear(acc);
+#pragma unroll
+  for (int w = 0; w < 2; ++w) {
+    const int n = min(cnt - 32 * w, 32);
+    for (int k0 = 0; k0 < n; k0 += fx::FX_FLUSH) {
+      const int k1 = min(n, k0 + fx::FX_FLUSH);
+#pragma unroll 2
+      for (int k = k0; k < k1; ++k) {
+        const float4 h = sm.h[32 * w + k], m = sm.m[32 * w + k];
+        const longlong2 a = sm.xy[32 * w + k], b = sm.zM[32 * w + k];
+        const fx::Pos pj = {a.x, a.y, b.x, h.x, h.y, h.z, m.x, m.y, m.z};
+        fx::pull(pi, pj, (u64)b.y, __float_as_int(m.w), A, !((near[w] >> k) & 1u), acc);
+      }
+      fx::flush(acc);
+    }
+  }
+  ax = fx::value(acc.h[0], acc.l[0], A, E);
+  ay = fx::value(acc.h[1], acc.l[1], A, E);
+  az = fx::value(acc.h[2], acc.l[2], A, E);
+  // the near pairs in FP64: listed by (body, partner), one a lane, added per body in partner order
+  {
+    const unsigned self = I * 32 + lane - j0;  // the body itself is not a pair
+    if (self < 32u) near[0] &= ~(1u << self);
+    else if (self < 64u) near[1] &= ~(1u << (self - 32u));
+    if (!ali) { near[0] = 0u; near[1] = 0u; }
+  }
+  const int nn = __popc(near[0]) + __popc(near[1]);
+  int incl = nn;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += t;
+  }
+  const int total = __shfl_sync(0xffffffffu, incl, 31);
+  if (total > 0 && total <= KX_LIST) {
+    KxList &L = slist[wid];
+    int at = incl - nn;
+#pragma unroll
+    for (int w = 0; w < 2; ++w)
+      for (unsigned bits = near[w]; bits; bits &= bits - 1) L.e[at++] = lane << 8 | (32 * w + __ffs(bits) - 1);
+    __syncwarp();
+    for (int k = lane; k < total; k += 32) {
+      double dx = 0.0, dy = 0.0, dz = 0.0;
+      const double g = near_pair(base + I * 32 + (L.e[k] >> 8), base + j0 + (L.e[k] & 255), dx, dy, dz);
+      L.f[0][k] = g * dx; L.f[1][k] = g * dy; L.f[2][k] = g * dz;
+    }
+    __syncwarp();
+    for (int k = incl - nn; k < incl; ++k) { ax += L.f[0][k]; ay += L.f[1][k]; az += L.f[2][k]; }
+  } else if (total > 0) {
+#pragma unroll
+    for (int w = 0; w < 2; ++w)
+      for (unsigned bits = near[w]; bits; bits &= bits - 1) {
+        double dx = 0.0, dy = 0.0, dz = 0.0;
+        const double g = near_pair(i, base + j0 + 32 * w + __ffs(bits) - 1, dx, dy, dz);
+        ax += g * dx; ay += g * dy; az += g * dz;
+      }
+  }
+  return true;
+}
+
+}  // namespace genga

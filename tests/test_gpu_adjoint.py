@@ -199,3 +199,22 @@ def test_autograd_function_and_single_body():
     got = np.concatenate([X.grad.cpu().numpy().ravel(), V.grad.cpu().numpy().ravel(), M.grad.cpu().numpy().ravel()])
     np.testing.assert_allclose(got[:6], ref[:6], rtol=1e-9, atol=1e-12 * np.abs(ref[:6]).max())
     eng.close()
+
+
+@pytest.mark.parametrize("n", [2, 31, 32, 33, 64, 65, 100, 129, 225, 256, 257, 400])
+def test_forward_kick_at_tile_and_chunk_edges(n):
+    """One step of three systems of n bodies, up to each number of tiles a CTA of the forward kick
+    takes and with ragged last tiles and chunks: the bound of the one-step test above."""
+    rng = np.random.default_rng(n)  # rings as dense as the compact ones above, however many bodies
+    d = [ics._disk(rng, n, 1e-7, 1e-6, 0.95, (0.9025 + 0.00418 * n) ** 0.5, 0.01, 0.005) for _ in range(3)]
+    x, v, m = (np.array([q[k] for q in d]) for k in "xvm")
+    x[2, 0] *= 300.0  # a system the kick's grid resolves less finely than its close pairs
+    v[2, 0] /= 300.0 ** 0.5
+    eng = AdjointEngine(np.ones(3), G, 6.0, 2, ckpt_every=10)
+    xo, vo = eng.forward(_t(x), _t(v), _t(m), 1)
+    ref = _oracle_run(x, v, m, 2, 1)
+    alt = _oracle_run(x, v, m, 2, 1, perturb=1e-15 * rng.standard_normal(x.shape))
+    for b in range(3):
+        for got, k in ((xo, 0), (vo, 1)):
+            assert _rel(got[b].cpu().numpy(), ref[b][k]) <= max(1e-12, 30 * _rel(alt[b][k], ref[b][k])), (b, k)
+    eng.close()
