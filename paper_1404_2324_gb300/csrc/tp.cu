@@ -17,6 +17,7 @@
 #include <cstring>
 
 #include "fxforce.cuh"
+#include "kick_fx.cuh"
 #include "genga_launch.h"
 
 namespace genga {
@@ -107,6 +108,111 @@ __device__ __forceinline__ void tp_close_forces_k(const TPSet &T, const DevParam
     T.cmask[i[k]] = cm[k];
     for (int c = 0; c < 3; ++c) acc[k][c] = f[k][c] + n[k][c];
   }
+}
+
+// The same forces in fixed point (fxpair.cuh) on two TPs a lane: the far pulls of the warp's planets on
+// a common grid with the TPs, the candidates (and pairs the grid does not resolve) in FP64 as above.
+// Called by whole warps; pl: the warp's shared memory. About 17 FP64 instructions a (TP, planet) pair,
+// 64-76 cycles each, become 115 others, 1-4 cycles each.
+struct PlanetFx {
+  float4 h[TP_MAXPL], m[TP_MAXPL];
+  longlong2 xy[TP_MAXPL], zM[TP_MAXPL];
+  float lim[TP_MAXPL];
+};
+
+__device__ __forceinline__ void tp_close_forces_fx(const TPSet &T, const DevParams &P, const PlanetSm &ps, PlanetFx &pl,
+                                                   int npl, const int (&i)[2], const bool (&act)[2],
+                                                   const double (&x)[2][3], double (&acc)[2][3], unsigned (&cm)[2]) {
+  const int lane = threadIdx.x & 31, np = T.npad;
+  float n2 = kx_norm2(ps.x[lane], ps.y[lane], ps.z[lane]);  // zero for a dead planet
+  const double gm = ps.gm[lane];
+  bool odd = kx_odd(ps.x[lane]) || kx_odd(ps.y[lane]) || kx_odd(ps.z[lane]) || kx_odd(gm) || (long long)dbits(gm) < 0;
+#pragma unroll
+  for (int k = 0; k < 2; ++k)
+    if (act[k]) {
+      n2 = fmaxf(n2, kx_norm2(x[k][0], x[k][1], x[k][2]));
+      odd |= kx_odd(x[k][0]) || kx_odd(x[k][1]) || kx_odd(x[k][2]);
+    }
+  const int nb = __reduce_max_sync(0xffffffffu, __float_as_int(n2));
+  if (__any_sync(0xffffffffu, odd) || nb >= 0x7f000000) {
+    tp_close_forces_k<2>(T, P, ps, npl, i, act, x, acc, cm);
+    return;
+  }
+  const int E = ((nb >> 23) - 127 + 2) >> 1;
+  int me_max;
+  {
+    fx::Pos p;
+    u64 M;
+    int me;
+    fx::set_pos(p, ps.x[lane], ps.y[lane], ps.z[lane], E);
+    fx::set_mass(gm, M, me);
+    me_max = __reduce_max_sync(0xffffffffu, M ? me : -2000);
+    pl.h[lane] = make_float4(p.hx, p.hy, p.hz, fx::mass_f(M, me, me_max));
+    pl.m[lane] = make_float4(p.mx, p.my, p.mz, __int_as_float(me));
+    pl.xy[lane] = make_longlong2(p.X, p.Y);
+    pl.zM[lane] = make_longlong2(p.Z, (long long)M);
+    pl.lim[lane] = kx_limit(ps.T[lane], E);
+  }
+  const unsigned live = __ballot_sync(0xffffffffu, ps.alive[lane] != 0);
+  __syncwarp();
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    cm[k] = 0u;
+    acc[k][0] = acc[k][1] = acc[k][2] = 0.0;
+    if (!__any_sync(0xffffffffu, act[k])) continue;
+    const u64 Ti = act[k] ? T.T[i[k]] : 0ULL;
+    fx::Pos pi;
+    fx::set_pos(pi, act[k] ? x[k][0] : 0.0, act[k] ? x[k][1] : 0.0, act[k] ? x[k][2] : 0.0, E);
+    const float limi = kx_limit(Ti, E);
+    unsigned near = 0u;
+    float B = 0.0f;
+    for (int j = 0; j < npl; ++j) {
+      const float4 h = pl.h[j];
+      const float r2 = fx::rough_r2(pi, h.x, h.y, h.z);
+      if (r2 >= fmaxf(limi, pl.lim[j])) B = fmaf(h.w, fx::frcp(r2), B);
+      else near |= 1u << j;
+    }
+    const int A = fx::units(B, me_max);
+    fx::Acc a;
+    fx::clear(a);
+    for (int j0 = 0; j0 < npl; j0 += fx::FX_FLUSH) {
+      const int j1 = min(npl, j0 + fx::FX_FLUSH);
+#pragma unroll 2
+      for (int j = j0; j < j1; ++j) {
+        const float4 h = pl.h[j], m = pl.m[j];
+        const longlong2 c = pl.xy[j], d = pl.zM[j];
+        const fx::Pos pj = {c.x, c.y, d.x, h.x, h.y, h.z, m.x, m.y, m.z};
+        fx::pull(pi, pj, (u64)d.y, __float_as_int(m.w), A, !((near >> j) & 1u), a);
+      }
+      fx::flush(a);
+    }
+    double f[3], n[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+    for (int c = 0; c < 3; ++c) f[c] = fx::value(a.h[c], a.l[c], A, E);
+    if (!act[k]) continue;
+    for (unsigned bits = near & live; bits; bits &= bits - 1) {
+      const int j = __ffs(bits) - 1;
+      const double dx = ps.x[j] - x[k][0], dy = ps.y[j] - x[k][1], dz = ps.z[j] - x[k][2];
+      const double r2 = r2_exact(dx, dy, dz);
+      const u64 rb = dbits(r2);
+      double g = ps.gm[j] * rcube_refined(r2);
+      if (rb < umax64(Ti, ps.T[j])) {
+        if (rb < umax64(T.rcsq[i[k]], ps.Q[j])) {  // inside the changeover zone (rare): the weight needs r
+          double wB, wA;
+          changeover_w(r2 * rsqrt_refined(r2), pmin(T.A[i[k]], ps.A[j]), P.kmode, wB, wA);
+          g *= wB;
+        }
+        cm[k] |= 1u << j;
+        n[0] = fma(g, dx, n[0]); n[1] = fma(g, dy, n[1]); n[2] = fma(g, dz, n[2]);
+      } else {
+        f[0] = fma(g, dx, f[0]); f[1] = fma(g, dy, f[1]); f[2] = fma(g, dz, f[2]);
+      }
+    }
+    T.afar[i[k]] = f[0]; T.afar[np + i[k]] = f[1]; T.afar[2 * np + i[k]] = f[2];
+    T.cmask[i[k]] = cm[k];
+    for (int c = 0; c < 3; ++c) acc[k][c] = f[c] + n[c];
+  }
+  __syncwarp();
 }
 
 // One TP (see tp_close_forces_k); returns its mask, the acceleration in (ax, ay, az).
@@ -567,6 +673,7 @@ __device__ unsigned char d_prep_slot[2 * TP_TAB];        // hf * TP_TAB + tab_in
 constexpr int TPB_WARPS = 12;
 constexpr int TP_WAIT_MAX = 500;  // naps of about 2 us
 constexpr int TPB_WPOS = TP_PRE * TP_TAB * 3;
+static_assert(sizeof(PlanetFx) <= 2 * TPB_WPOS * sizeof(double) && (2 * TPB_WPOS * sizeof(double)) % 16 == 0, "PlanetFx fits");
 constexpr size_t TPB_SMEM = (size_t)TPB_WARPS * (2 * TPB_WPOS + 2 * 16) * sizeof(double);
 
 // A warp of the BS pass is done; the last of all empties the BS list for the next substep (every
@@ -595,7 +702,7 @@ __device__ __noinline__ unsigned tp_bs_close(const TPSet &T, const DevParams &P,
 __global__ void __launch_bounds__(32 * TPB_WARPS, 1) k_tp_bs(Sim S, TPSet T, DevParams P, double tau, double h1,
                                                            double h2, double hcm_last) {
   constexpr int WPOS = TPB_WPOS;
-  extern __shared__ double tpb_smem[];  // per warp: planet positions of both attempts, then s_zt
+  extern __shared__ __align__(16) double tpb_smem[];  // per warp: planet positions of both attempts, then s_zt
   __shared__ PlanetSm s_ps[TPB_WARPS];  // per warp: the planets at the end of the substep, for the
   __shared__ double s_shc[TPB_WARPS][3];  // closing kicks, and the last Sun drift's shift
   const int lane = threadIdx.x & 31, half = lane >> 4, l16 = lane & 15, warp = threadIdx.x >> 5;
@@ -819,7 +926,8 @@ __global__ void __launch_bounds__(32 * TPB_WARPS, 1) k_tp_bs(Sim S, TPSet T, Dev
       act[k] = i < T.n && T.alive[i] && T.emask[i] == 0u && !T.fail[i];
       for (int q = 0; q < 3; ++q) x[k][q] = act[k] ? T.x[q * np + i] : 0.0;
     }
-    tp_close_forces_k<2>(T, P, s_ps[warp], S.n, ii, act, x, acc, cm);
+    // the warp's midpoint positions are free once it takes closing kicks
+    tp_close_forces_fx(T, P, s_ps[warp], *reinterpret_cast<PlanetFx *>(wpos0), S.n, ii, act, x, acc, cm);
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
       if (act[k])

@@ -219,3 +219,38 @@ def test_particles_meeting_a_planet_in_a_group_match_oracle():
     finally:
         genga.genga_free(h)
         o.close()
+
+
+@pytest.mark.parametrize("n_planets,n_tp,far", [(1, 1, 0.0), (1, 63, 0.0), (2, 64, 0.0), (3, 65, 300.0), (4, 127, 0.0), (5, 129, 1e4),
+                                                (17, 200, 300.0), (31, 64, 0.0), (32, 333, 0.0), (32, 333, 300.0)])
+def test_closing_kick_at_the_edges_of_its_groups(n_planets, n_tp, far):
+    """One step with every number of planets of the fixed-point closing kick's flush groups, particle
+    numbers around its 64 a warp, and a particle so far out that the grid does not resolve the close
+    pairs of its warp: the bounds of the one-step test above."""
+    rng = np.random.default_rng(n_planets * 1000 + n_tp)
+    d = ics.tp_disk(5, n_tp=max(n_tp, 8))
+    a = 0.5 * 1.15 ** np.arange(n_planets)
+    ph = rng.uniform(0, 2 * np.pi, n_planets)
+    d["x"] = np.stack([a * np.cos(ph), a * np.sin(ph), 0.01 * a * np.cos(3 * ph)], 1)
+    d["v"] = np.sqrt(d["G"] * d["m0"] / a)[:, None] * np.stack([-np.sin(ph), np.cos(ph), 0 * ph], 1)
+    d["m"], d["R"] = 10.0 ** rng.uniform(-8, -5, n_planets), np.full(n_planets, 1e-6)
+    d["x_tp"], d["v_tp"] = d["x_tp"][:n_tp].copy(), d["v_tp"][:n_tp].copy()
+    d["R_tp"] = np.full(n_tp, 1e-6)
+    for k in range(0, n_tp, 9):
+        d["x_tp"][k] = d["x"][k % n_planets] + rng.normal(0, 0.02, 3)
+        d["v_tp"][k] = d["v"][k % n_planets] + rng.normal(0, 3e-4, 3)
+    if far:
+        d["x_tp"][n_tp // 2] = [far, 0.3, -0.2]
+        d["v_tp"][n_tp // 2] = [0.0, np.sqrt(d["G"] * d["m0"] / far), 0.0]
+    h, o = _gpu(d, 2), _oracle(d, 2)
+    try:
+        genga.genga_step(h, 1)
+        o.step(1)
+        os_ = o.state()
+        e, live = _check(genga.genga_get_state_tp(h, n_tp), os_, _sensitivity(d, 2, 1), 1e-12, 10.0)
+        met = np.zeros(n_tp, bool)
+        met[[int(t) for t, _ in o.encounters(-1)]] = True
+        assert (e[~met[live]] <= 1e-13).all()
+    finally:
+        genga.genga_free(h)
+        o.close()
