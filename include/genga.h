@@ -336,13 +336,12 @@ int genga_phase_energy(int n, double G, double m0, const double *m, const int *a
  *   Unlike genga_phase_kick this call cannot return GENGA_ECAP, since the count stays on the
  *   device: when *ncand exceeds cap, only the first cap pairs were written, and the caller must
  *   compare *ncand with cap itself.
- * Only cudaMemsetAsync, kernel launches and a device-to-device copy are enqueued on stream. The
- * first call on a device looks up the scratch array's device address (cudaGetSymbolAddress) with
- * that device current; make that first call before any stream capture. The address is kept for the
- * life of the process: after a reset of the device (cudaDeviceReset) it is stale, so do not call
- * this entry point again in that process. All calls share the one array, which keeps the last
- * call's contents: calls that overlap on the GPU (different streams without ordering between them)
- * race on it. */
+ * Only kernel launches are enqueued on stream. The first call on a device looks up the scratch
+ * array's device address (cudaGetSymbolAddress) with that device current; make that first call
+ * before any stream capture. The address is kept for the life of the process: after a reset of the
+ * device (cudaDeviceReset) it is stale, so do not call this entry point again in that process. All
+ * calls share the one array, which keeps the last call's contents: calls that overlap on the GPU
+ * (different streams without ordering between them) race on it. */
 int genga_kick_noalloc(int n, double G, double pc, int kmode, int precise_div, const double *m,
                        const int *alive, const double *x, const double *rc, double *a, int *cand,
                        int cap, int *ncand, void *stream);

@@ -241,7 +241,7 @@ int first_kick(genga_ctx *c) {
     return GENGA_OK;
   }
   launch_kick(S, c->P, false, c->prm.precise_div != 0, st);
-  launch_fin(S, c->P, FIN_INIT, c->prm.precise_div != 0, 0.0, 0.0, nullptr, st);
+  launch_fin(S, c->P, FIN_INIT, c->prm.precise_div != 0, 0.0, 0.0, nullptr, 0, st);
   if (c->tpmode) {
     CK(cudaMemsetAsync(c->T.npairs, 0, sizeof(unsigned), st));
     CK(cudaMemsetAsync(c->T.bsnext, 0, (4 + 4 * TP_BS_MAXBLOCKS) * sizeof(unsigned), st));
@@ -311,7 +311,7 @@ void enqueue_step(genga_ctx *c, cudaStream_t st) {
   const TPSet &T = c->T;
   launch_rcrit(S, P, std::fabs(dt), 1, st);
   launch_kick(S, P, true, precise, st);  // runs only if the critical radii grew too much
-  launch_fin(S, P, FIN_OPEN, precise, 0.5 * c->w[0] * dt, 0.0, nullptr, st);
+  launch_fin(S, P, FIN_OPEN, precise, 0.5 * c->w[0] * dt, 0.0, nullptr, 0, st);
   for (int j = 0; j < c->nsub; ++j) {
     const double tau = c->w[j] * dt;
     const double hcm2 = j > 0 ? 0.5 * c->w[j - 1] * dt * inv_m0 : 0.0;
@@ -357,7 +357,7 @@ void enqueue_step(genga_ctx *c, cudaStream_t st) {
     launch_kick(S, P, inner, precise, st, inner);
     if (c->profiling) cudaEventRecordWithFlags(c->kev[2 * j + 1], st, cudaEventRecordExternal);
     const double h2 = (j + 1 < c->nsub) ? 0.5 * c->w[j + 1] * dt : 0.0;
-    launch_fin(S, P, inner ? FIN_CLOSE_ALL : FIN_CLOSE, precise, 0.5 * tau, h2, nullptr, st);
+    launch_fin(S, P, inner ? FIN_CLOSE_ALL : FIN_CLOSE, precise, 0.5 * tau, h2, nullptr, 0, st);
     if (tp) {  // join; the particles' BS and every particle's closing kick (after the last substep
                // with their last Sun drift, from the massive momentum before the closing kick)
       cudaStreamWaitEvent(st, c->ev_join, 0);
@@ -1279,7 +1279,7 @@ int genga_encounters(genga_ctx *c, int substep, int *pairs, int cap, int *n_pair
   if (substep < 0) substep = c->nsub - 1;
   if (substep >= c->nsub) return GENGA_EINVAL;
   cudaStream_t st = c->stream;
-  launch_bitmap_pairs(c->S.ebm + (size_t)substep * c->S.npad * c->S.W, c->S.npad, c->S.W, c->spairs,
+  launch_bitmap_pairs(c->S.ebm + (size_t)substep * c->S.npad * c->S.W, nullptr, c->S.npad, c->S.W, c->spairs,
                       (int)c->pair_cap, c->scount, st);
   CK(cudaGetLastError());
   int cnt = 0;
@@ -1494,15 +1494,13 @@ int genga_phase_kick(int n, double G, double pc, int kmode, int precise_div, con
   cudaStream_t st = (cudaStream_t)stream;
   genga_params prm; genga_default_params(&prm); prm.pc = pc; prm.kmode = kmode;
   DevParams P = make_params(G, 1.0, prm);
-  double *aout = mem.get<double>(3 * (size_t)S.npad);
   int *dcnt = mem.get<int>(1);
   int *tmp = mem.get<int>(2 * ((size_t)S.npad * (S.npad - 1) / 2 + 1));
   if (mem.err != cudaSuccess) { mem.release(); return GENGA_ENOMEM; }
   launch_soa_setup(S, P, m, alive, x, nullptr, rc, n, st);
   launch_kick(S, P, false, precise_div != 0, st);
-  launch_fin(S, P, FIN_INIT, precise_div != 0, 0.0, 0.0, aout, st);
-  soa_copy(a, n, aout, S.npad, n, st);
-  launch_bitmap_pairs(S.cbm, S.npad, S.W, tmp, S.npad * (S.npad - 1) / 2 + 1, dcnt, st);
+  launch_fin(S, P, FIN_INIT, precise_div != 0, 0.0, 0.0, a, n, st);
+  launch_bitmap_pairs(S.cbm, S.rowany, S.npad, S.W, tmp, S.npad * (S.npad - 1) / 2 + 1, dcnt, st);
   int cnt = 0;
   cudaMemcpyAsync(&cnt, dcnt, sizeof(int), cudaMemcpyDeviceToHost, st);
   cudaStreamSynchronize(st);
@@ -1541,7 +1539,7 @@ int genga_phase_encounters(int n, const int *alive, const double *x0, const doub
   soa_copy(S.v0, S.npad, v0, n, n, st);
   launch_pairs_to_bitmap(S, cand, ncand, st);
   launch_encounter(S, tau, S.ebm, st);
-  launch_bitmap_pairs(S.ebm, S.npad, S.W, tmp, S.npad * (S.npad - 1) / 2 + 1, dcnt, st);
+  launch_bitmap_pairs(S.ebm, nullptr, S.npad, S.W, tmp, S.npad * (S.npad - 1) / 2 + 1, dcnt, st);
   int cnt = 0;
   cudaMemcpyAsync(&cnt, dcnt, sizeof(int), cudaMemcpyDeviceToHost, st);
   cudaStreamSynchronize(st);

@@ -16,7 +16,7 @@ void launch_rcrit(const Sim &S, const DevParams &P, double tau_abs, int check_re
 void launch_kick(const Sim &S, const DevParams &P, bool full, bool precise, cudaStream_t st, bool force = false);
 // precise: which pair kernel wrote the partial sums
 void launch_fin(const Sim &S, const DevParams &P, FinMode mode, bool precise, double h1, double h2, double *aout,
-                cudaStream_t st);
+                int ald, cudaStream_t st);  // aout: accelerations [3][ald] of the S.n bodies, or null
 void launch_hc(const Sim &S, double hcm, cudaStream_t st);
 // the fixed-point pair kernel's chunks of partners per tile, partners per chunk
 void kick_split(int npad, int sms, int *chunks, int *chunk, int systems = 1);
@@ -32,7 +32,9 @@ void launch_encounter_group(const Sim &S, double tau, unsigned *ebm, cudaStream_
 void launch_kepler_phase(int n, double mu, double dt, int maxit, const int *alive, double *x, double *v,
                          int *fail, cudaStream_t st);
 void launch_pairs_to_bitmap(const Sim &S, const int *pairs, int npairs, cudaStream_t st);
-void launch_bitmap_pairs(const unsigned *bm, int npad, int W, int *out, int cap, int *count, cudaStream_t st);
+// rows: row-nonempty bits of the bitmap, or null
+void launch_bitmap_pairs(const unsigned *bm, const unsigned *rows, int npad, int W, int *out, int cap, int *count,
+                         cudaStream_t st);
 void launch_single_to_fail(const Sim &S, const int *single, cudaStream_t st);
 void launch_copy_edges(const Sim &S, const int *pairs, int npairs, cudaStream_t st);
 

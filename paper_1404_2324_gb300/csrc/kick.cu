@@ -294,14 +294,14 @@ __device__ __forceinline__ double near_term(const Sim &S, const DevParams &P, in
 //          kernel recorded before the velocities changed.
 //   OPEN : first kick of a full step with the new critical radii: a = stored far field + near
 //          pairs recomputed (KickA; KickB when there are none), or the full recompute's partials.
-//   INIT : the very first kick: store the far field (and a = far + near into aout if given).
+//   INIT : the very first kick: store the far field (and a = far + near into aout [3][ald] if given).
 // The near pairs of the tile's 32 bodies are gathered from the candidate lists (one coalesced pass
 // into shared memory), put in ascending partner order per body (each entry goes to its rank),
 // evaluated one per thread across the CTA and summed per body in partner order.
 // Also writes the per-tile momentum of the new velocities for the next Sun drift.
 // ---------------------------------------------------------------------------------------------
 template <int MODE>
-__global__ void __launch_bounds__(128) k_fin(Sim S, DevParams P, double h1, double h2, double *aout, int nslot) {
+__global__ void __launch_bounds__(128) k_fin(Sim S, DevParams P, double h1, double h2, double *aout, int ald, int nslot) {
   constexpr bool ALL = MODE == FIN_CLOSE_ALL;  // the pair kernel weighed every pair: no near pass
   const int B = blockIdx.x, c = blockIdx.y, wi = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int np = S.npad, i = B * 32 + lane;
@@ -372,7 +372,7 @@ __global__ void __launch_bounds__(128) k_fin(Sim S, DevParams P, double h1, doub
   if (MODE != FIN_OPEN && !ALL) S.afar[c * np + i] = a;
   for (int k = off[lane]; k < off[lane + 1]; ++k) a += contrib[k];
   if (overflow) a += near_accel(S, P, i, c);
-  if (aout) aout[c * np + i] = a;
+  if (aout && i < S.n) aout[(size_t)c * ald + i] = a;
   if (MODE == FIN_INIT) return;
   double v = v_old;
   if (alive) {
@@ -402,13 +402,13 @@ void launch_kick(const Sim &S, const DevParams &P, bool full, bool precise, cuda
 }
 
 void launch_fin(const Sim &S, const DevParams &P, FinMode mode, bool precise, double h1, double h2, double *aout,
-                cudaStream_t st) {
+                int ald, cudaStream_t st) {
   dim3 grid(S.nt, 3);
   const int nslot = precise ? 2 * S.nt : S.kch;  // partial-sum slots per tile of the pair kernel used
-  if (mode == FIN_CLOSE) k_fin<FIN_CLOSE><<<grid, 128, 0, st>>>(S, P, h1, h2, aout, nslot);
-  else if (mode == FIN_CLOSE_ALL) k_fin<FIN_CLOSE_ALL><<<grid, 128, 0, st>>>(S, P, h1, h2, aout, nslot);
-  else if (mode == FIN_OPEN) k_fin<FIN_OPEN><<<grid, 128, 0, st>>>(S, P, h1, h2, aout, nslot);
-  else k_fin<FIN_INIT><<<grid, 128, 0, st>>>(S, P, h1, h2, aout, nslot);
+  if (mode == FIN_CLOSE) k_fin<FIN_CLOSE><<<grid, 128, 0, st>>>(S, P, h1, h2, aout, ald, nslot);
+  else if (mode == FIN_CLOSE_ALL) k_fin<FIN_CLOSE_ALL><<<grid, 128, 0, st>>>(S, P, h1, h2, aout, ald, nslot);
+  else if (mode == FIN_OPEN) k_fin<FIN_OPEN><<<grid, 128, 0, st>>>(S, P, h1, h2, aout, ald, nslot);
+  else k_fin<FIN_INIT><<<grid, 128, 0, st>>>(S, P, h1, h2, aout, ald, nslot);
 }
 
 // Second Sun drift after the last substep: x += hcm * P, P the momentum before the closing kick.

@@ -383,8 +383,10 @@ __global__ void k_pairs_to_bitmap(Sim S, const int *pairs, int npairs) {
   if (kj < CCAP) S.clist[j * CCAP + kj] = i;
 }
 
-// Pairs (i < j) of a bitmap, ascending, into out[2*cap]; *count receives the total.
-__global__ void __launch_bounds__(1024) k_bitmap_pairs(const unsigned *bm, int npad, int W, int *out, int cap, int *count) {
+// Pairs (i < j) of a bitmap, ascending, into out[2*cap]; *count receives the total. Rows whose bit in
+// rows (if given) is clear are empty and not read.
+__global__ void __launch_bounds__(1024) k_bitmap_pairs(const unsigned *bm, const unsigned *rows, int npad, int W, int *out,
+                                                       int cap, int *count) {
   __shared__ int wtot[32];
   __shared__ int s_base;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -393,14 +395,12 @@ __global__ void __launch_bounds__(1024) k_bitmap_pairs(const unsigned *bm, int n
   for (int r0 = 0; r0 < npad; r0 += 1024) {
     const int i = r0 + tid;
     int c = 0;
-    if (i < npad) {
-      for (int w = 0; w < W; ++w) {
-        unsigned bits = bm[(size_t)i * W + w];
-        const int lo = w * 32;
-        if (lo + 31 <= i) bits = 0u;
-        else if (lo <= i) bits &= (i - lo + 1 >= 32) ? 0u : (0xffffffffu << (i - lo + 1));
-        c += __popc(bits);
-      }
+    const bool any = i < npad && (!rows || ((rows[i >> 5] >> (i & 31)) & 1u));
+    if (any) {  // the upper triangle: words from the body's own on
+      unsigned own = bm[(size_t)i * W + (i >> 5)] & ((i & 31) == 31 ? 0u : 0xffffffffu << ((i & 31) + 1));
+      c = __popc(own);
+#pragma unroll 8
+      for (int w = (i >> 5) + 1; w < W; ++w) c += __popc(bm[(size_t)i * W + w]);
     }
     int incl = c;
 #pragma unroll
@@ -421,12 +421,13 @@ __global__ void __launch_bounds__(1024) k_bitmap_pairs(const unsigned *bm, int n
     }
     __syncthreads();
     int pos = s_base + wtot[wid] + incl - c;
-    if (i < npad && c) {
-      for (int w = 0; w < W; ++w) {
+    if (c) {
+      int left = c;
+      for (int w = i >> 5; w < W && left; ++w) {
         unsigned bits = bm[(size_t)i * W + w];
         const int lo = w * 32;
-        if (lo + 31 <= i) bits = 0u;
-        else if (lo <= i) bits &= (i - lo + 1 >= 32) ? 0u : (0xffffffffu << (i - lo + 1));
+        if (lo <= i) bits &= (i - lo + 1 >= 32) ? 0u : (0xffffffffu << (i - lo + 1));
+        left -= __popc(bits);
         while (bits) {
           const int b = __ffs(bits) - 1;
           bits &= bits - 1;
@@ -475,8 +476,9 @@ void launch_kepler_phase(int n, double mu, double dt, int maxit, const int *aliv
 void launch_pairs_to_bitmap(const Sim &S, const int *pairs, int npairs, cudaStream_t st) {
   if (npairs > 0) k_pairs_to_bitmap<<<(npairs + 127) / 128, 128, 0, st>>>(S, pairs, npairs);
 }
-void launch_bitmap_pairs(const unsigned *bm, int npad, int W, int *out, int cap, int *count, cudaStream_t st) {
-  k_bitmap_pairs<<<1, 1024, 0, st>>>(bm, npad, W, out, cap, count);
+void launch_bitmap_pairs(const unsigned *bm, const unsigned *rows, int npad, int W, int *out, int cap, int *count,
+                         cudaStream_t st) {
+  k_bitmap_pairs<<<1, 1024, 0, st>>>(bm, rows, npad, W, out, cap, count);
 }
 void launch_single_to_fail(const Sim &S, const int *single, cudaStream_t st) {
   k_single_to_fail<<<(S.n + 127) / 128, 128, 0, st>>>(S, single);

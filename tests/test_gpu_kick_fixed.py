@@ -87,3 +87,22 @@ def test_fixed_point_kick_passes_on_numbers_it_cannot_hold():
         np.testing.assert_array_equal(np.isfinite(a), np.isfinite(b), err_msg=what)
         f = np.isfinite(a) & np.isfinite(b)
         np.testing.assert_allclose(a[f], b[f], rtol=0, atol=1e-13 * np.abs(b[f]).max() if f.any() else 0, err_msg=what)
+
+
+@pytest.mark.parametrize("precise", [0, 1])
+def test_kick_without_allocation_clears_its_scratch_between_sizes(precise):
+    """Calls of rising and falling size, one after the other on the one scratch array: each gives the
+    allocating kick's numbers and candidates, so nothing of the call before is left."""
+    import torch
+
+    for n in (1024, 1, 33, 1000, 31, 32, 65, 1023, 2):
+        G, m, alive, x, rc = _case("ghosts" if n % 2 else "disk", n)
+        cap = max(1, n * (n - 1) // 2)
+        want, pairs = _run(G, m, alive, x, rc, precise)
+        a, cand, cnt = dev(np.zeros((3, n))), dev(np.zeros(2 * cap, np.int32)), dev(np.zeros(1, np.int32))
+        genga.genga_kick_noalloc(n, G, 3.0, 0, precise, dev(m), dev(alive), soa(x), dev(rc), a, cand, cap, cnt)
+        torch.cuda.synchronize()
+        assert int(cnt.item()) == len(pairs), n
+        np.testing.assert_array_equal(cand.cpu().numpy()[: 2 * len(pairs)].reshape(-1, 2), pairs, err_msg=str(n))
+        live = alive == 1
+        np.testing.assert_array_equal(aos(a)[live], want[live], err_msg=str(n))
