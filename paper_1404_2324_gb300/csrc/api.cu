@@ -61,7 +61,7 @@ bool alloc_sim(Sim &S, DevMem &mem, int n, int nsub) {
   S.afar = mem.get<double>(3 * np);
   kick_split(S.npad, num_sms(), &S.kch, &S.kchunk);
   S.part = mem.get<double>(nt * std::max(2 * nt, (size_t)S.kch) * 96);
-  S.pkick = mem.get<double>(nt * 3); S.pfin = mem.get<double>(nt * 3);
+  S.pkick = mem.get<double>(nt * 3); S.pfin = mem.get<double>(nt * FIN_PER_TILE * 3);
   S.cbm = mem.get<unsigned>(np * W); S.rowany = mem.get<unsigned>(W);
   S.ccnt = mem.get<int>(np); S.clist = mem.get<int>(np * CCAP);
   S.ebm = mem.get<unsigned>((size_t)nsub * np * W);

@@ -22,6 +22,7 @@ constexpr int BS_HEAVY = 2;      // batched: groups with a member that needed >=
 constexpr int BS_SMALL = 4;      // batched: groups of 3 .. BS_SMALL members run on 128-thread CTAs
 constexpr int BS_SEQCAP = 256;   // accepted BS substeps one group may record per substep
 constexpr int NCOUNTERS = 8;
+constexpr int FIN_PER_TILE = 4;   // CTAs of the kick's finalisation per 32 bodies
 constexpr int CCAP = 32;          // candidate-list slots per body (more: the bitmap row is scanned)
 constexpr double PARK = 1.0e8;    // ghosts are parked this far out (AU) so no pair ever sees them
 
@@ -81,7 +82,7 @@ struct Sim {
   u64 *T, *rcsq;                 // [npad]; bits of (pc rc)^2 and rc^2
   double *afar;                  // [3 npad] far-field accelerations of the last kick
   double *part;                  // [nt * max(2 nt, kch) * 3 * 32] kick partial sums
-  double *pkick, *pfin;          // [nt * 3] per-tile momentum partials
+  double *pkick, *pfin;          // momentum partials [nt * 3] per tile, [nt * FIN_PER_TILE * 3] per k_fin CTA
   unsigned *cbm, *rowany;        // candidate bitmap [npad * W], row-nonempty bits [W]
   int *ccnt, *clist;             // per-body candidate count [npad] and partners [npad * CCAP]
   unsigned *ebm;                 // encounter bitmaps [nsub * npad * W] (upper triangle)
@@ -602,6 +603,36 @@ __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
+}
+
+// The warp's sums of three numbers at once: lanes 0-7 receive that of x, 8-15 of y, 16-31 of z. Six FP64
+// additions where three butterflies take fifteen.
+__device__ __forceinline__ double warp_sum3(double x, double y, double z) {
+  const int lane = threadIdx.x & 31;
+  const bool up = lane & 16, odd = lane & 8;
+  const double p = (up ? z : x) + __shfl_xor_sync(0xffffffffu, up ? x : z, 16);
+  const double q = y + __shfl_xor_sync(0xffffffffu, y, 16);
+  double r = (!up && odd ? q : p) + __shfl_xor_sync(0xffffffffu, !up && !odd ? q : p, 8);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+  return r;
+}
+
+// The Sun drift's shift, h1 times the momentum after the last kick plus h2 times the one before its
+// velocities changed (h2 = 0: none), by a whole warp; every lane receives it.
+__device__ __forceinline__ void sun_shift(const Sim &S, double h1, double h2, double (&sh)[3]) {
+  const int lane = threadIdx.x & 31;
+  double a[3] = {0.0, 0.0, 0.0};
+  for (int t = lane; t < FIN_PER_TILE * S.nt; t += 32)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) a[c] = fma(h1, S.pfin[t * 3 + c], a[c]);
+  if (h2 != 0.0)
+    for (int t = lane; t < S.nt; t += 32)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) a[c] = fma(h2, S.pkick[t * 3 + c], a[c]);
+  const double s = warp_sum3(a[0], a[1], a[2]);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) sh[c] = __shfl_sync(0xffffffffu, s, 8 * c);
 }
 
 }  // namespace genga

@@ -246,47 +246,17 @@ static void launch_kick_fx(const Sim &S, const DevParams &P, int force, cudaStre
   else k_kick_fx<FULL, 1><<<grid, 32 * KX_WARPS, 0, st>>>(S, P, force);
 }
 
-// Component c of the near-pair acceleration of body i: the precheck candidates recorded in row i
-// of the bitmap, with the changeover weight of the current critical radii (IEEE sqrt/division).
-__device__ double near_accel(const Sim &S, const DevParams &P, int i, int c) {
-  const int np = S.npad;
-  const unsigned *row = S.cbm + (size_t)i * S.W;
-  const double xi = S.x[i], yi = S.x[np + i], zi = S.x[2 * np + i];
-  const u64 Qi = S.rcsq[i];
-  const double Ai = S.A[i];
-  double acc = 0.0;
-  for (int w = 0; w < S.W; ++w) {
-    unsigned bits = row[w];
-    while (bits) {
-      const int b = __ffs(bits) - 1;
-      bits &= bits - 1;
-      const int j = w * 32 + b;
-      const double dx = S.x[j] - xi, dy = S.x[np + j] - yi, dz = S.x[2 * np + j] - zi;
-      const double r2 = __fma_rn(dz, dz, __fma_rn(dy, dy, __dmul_rn(dx, dx)));
-      const double r = sqrt(r2);
-      double wB = 1.0, wA;
-      if (dbits(r2) < umax64(Qi, S.rcsq[j])) changeover_w(r, pmin(Ai, S.A[j]), P.kmode, wB, wA);
-      const double f = S.gm[j] * wB / (r2 * r);
-      acc = fma(f, c == 0 ? dx : (c == 1 ? dy : dz), acc);
-    }
-  }
-  return acc;
-}
-
-// Component c of the near-pair pull of partner j on body i with the current critical radii
+// The near-pair pull of partner j on body i, per unit separation, with the current critical radii
 // (refined inverse square root; the changeover weight as in the kick).
-__device__ __forceinline__ double near_term(const Sim &S, const DevParams &P, int i, int j, int c) {
-  const int np = S.npad;
-  const double dx = S.x[j] - S.x[i], dy = S.x[np + j] - S.x[np + i], dz = S.x[2 * np + j] - S.x[2 * np + i];
-  const double r2 = __fma_rn(dz, dz, __fma_rn(dy, dy, __dmul_rn(dx, dx)));
+__device__ __forceinline__ double near_factor(const Sim &S, const DevParams &P, u64 Qi, double Ai, int j, double r2) {
   const double yr = rsqrt_refined(r2);
   double wB = 1.0, wA;
-  if (dbits(r2) < umax64(S.rcsq[i], S.rcsq[j])) changeover_w(r2 * yr, pmin(S.A[i], S.A[j]), P.kmode, wB, wA);
-  return S.gm[j] * wB * (yr * yr * yr) * (c == 0 ? dx : (c == 1 ? dy : dz));
+  if (dbits(r2) < umax64(Qi, S.rcsq[j])) changeover_w(r2 * yr, pmin(Ai, S.A[j]), P.kmode, wB, wA);
+  return S.gm[j] * wB * (yr * yr * yr);
 }
 
 // ---------------------------------------------------------------------------------------------
-// Finalisation, one CTA per (body tile, component):
+// Finalisation, one warp per body, FIN_BODIES bodies per CTA:
 //   CLOSE: a = sum of the pair partials (far field, stored for reuse) + near pairs;
 //          v += h1 a (+ h2 a for the next substep's opening kick). The second Sun drift of the
 //          substep (which the kick does not see: it shifts every body alike) is applied by the
@@ -295,93 +265,91 @@ __device__ __forceinline__ double near_term(const Sim &S, const DevParams &P, in
 //   OPEN : first kick of a full step with the new critical radii: a = stored far field + near
 //          pairs recomputed (KickA; KickB when there are none), or the full recompute's partials.
 //   INIT : the very first kick: store the far field (and a = far + near into aout [3][ald] if given).
-// The near pairs of the tile's 32 bodies are gathered from the candidate lists (one coalesced pass
-// into shared memory), put in ascending partner order per body (each entry goes to its rank),
-// evaluated one per thread across the CTA and summed per body in partner order.
-// Also writes the per-tile momentum of the new velocities for the next Sun drift.
+// Eight lanes a component sum the pair partials. The near partners are read from the body's row of the
+// candidate bitmap, in ascending order, and evaluated one per lane, once for all three components; the
+// sums have a fixed order. Also writes the CTA's momentum of the new velocities for the next Sun drift.
+//
+// Bound by latency (launch, the chain row -> positions -> FP64 terms -> sums) and, with wide critical
+// radii, by the near pairs' FP64 issue. Measured against one CTA per tile and component, which gathered
+// and ranked the candidate lists of 32 bodies and left rows of more than 32 partners to one lane each:
+// 1024 bodies with wide radii 58 -> 9.7 us (opening 39 -> 7.4), 2048 bodies 12.9 -> 9, 32 bodies
+// 10.0 -> 7.4.
 // ---------------------------------------------------------------------------------------------
+constexpr int FIN_BODIES = 32 / FIN_PER_TILE;
+
 template <int MODE>
-__global__ void __launch_bounds__(128) k_fin(Sim S, DevParams P, double h1, double h2, double *aout, int ald, int nslot) {
+__global__ void __launch_bounds__(32 * FIN_BODIES) k_fin(Sim S, DevParams P, double h1, double h2, double *aout, int ald,
+                                                         int nslot) {
   constexpr bool ALL = MODE == FIN_CLOSE_ALL;  // the pair kernel weighed every pair: no near pass
-  const int B = blockIdx.x, c = blockIdx.y, wi = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int np = S.npad, i = B * 32 + lane;
-  __shared__ double red[4][32];
-  __shared__ int ent[32 * CCAP], raw[32 * CCAP];
-  __shared__ double contrib[32 * CCAP];
-  __shared__ int off[33], s_cnt[32];
-  const bool use_part = (MODE != FIN_OPEN) || (S.flags[0] != 0);
-  const bool full_open = (MODE == FIN_OPEN) && (S.flags[0] != 0);
-  // the loads of the final update first (warp 0), so that their latency passes under the sums
-  double a_far = 0.0, v_old = 0.0, m_i = 0.0;
-  bool alive = false;
-  if (wi == 0) {
-    if (!use_part) a_far = S.afar[c * np + i];
-    if (MODE != FIN_INIT) { v_old = S.v[c * np + i]; m_i = S.m[i]; alive = S.alive[i] != 0; }
-  }
-  // this tile's candidate partners: counts and offsets (warp 0), then the lists (all threads)
-  bool overflow = false;
-  if (wi == 0) {
-    const bool any = !ALL && !full_open && ((S.rowany[i >> 5] >> (i & 31)) & 1u);
-    int cnt = any ? S.ccnt[i] : 0;
-    overflow = cnt > CCAP;
-    if (overflow) cnt = 0;
-    int incl = cnt;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int t = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += t;
+  __shared__ unsigned short s_j[FIN_BODIES][1024];  // partners found in 32 words of the row
+  __shared__ double s_pm[3][FIN_BODIES];
+  const int wi = threadIdx.x >> 5, lane = threadIdx.x & 31, np = S.npad;
+  const int i = blockIdx.x * FIN_BODIES + wi, c = lane >> 3, sl = lane & 7;
+  const bool comp = c < 3, use_part = (MODE != FIN_OPEN) || (S.flags[0] != 0);
+  const bool near = !ALL && !(MODE == FIN_OPEN && use_part);
+  // the loads of the final update first, so that their latency passes under the sums
+  const double a_far = (!use_part && comp) ? S.afar[c * np + i] : 0.0;
+  const double v_old = (MODE != FIN_INIT && comp) ? S.v[c * np + i] : 0.0;
+  const double m_i = S.m[i];
+  const bool alive = S.alive[i] != 0;
+  double a = a_far;
+  if (use_part) {
+    double a0 = 0.0, a1 = 0.0;
+    if (comp) {
+      const double *p = S.part + (size_t)(i >> 5) * nslot * 96 + c * 32 + (i & 31);
+      int s = sl;
+#pragma unroll 4
+      for (; s + 8 < nslot; s += 16) { a0 += p[(size_t)s * 96]; a1 += p[(size_t)(s + 8) * 96]; }
+      if (s < nslot) a0 += p[(size_t)s * 96];
     }
-    off[lane + 1] = incl;
-    s_cnt[lane] = cnt;
-    if (lane == 0) off[0] = 0;
+    a = a0 + a1;
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
   }
-  if (use_part) {  // far-field partial sums: each warp a quarter of the slots, two chains of alternate slots
-    const int s0 = wi * nslot / 4, s1 = (wi + 1) * nslot / 4;
-    const double *base = S.part + (size_t)B * nslot * 96 + c * 32 + lane;
-    double acc0 = 0.0, acc1 = 0.0;
-    int s = s0;
-    for (; s + 1 < s1; s += 2) { acc0 += base[(size_t)s * 96]; acc1 += base[(size_t)(s + 1) * 96]; }
-    if (s < s1) acc0 += base[(size_t)s * 96];
-    red[wi][lane] = acc0 + acc1;
+  if (MODE != FIN_OPEN && !ALL && comp && sl == 0) S.afar[c * np + i] = a;
+  if (near && ((S.rowany[i >> 5] >> (i & 31)) & 1u)) {
+    const double xi = S.x[i], yi = S.x[np + i], zi = S.x[2 * np + i], Ai = S.A[i];
+    const u64 Qi = S.rcsq[i];
+    double nx = 0.0, ny = 0.0, nz = 0.0;
+    for (int w0 = 0; w0 < S.W; w0 += 32) {
+      unsigned bits = w0 + lane < S.W ? S.cbm[(size_t)i * S.W + w0 + lane] : 0u;
+      const int mine = __popc(bits);
+      int incl = mine;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+      }
+      const int cnt = __shfl_sync(0xffffffffu, incl, 31);
+      for (int k = incl - mine; bits; ++k, bits &= bits - 1) s_j[wi][k] = (unsigned short)((w0 + lane) * 32 + __ffs(bits) - 1);
+      __syncwarp();
+      for (int k = lane; k < cnt; k += 32) {
+        const int j = s_j[wi][k];
+        const double dx = S.x[j] - xi, dy = S.x[np + j] - yi, dz = S.x[2 * np + j] - zi;
+        const double f = near_factor(S, P, Qi, Ai, j, r2_exact(dx, dy, dz));
+        nx = fma(f, dx, nx); ny = fma(f, dy, ny); nz = fma(f, dz, nz);
+      }
+      __syncwarp();
+    }
+    a += warp_sum3(nx, ny, nz);
   }
-  __syncthreads();
-  const int M = off[32];
-  for (int e = threadIdx.x; e < 32 * CCAP; e += 128) {
-    const int b = e / CCAP, k = e % CCAP;
-    if (k < s_cnt[b]) raw[off[b] + k] = S.clist[(B * 32 + b) * CCAP + k];
+  if (aout && i < S.n && comp && sl == 0) aout[(size_t)c * ald + i] = a;
+  if (MODE == FIN_INIT) return;
+  if (comp && sl == 0) {
+    double v = v_old;
+    if (alive) {
+      v = fma(h1, a, v);
+      if (h2 != 0.0) v = fma(h2, a, v);
+      S.v[c * np + i] = v;
+    }
+    s_pm[c][wi] = m_i * v;
   }
-  __syncthreads();
-  auto owner = [&](int k) {  // the last body whose offset is <= k
-    int b = 0;
-    for (int s = 16; s > 0; s >>= 1)
-      if (b + s <= 32 && off[b + s] <= k) b += s;
-    return b;
-  };
-  for (int k = threadIdx.x; k < M; k += 128) {  // ascending partner order: each entry to its rank
-    const int b = owner(k), o = off[b], n = off[b + 1] - o;
-    const int j = raw[k];
-    int r = 0;
-    for (int q = 0; q < n; ++q) r += raw[o + q] < j;
-    ent[o + r] = j;
-  }
-  __syncthreads();
-  for (int k = threadIdx.x; k < M; k += 128) contrib[k] = near_term(S, P, B * 32 + owner(k), ent[k], c);
   __syncthreads();
   if (wi != 0) return;
-  double a = use_part ? (red[0][lane] + red[1][lane]) + (red[2][lane] + red[3][lane]) : a_far;
-  if (MODE != FIN_OPEN && !ALL) S.afar[c * np + i] = a;
-  for (int k = off[lane]; k < off[lane + 1]; ++k) a += contrib[k];
-  if (overflow) a += near_accel(S, P, i, c);
-  if (aout && i < S.n) aout[(size_t)c * ald + i] = a;
-  if (MODE == FIN_INIT) return;
-  double v = v_old;
-  if (alive) {
-    v = fma(h1, a, v);
-    if (h2 != 0.0) v = fma(h2, a, v);
-    S.v[c * np + i] = v;
-  }
-  const double pm = warp_sum(m_i * v);
-  if (lane == 0) S.pfin[B * 3 + c] = pm;
+  double pm = comp ? s_pm[c][sl] : 0.0;
+#pragma unroll
+  for (int o = FIN_BODIES / 2; o > 0; o >>= 1) pm += __shfl_xor_sync(0xffffffffu, pm, o);
+  if (comp && sl == 0) S.pfin[blockIdx.x * 3 + c] = pm;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -403,25 +371,24 @@ void launch_kick(const Sim &S, const DevParams &P, bool full, bool precise, cuda
 
 void launch_fin(const Sim &S, const DevParams &P, FinMode mode, bool precise, double h1, double h2, double *aout,
                 int ald, cudaStream_t st) {
-  dim3 grid(S.nt, 3);
+  const int grid = S.nt * FIN_PER_TILE, block = 32 * FIN_BODIES;
   const int nslot = precise ? 2 * S.nt : S.kch;  // partial-sum slots per tile of the pair kernel used
-  if (mode == FIN_CLOSE) k_fin<FIN_CLOSE><<<grid, 128, 0, st>>>(S, P, h1, h2, aout, ald, nslot);
-  else if (mode == FIN_CLOSE_ALL) k_fin<FIN_CLOSE_ALL><<<grid, 128, 0, st>>>(S, P, h1, h2, aout, ald, nslot);
-  else if (mode == FIN_OPEN) k_fin<FIN_OPEN><<<grid, 128, 0, st>>>(S, P, h1, h2, aout, ald, nslot);
-  else k_fin<FIN_INIT><<<grid, 128, 0, st>>>(S, P, h1, h2, aout, ald, nslot);
+  if (mode == FIN_CLOSE) k_fin<FIN_CLOSE><<<grid, block, 0, st>>>(S, P, h1, h2, aout, ald, nslot);
+  else if (mode == FIN_CLOSE_ALL) k_fin<FIN_CLOSE_ALL><<<grid, block, 0, st>>>(S, P, h1, h2, aout, ald, nslot);
+  else if (mode == FIN_OPEN) k_fin<FIN_OPEN><<<grid, block, 0, st>>>(S, P, h1, h2, aout, ald, nslot);
+  else k_fin<FIN_INIT><<<grid, block, 0, st>>>(S, P, h1, h2, aout, ald, nslot);
 }
 
 // Second Sun drift after the last substep: x += hcm * P, P the momentum before the closing kick.
 __global__ void k_hc(Sim S, double hcm) {
   const int lane = threadIdx.x & 31;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  double p[3];
+  double p[3] = {0.0, 0.0, 0.0};
+  for (int t = lane; t < S.nt; t += 32)
+    for (int c = 0; c < 3; ++c) p[c] += S.pkick[t * 3 + c];
+  const double ps = warp_sum3(p[0], p[1], p[2]);
 #pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    double a = 0.0;
-    for (int t = lane; t < S.nt; t += 32) a += S.pkick[t * 3 + c];
-    p[c] = warp_sum(a);
-  }
+  for (int c = 0; c < 3; ++c) p[c] = __shfl_sync(0xffffffffu, ps, 8 * c);
   if (i >= S.npad || !S.alive[i]) return;
 #pragma unroll
   for (int c = 0; c < 3; ++c) S.x[c * S.npad + i] = fma(hcm, p[c], S.x[c * S.npad + i]);

@@ -36,7 +36,7 @@ constexpr size_t O_AFAR = O_RCSQ + align256(NA_NMAX * sizeof(u64));
 constexpr size_t O_PART = O_AFAR + align256(3 * NA_NMAX * sizeof(double));
 constexpr size_t O_PKICK = O_PART + align256((size_t)NA_NT * NA_NT * 2 * 96 * sizeof(double));
 constexpr size_t O_PFIN = O_PKICK + align256(NA_NT * 3 * sizeof(double));
-constexpr size_t O_CBM = O_PFIN + align256(NA_NT * 3 * sizeof(double));
+constexpr size_t O_CBM = O_PFIN + align256(NA_NT * FIN_PER_TILE * 3 * sizeof(double));
 constexpr size_t O_ROWANY = O_CBM + align256((size_t)NA_NMAX * NA_W * sizeof(unsigned));
 constexpr size_t O_CCNT = O_ROWANY + align256(NA_W * sizeof(unsigned));
 constexpr size_t O_CLIST = O_CCNT + align256(NA_NMAX * sizeof(int));

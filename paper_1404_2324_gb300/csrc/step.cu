@@ -13,23 +13,13 @@ namespace genga {
 __global__ void __launch_bounds__(32) k_drift(Sim S, DevParams P, double tau, double hcm1, double hcm2, int substep) {
   const int lane = threadIdx.x;
   const int i = blockIdx.x * 32 + lane;
-  const int np = S.npad, nt = S.nt;
+  const int np = S.npad;
   if (i == 0) {
     if (substep == 0) { S.flags[0] = 0; S.flags[3] = 0; }  // the opening kick of this step has consumed the flags
     S.flags[2] = substep;              // for the collision reports of this substep's BS
   }
   double shift[3];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    double a = 0.0, b = 0.0;
-    for (int t = lane; t < nt; t += 32) {
-      a += S.pfin[t * 3 + c];
-      if (hcm2 != 0.0) b += S.pkick[t * 3 + c];
-    }
-    a = warp_sum(a);
-    shift[c] = hcm1 * a;
-    if (hcm2 != 0.0) shift[c] = fma(hcm2, warp_sum(b), shift[c]);
-  }
+  sun_shift(S, hcm1, hcm2, shift);
   if (!S.alive[i]) return;
   double x = S.x[i] + shift[0], y = S.x[np + i] + shift[1], z = S.x[2 * np + i] + shift[2];
   double vx = S.v[i], vy = S.v[np + i], vz = S.v[2 * np + i];

@@ -309,19 +309,9 @@ __global__ void __launch_bounds__(128) k_tp_kick(Sim S, TPSet T, DevParams P) {
 __global__ void k_tp_drift(Sim S, TPSet T, DevParams P, double tau, double hcm1, double hcm2) {
   __shared__ double sh[3];
   if (threadIdx.x < 32) {
-    const int lane = threadIdx.x;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      double a = 0.0, b = 0.0;
-      for (int t = lane; t < S.nt; t += 32) {
-        a += S.pfin[t * 3 + c];
-        if (hcm2 != 0.0) b += S.pkick[t * 3 + c];
-      }
-      a = warp_sum(a);
-      double v = hcm1 * a;
-      if (hcm2 != 0.0) v = fma(hcm2, warp_sum(b), v);
-      if (lane == 0) sh[c] = v;
-    }
+    double v[3];
+    sun_shift(S, hcm1, hcm2, v);
+    if (threadIdx.x == 0) { sh[0] = v[0]; sh[1] = v[1]; sh[2] = v[2]; }
   }
   __syncthreads();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -356,14 +346,9 @@ __global__ void __launch_bounds__(128) k_tp_open_drift(Sim S, TPSet T, DevParams
   __shared__ PlanetSm ps;
   __shared__ double sh[3];
   if (threadIdx.x < 32) {
-    const int lane = threadIdx.x;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      double a = 0.0;
-      for (int t = lane; t < S.nt; t += 32) a += S.pfin[t * 3 + c];
-      a = warp_sum(a);
-      if (lane == 0) sh[c] = hcm1 * a;
-    }
+    double v[3];
+    sun_shift(S, hcm1, 0.0, v);
+    if (threadIdx.x == 0) { sh[0] = v[0]; sh[1] = v[1]; sh[2] = v[2]; }
   }
   load_planets(S, ps);
   const int i = blockIdx.x * blockDim.x + threadIdx.x;

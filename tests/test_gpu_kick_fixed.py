@@ -106,3 +106,23 @@ def test_kick_without_allocation_clears_its_scratch_between_sizes(precise):
         np.testing.assert_array_equal(cand.cpu().numpy()[: 2 * len(pairs)].reshape(-1, 2), pairs, err_msg=str(n))
         live = alive == 1
         np.testing.assert_array_equal(aos(a)[live], want[live], err_msg=str(n))
+
+
+@pytest.mark.parametrize("n", [40, 300, 1025])
+@pytest.mark.parametrize("precise", [0, 1])
+def test_rows_of_many_near_partners_are_summed_in_full(n, precise):
+    """Critical radii so wide that a body has far more than 32 near partners, on both sides of the
+    changeover. A near term carries about 20 roundings, counted in the bound's constant."""
+    G, m, alive, x, rc = _case("ghosts", n)
+    rc = np.where(alive == 1, 0.6, 0.0)
+    p = O.params(G=G, m0=1.0, dt=6.0)
+    a, cand = _run(G, m, alive, x, rc, precise)
+    want = O.accel_B(p, m, alive, x, rc)
+    np.testing.assert_array_equal(cand, np.asarray(O.precheck(p, alive, x, rc)).reshape(-1, 2))
+    live = alive == 1
+    r = np.linalg.norm(x[None] - x[:, None], axis=-1)
+    np.fill_diagonal(r, np.inf)
+    t = G * np.where(live, m, 0.0)[None] / r ** 2
+    assert n < 300 or np.bincount(cand.ravel()).max() > 40
+    err = np.linalg.norm(a - want, axis=1)
+    assert np.all(err[live] <= (2.0 ** -53 * (1.2 * n + 100) * t.sum(1))[live]), np.max(err / t.sum(1))
