@@ -6,10 +6,9 @@
 // has an SM of its own. After every second evaluation the CTAs meet at a cluster barrier; level Lc
 // is then complete in CTA Lc - 1, every CTA reads its T_{Lc,1} from that CTA's shared memory
 // (distributed shared memory), extends its own copy of the Neville tableau and tests level Lc, with
-// the same arithmetic and order in every CTA. Groups of more than 8 members evaluate each pair
-// once (Newton's third law), so that up to 15 members take one FP64 round per SM sub-partition per
-// force evaluation. All CTAs therefore take the same decision
-// and follow the same control flow: every cluster barrier is reached by all 8 CTAs the same number
+// the same arithmetic and order in every CTA. Each pair is evaluated once (Newton's third law); of
+// large groups only the pairs that may be inside their critical radius. All CTAs therefore take the
+// same decision and follow the same control flow: every cluster barrier is reached by all 8 CTAs the same number
 // of times. Level results are double-buffered by attempt parity. Cluster k takes the k-th entry of
 // the large-group list that the grouping kernel writes.
 #include <cooperative_groups.h>
@@ -23,9 +22,8 @@ namespace genga {
 
 constexpr int CL_SIZE = BS_LEVELS;  // CTAs per cluster, one per level
 constexpr int CL_THREADS = 256;
-constexpr int CL_TPS = CL_THREADS / BS_GMAX;  // lanes per member (8)
+constexpr int CL_TPS = CL_THREADS / BS_GMAX;  // lanes per member that list pairs (8)
 constexpr int CL_PAIRS = BS_GMAX * (BS_GMAX - 1) / 2;
-constexpr int CL_ITEMS = BS_GMAX + CL_PAIRS;  // a force evaluation's terms: one per member, one per pair
 // the first level whose convergence is tested: groups of five or more members converge at level 5
 // or later in practice, and a level below it that converges is still found (its row is kept), at
 // the cost of the evaluations up to this level
@@ -41,9 +39,12 @@ struct BsClShared {
   double y[BS_GMAX][6], yn[BS_GMAX][6];
   double isc[BS_GMAX][2];                // 1/|x|, 1/|v| at the start of the attempt
   double pos[2][BS_GMAX][3];             // chain positions, double-buffered by evaluation
-  double term[CL_ITEMS][3];              // this evaluation's terms: central pulls, then pair factors
-  double acc[BS_GMAX][3];                // this evaluation's accelerations
-  unsigned char pa[CL_PAIRS], pb[CL_PAIRS];  // pair k = (pa[k], pb[k]), pa < pb, row by row
+  float fp[2][BS_GMAX][3];               // the same in single precision
+  double term[BS_GMAX][BS_GMAX][3];      // this evaluation's factors of partner [j] on member [i] ([i][i]: central pull)
+  float rcf[BS_GMAX];                    // critical radii, rounded up
+  unsigned mask[2][BS_GMAX];             // partners inside the critical radius, by evaluation
+  int cnt[2];                            // pairs listed, by evaluation
+  unsigned short pair[CL_PAIRS];         // the listed pairs i << 8 | j, i < j
   double T1[2][BS_GMAX][6];              // this level's result, double-buffered by attempt
   u64 err[BS_LEVELS];
   unsigned char cont[BS_GMAX * (BS_GMAX - 1) / 2];
@@ -55,73 +56,77 @@ struct BsClShared {
   unsigned char seqk[BS_SEQCAP];
 };
 
-// Groups of up to CL_TPS members: the terms of member q over partners p = sub, sub + CL_TPS, ...
-// (p == q: the central mass; one term per lane), summed over the member's lanes by a butterfly;
-// the same straight-line code on every lane (see bs.cu).
-__device__ __forceinline__ void cl_terms(const BsClShared &sh, const DevParams &P, double Gm0, int g, int q, int sub,
-                                         const double (*pos)[3], bool q_alive, double &ax, double &ay, double &az) {
-  ax = ay = az = 0.0;
-  const double xq = pos[q][0], yq = pos[q][1], zq = pos[q][2];
-  if (q_alive) {
-    for (int p = sub; p < g; p += CL_TPS) {
-      const bool cen = p == q;
-      const double dx = (cen ? 0.0 : pos[p][0]) - xq, dy = (cen ? 0.0 : pos[p][1]) - yq,
-                   dz = (cen ? 0.0 : pos[p][2]) - zq;
-      const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-      const bool inside = sh.alive[p] && dbits(r2) < umax64(sh.rcsq[q], sh.rcsq[p]);
-      const double f = bs_factor(r2, cen ? Gm0 : sh.gm[p], pmin(sh.A[q], sh.A[p]), cen, inside, P.kmode);
-      ax = fma(f, dx, ax); ay = fma(f, dy, ay); az = fma(f, dz, az);
-    }
-  }
-#pragma unroll
-  for (int o = CL_TPS >> 1; o > 0; o >>= 1) {
-    ax += __shfl_xor_sync(0xffffffffu, ax, o);
-    ay += __shfl_xor_sync(0xffffffffu, ay, o);
-    az += __shfl_xor_sync(0xffffffffu, az, o);
-  }
+// Single precision by truncation, on the integer pipe (a conversion takes an FP64 slot): within 2^-23,
+// 0 below 2^-126, infinite from 2^128 on.
+__device__ __forceinline__ float cl_float(double x) {
+  const u64 b = dbits(x);
+  const unsigned hi = (unsigned)(b >> 32), ex = (hi >> 20) & 0x7ffu;
+  const unsigned m = ex < 897u ? 0u : (ex > 1150u ? 0x7f800000u : ((hi & 0x7fffffffu) - (896u << 20)) << 3 | (unsigned)b >> 29);
+  return __uint_as_float(m | (hi & 0x80000000u));
 }
 
-// Groups of more than CL_TPS members: one force evaluation at positions pos, by all threads of the
-// CTA, into sh.acc.
-// Every unordered pair is evaluated once (Newton's third law), beside the central mass's pull on
-// each member: term t < g is member t's central pull G m0 d / r^3 (d from the member to the central
-// mass; zero for a ghost), term g + k the factor w d / r^3 of pair k = (a, b), d = x_b - x_a, w the
-// (1 - K) weight inside the pair's critical radius and 0 outside or for a ghost. Then member a sums,
-// one component per thread group, its central pull and G m_b times its pair factors (with the sign
-// of d) over the partners b in a fixed order. Item after item, every lane runs the same
-// straight-line code; a group of up to 15 members needs one FP64 round per SM sub-partition, where
-// a thread per (member, partner slot) needs two.
-__device__ __forceinline__ void cl_eval(BsClShared &sh, const DevParams &P, double Gm0, int g, const double (*pos)[3]) {
+// One force evaluation at the positions pos (fp: the same in single precision) by all threads of the
+// CTA; returns the acceleration of member a, component c, on the thread of (a, c).
+//  1. Groups whose pairs are more than the threads: eight lanes a member list the pairs that may be
+//     inside the pair's critical radius, from the single-precision distance with a bound on its error
+//     (outside, the weight 1 - K is zero). Smaller groups list every pair, once for the group.
+//  2. One item per thread (Newton's third law): item t < g is member t's central pull G m0 d / r^3, then
+//     the factor w d / r^3 of each listed pair (i < j), d = x_j - x_i, w the weight. A pair inside the
+//     radius (decided in FP64) leaves the factor for both members and marks each for the other.
+//  3. Member a sums its central pull and G m_b times the factors of its marked partners in ascending
+//     order (whatever the order of the list).
+// Bound by latency, the instructions of one item and of one sum after the other (levels of a small
+// group), and by FP64 issue, 64-76 cycles a warp instruction, where a group has many pairs inside.
+// Measured against every pair a term, summed over all partners with barriers between: 1024 bodies with
+// wide radii 89 -> 56 us a launch, 2048 bodies (groups of 5-12) 59.5 -> 51.7 us.
+__device__ __forceinline__ double cl_eval(BsClShared &sh, const DevParams &P, double Gm0, int g, const double (*pos)[3],
+                                          const float (*fp)[3], int &par, int a, int c) {
   const int tid = threadIdx.x;
-  const int nitems = g + g * (g - 1) / 2;
+  int nitems = g + g * (g - 1) / 2;
+  if (nitems > CL_THREADS) {
+    const int m = tid / CL_TPS, sub = tid % CL_TPS;
+    if (m < g && sh.alive[m]) {
+      const float x = fp[m][0], y = fp[m][1], z = fp[m][2], rc = sh.rcf[m], e = fabsf(x) + fabsf(y) + fabsf(z);
+      for (int q = m + 1 + sub; q < g; q += CL_TPS) {
+        const float qx = fp[q][0], qy = fp[q][1], qz = fp[q][2], dx = qx - x, dy = qy - y, dz = qz - z;
+        const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
+        // truncation moves a coordinate by at most 2^-23 of itself
+        const float lim = fmaxf(rc, sh.rcf[q]) + 4.0e-7f * (e + (fabsf(qx) + fabsf(qy) + fabsf(qz)));
+        if (!(r2 > fmaxf(lim * lim, 1.0e-30f) && r2 < 3.0e38f)) sh.pair[atomicAdd(&sh.cnt[par], 1)] = (unsigned short)(m << 8 | q);
+      }
+    }
+    __syncthreads();
+    nitems = g + sh.cnt[par];
+  }
+  if (tid < g) sh.mask[par ^ 1][tid] = 0u;  // the next evaluation's marks and list
+  if (tid == 0) sh.cnt[par ^ 1] = 0;
   for (int t = tid; t < nitems; t += CL_THREADS) {
     const bool cen = t < g;
-    const int a = cen ? t : sh.pa[t - g], b = cen ? t : sh.pb[t - g];
-    const double dx = (cen ? 0.0 : pos[b][0]) - pos[a][0], dy = (cen ? 0.0 : pos[b][1]) - pos[a][1],
-                 dz = (cen ? 0.0 : pos[b][2]) - pos[a][2];
+    const int pr = cen ? t << 8 | t : sh.pair[t - g], i = pr >> 8, j = pr & 255;
+    const double dx = (cen ? 0.0 : pos[j][0]) - pos[i][0], dy = (cen ? 0.0 : pos[j][1]) - pos[i][1],
+                 dz = (cen ? 0.0 : pos[j][2]) - pos[i][2];
     const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-    const bool inside = !cen && sh.alive[a] && sh.alive[b] && dbits(r2) < umax64(sh.rcsq[a], sh.rcsq[b]);
-    const double f = bs_factor(r2, cen ? Gm0 : 1.0, pmin(sh.A[a], sh.A[b]), cen && sh.alive[a], inside, P.kmode);
-    sh.term[t][0] = f * dx; sh.term[t][1] = f * dy; sh.term[t][2] = f * dz;
-  }
-  __syncthreads();
-  // member a, component c: ns threads, thread s takes the partners b = s, s + ns, ... (s = 0 also
-  // the central pull), partial sums combined by a butterfly over the ns lanes
-  const int ns = 24 * g <= CL_THREADS ? 8 : (12 * g <= CL_THREADS ? 4 : 2);
-  const int a = tid / (3 * ns), c = (tid / ns) % 3, sl = tid % ns;
-  double v = 0.0;
-  if (a < g) {
-    if (sl == 0) v = sh.term[a][c];
-    const int rowa = g + a * (g - 1) - a * (a - 1) / 2 - a - 1;  // term of pair (a, b > a): rowa + b
-    for (int bq = sl; bq < g; bq += ns) {
-      if (bq == a) continue;
-      if (bq > a) v = fma(sh.gm[bq], sh.term[rowa + bq][c], v);
-      else v = fma(-sh.gm[bq], sh.term[g + bq * (g - 1) - bq * (bq - 1) / 2 + a - bq - 1][c], v);
+    const bool inside = !cen && sh.alive[i] && sh.alive[j] && dbits(r2) < umax64(sh.rcsq[i], sh.rcsq[j]);
+    const double f = bs_factor(r2, cen ? Gm0 : 1.0, pmin(sh.A[i], sh.A[j]), cen && sh.alive[i], inside, P.kmode);
+    const double fx = f * dx, fy = f * dy, fz = f * dz;
+    if (cen || inside) { sh.term[i][j][0] = fx; sh.term[i][j][1] = fy; sh.term[i][j][2] = fz; }
+    if (inside) {
+      sh.term[j][i][0] = -fx; sh.term[j][i][1] = -fy; sh.term[j][i][2] = -fz;
+      atomicOr(&sh.mask[par][i], 1u << j);
+      atomicOr(&sh.mask[par][j], 1u << i);
     }
   }
-  for (int o = ns >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if (a < g && sl == 0) sh.acc[a][c] = v;
   __syncthreads();
+  double v = 0.0;
+  if (a < g) {
+    v = sh.term[a][a][c];
+    for (unsigned bits = sh.mask[par][a]; bits; bits &= bits - 1) {
+      const int q = __ffs(bits) - 1;
+      v = fma(sh.gm[q], sh.term[a][q][c], v);
+    }
+  }
+  par ^= 1;
+  return v;
 }
 
 __global__ void __cluster_dims__(CL_SIZE, 1, 1) __launch_bounds__(CL_THREADS, 2)
@@ -130,7 +135,7 @@ __global__ void __cluster_dims__(CL_SIZE, 1, 1) __launch_bounds__(CL_THREADS, 2)
   cg::cluster_group cluster = cg::this_cluster();
   const int rank = (int)cluster.block_rank();
   const int L = rank + 1, nk = 2 * L;
-  const int tid = threadIdx.x, q = tid / CL_TPS, sub = tid % CL_TPS;
+  const int tid = threadIdx.x;
   const int np = S.npad;
   const int ngroups = *S.ngroups;
   const int ncl = gridDim.x / CL_SIZE, cid = blockIdx.x / CL_SIZE;
@@ -142,22 +147,23 @@ __global__ void __cluster_dims__(CL_SIZE, 1, 1) __launch_bounds__(CL_THREADS, 2)
     if (g < gmin || g > BS_GMAX) continue;  // the same for all CTAs of the cluster (g < gmin: one-CTA kernel)
     const double m0 = S.sys_of ? S.sys_m0[S.sys_of[S.gmem[g0]]] : P.m0;
     const double Gm0 = P.G * m0;
+    const int q = tid / 3, c = tid % 3;  // chain threads: one per (member, component)
     const bool act = q < g;
+    int par = 0;
     if (tid < g) {
       const int i = S.gmem[g0 + tid];
       sh.idx[tid] = i;
       sh.alive[tid] = S.alive[i];
       sh.gm[tid] = S.gm[i]; sh.m[tid] = S.m[i]; sh.R[tid] = S.R[i]; sh.A[tid] = S.A[i];
       sh.rcsq[tid] = S.rcsq[i];
+      sh.rcf[tid] = 1.0001f * sqrtf(__double2float_ru(__longlong_as_double((long long)S.rcsq[i])));
       for (int c = 0; c < 3; ++c) { sh.y[tid][c] = S.x0[c * np + i]; sh.y[tid][3 + c] = S.v0[c * np + i]; }
     }
     if (tid == 0) { sh.H = tau; sh.rem = tau; sh.U = 0.0; sh.nseq = 0; }
-    for (int k = tid; k < g * (g - 1) / 2; k += CL_THREADS) {
-      int pa = 0, rest = k;
-      while (rest >= g - 1 - pa) { rest -= g - 1 - pa; pa++; }
-      sh.pa[k] = (unsigned char)pa;
-      sh.pb[k] = (unsigned char)(pa + 1 + rest);
-    }
+    if (tid < 2) sh.cnt[tid] = 0;
+    if (tid < 2 * BS_GMAX) sh.mask[tid / BS_GMAX][tid % BS_GMAX] = 0u;
+    if (g + g * (g - 1) / 2 <= CL_THREADS && tid < g)  // every pair, row by row
+      for (int j = tid + 1, k = tid * (g - 1) - tid * (tid - 1) / 2; j < g; ++j, ++k) sh.pair[k] = (unsigned short)(tid << 8 | j);
     __syncthreads();
     int halvings = 0, attempts = 0, steps = 0, buf = 0;
     while (true) {
@@ -180,25 +186,16 @@ __global__ void __cluster_dims__(CL_SIZE, 1, 1) __launch_bounds__(CL_THREADS, 2)
       // barrier, read T_{Lc,1} from its CTA, extend their tableau rows (thread (qc, cc): member
       // qc, component cc) and test level Lc; the first converged level ends the attempt in every
       // CTA at once (the same data, the same arithmetic, so the same decision).
-      double zA[6], zB[6], out[6];
-      for (int c = 0; c < 6; ++c) zA[c] = act ? sh.y[q][c] : 0.0;
-      if (act && sub == 0) for (int c = 0; c < 3; ++c) sh.pos[0][q][c] = zA[c];
+      double xA = act ? sh.y[q][c] : 0.0, vA = act ? sh.y[q][3 + c] : 0.0, xB = xA, vB = vA;
+      if (act) { sh.pos[0][q][c] = xA; sh.fp[0][q][c] = cl_float(xA); }
       const int qc = tid / 6, cc = tid % 6;
       const bool rowth = qc < g;
       if (tid < BS_LEVELS) sh.err[tid] = 0ULL;
       __syncthreads();
-      double ax = 0.0, ay = 0.0, az = 0.0;
-      if (g > CL_TPS) {
-        cl_eval(sh, P, Gm0, g, sh.pos[0]);
-        if (act) { ax = sh.acc[q][0]; ay = sh.acc[q][1]; az = sh.acc[q][2]; }
-      } else if (__any_sync(0xffffffffu, act)) {
-        cl_terms(sh, P, Gm0, g, act ? q : 0, sub, sh.pos[0], qa, ax, ay, az);
-      }
+      double acc_c = cl_eval(sh, P, Gm0, g, sh.pos[0], sh.fp[0], par, q, c);
       if (qa) {
-        zB[0] = fma(h, zA[3], zA[0]); zB[1] = fma(h, zA[4], zA[1]); zB[2] = fma(h, zA[5], zA[2]);
-        zB[3] = fma(h, ax, zA[3]); zB[4] = fma(h, ay, zA[4]); zB[5] = fma(h, az, zA[5]);
-      } else {
-        for (int c = 0; c < 6; ++c) zB[c] = zA[c];
+        xB = fma(h, vA, xA);
+        vB = fma(h, acc_c, vA);
       }
       const int lmax = P.bs_kmax < BS_LEVELS ? P.bs_kmax : BS_LEVELS;
       const u64 eps = dbits(P.bs_eps);
@@ -209,32 +206,18 @@ __global__ void __cluster_dims__(CL_SIZE, 1, 1) __launch_bounds__(CL_THREADS, 2)
       for (int e = 1; e <= 2 * lmax; ++e) {
         const bool lv = e <= nk;  // this CTA's level is still integrating
         if (lv) {
-          if (act && sub == 0) for (int c = 0; c < 3; ++c) sh.pos[b][q][c] = zB[c];
+          if (act) { sh.pos[b][q][c] = xB; sh.fp[b][q][c] = cl_float(xB); }
           __syncthreads();
-          if (g > CL_TPS) {
-            cl_eval(sh, P, Gm0, g, sh.pos[b]);
-            if (act) { ax = sh.acc[q][0]; ay = sh.acc[q][1]; az = sh.acc[q][2]; }
-          } else if (__any_sync(0xffffffffu, act)) {
-            cl_terms(sh, P, Gm0, g, act ? q : 0, sub, sh.pos[b], qa, ax, ay, az);
+          acc_c = cl_eval(sh, P, Gm0, g, sh.pos[b], sh.fp[b], par, q, c);
+          if (qa && e < nk) {
+            const double xn = fma(h2, vB, xA), vn = fma(h2, acc_c, vA);
+            xA = xB; vA = vB;
+            xB = xn; vB = vn;
           }
-          if (qa) {
-            if (e < nk) {
-              double zn[6];
-              zn[0] = fma(h2, zB[3], zA[0]); zn[1] = fma(h2, zB[4], zA[1]); zn[2] = fma(h2, zB[5], zA[2]);
-              zn[3] = fma(h2, ax, zA[3]); zn[4] = fma(h2, ay, zA[4]); zn[5] = fma(h2, az, zA[5]);
-              for (int c = 0; c < 6; ++c) { zA[c] = zB[c]; zB[c] = zn[c]; }
-            } else {
-              out[0] = 0.5 * fma(h, zB[3], zB[0] + zA[0]);
-              out[1] = 0.5 * fma(h, zB[4], zB[1] + zA[1]);
-              out[2] = 0.5 * fma(h, zB[5], zB[2] + zA[2]);
-              out[3] = 0.5 * fma(h, ax, zB[3] + zA[3]);
-              out[4] = 0.5 * fma(h, ay, zB[4] + zA[4]);
-              out[5] = 0.5 * fma(h, az, zB[5] + zA[5]);
-            }
-          } else if (act && e == nk) {
-            for (int c = 0; c < 6; ++c) out[c] = zA[c];
+          if (e == nk && act) {  // T_{L,1}
+            sh.T1[buf][q][c] = qa ? 0.5 * fma(h, vB, xB + xA) : xA;
+            sh.T1[buf][q][3 + c] = qa ? 0.5 * fma(h, acc_c, vB + vA) : vA;
           }
-          if (e == nk && act && sub == 0) for (int c = 0; c < 6; ++c) sh.T1[buf][q][c] = out[c];
           b ^= 1;
         }
         if (e & 1) continue;

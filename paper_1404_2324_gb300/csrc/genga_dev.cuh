@@ -605,16 +605,17 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// The warp's sums of three numbers at once: lanes 0-7 receive that of x, 8-15 of y, 16-31 of z. Six FP64
-// additions where three butterflies take fifteen.
-__device__ __forceinline__ double warp_sum3(double x, double y, double z) {
-  const int lane = threadIdx.x & 31;
-  const bool up = lane & 16, odd = lane & 8;
-  const double p = (up ? z : x) + __shfl_xor_sync(0xffffffffu, up ? x : z, 16);
-  const double q = y + __shfl_xor_sync(0xffffffffu, y, 16);
-  double r = (!up && odd ? q : p) + __shfl_xor_sync(0xffffffffu, !up && !odd ? q : p, 8);
+// The sums of three numbers over each segment of LPB lanes (8, 16 or 32) at once: the segment's first
+// quarter receives that of x, the second of y, the second half of z. Two or three FP64 additions more
+// than one butterfly, where three take fifteen (LPB = 32).
+template <int LPB>
+__device__ __forceinline__ double segment_sum3(double x, double y, double z) {
+  const bool up = threadIdx.x & (LPB / 2), odd = threadIdx.x & (LPB / 4);
+  const double p = (up ? z : x) + __shfl_xor_sync(0xffffffffu, up ? x : z, LPB / 2);
+  const double q = y + __shfl_xor_sync(0xffffffffu, y, LPB / 2);
+  double r = (!up && odd ? q : p) + __shfl_xor_sync(0xffffffffu, !up && !odd ? q : p, LPB / 4);
 #pragma unroll
-  for (int o = 4; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+  for (int o = LPB / 8; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
   return r;
 }
 
@@ -630,7 +631,7 @@ __device__ __forceinline__ void sun_shift(const Sim &S, double h1, double h2, do
     for (int t = lane; t < S.nt; t += 32)
 #pragma unroll
       for (int c = 0; c < 3; ++c) a[c] = fma(h2, S.pkick[t * 3 + c], a[c]);
-  const double s = warp_sum3(a[0], a[1], a[2]);
+  const double s = segment_sum3<32>(a[0], a[1], a[2]);
 #pragma unroll
   for (int c = 0; c < 3; ++c) sh[c] = __shfl_sync(0xffffffffu, s, 8 * c);
 }

@@ -256,7 +256,7 @@ __device__ __forceinline__ double near_factor(const Sim &S, const DevParams &P, 
 }
 
 // ---------------------------------------------------------------------------------------------
-// Finalisation, one warp per body, FIN_BODIES bodies per CTA:
+// Finalisation, LPB lanes per body, FIN_BODIES bodies per CTA:
 //   CLOSE: a = sum of the pair partials (far field, stored for reuse) + near pairs;
 //          v += h1 a (+ h2 a for the next substep's opening kick). The second Sun drift of the
 //          substep (which the kick does not see: it shifts every body alike) is applied by the
@@ -265,91 +265,93 @@ __device__ __forceinline__ double near_factor(const Sim &S, const DevParams &P, 
 //   OPEN : first kick of a full step with the new critical radii: a = stored far field + near
 //          pairs recomputed (KickA; KickB when there are none), or the full recompute's partials.
 //   INIT : the very first kick: store the far field (and a = far + near into aout [3][ald] if given).
-// Eight lanes a component sum the pair partials. The near partners are read from the body's row of the
-// candidate bitmap, in ascending order, and evaluated one per lane, once for all three components; the
-// sums have a fixed order. Also writes the CTA's momentum of the new velocities for the next Sun drift.
+// The near partners are read from the body's row of the candidate bitmap, in ascending order, and
+// evaluated one per lane, once for all three components; the sums have a fixed order. Also writes the
+// CTA's momentum of the new velocities for the next Sun drift.
 //
-// Bound by latency (launch, the chain row -> positions -> FP64 terms -> sums) and, with wide critical
-// radii, by the near pairs' FP64 issue. Measured against one CTA per tile and component, which gathered
-// and ranked the candidate lists of 32 bodies and left rows of more than 32 partners to one lane each:
-// 1024 bodies with wide radii 58 -> 9.7 us (opening 39 -> 7.4), 2048 bodies 12.9 -> 9, 32 bodies
-// 10.0 -> 7.4.
+// Bound by latency (launch, the chain row -> positions -> FP64 terms -> sums) and by FP64 issue, 64-76
+// cycles a warp instruction whatever its active lanes: LPB is the most (8, 16 or 32) that leaves one
+// warp on each sub-partition. Measured against one CTA per tile and component, which gathered and
+// ranked the candidate lists of 32 bodies and left rows of more than 32 partners to one lane each:
+// 1024 bodies with wide radii 58 -> 10 us (opening 39 -> 8), 32 bodies 10.0 -> 7.4 us; against one warp
+// per body at every size, 4 steps of 2048 bodies 1.69 -> 1.62 ms (with the cluster kernel's change).
 // ---------------------------------------------------------------------------------------------
 constexpr int FIN_BODIES = 32 / FIN_PER_TILE;
 
-template <int MODE>
-__global__ void __launch_bounds__(32 * FIN_BODIES) k_fin(Sim S, DevParams P, double h1, double h2, double *aout, int ald,
-                                                         int nslot) {
+template <int MODE, int LPB>
+__global__ void __launch_bounds__(FIN_BODIES * LPB) k_fin(Sim S, DevParams P, double h1, double h2, double *aout, int ald,
+                                                          int nslot) {
   constexpr bool ALL = MODE == FIN_CLOSE_ALL;  // the pair kernel weighed every pair: no near pass
-  __shared__ unsigned short s_j[FIN_BODIES][1024];  // partners found in 32 words of the row
+  __shared__ unsigned short s_j[FIN_BODIES][NMAX];  // near partners
   __shared__ double s_pm[3][FIN_BODIES];
-  const int wi = threadIdx.x >> 5, lane = threadIdx.x & 31, np = S.npad;
-  const int i = blockIdx.x * FIN_BODIES + wi, c = lane >> 3, sl = lane & 7;
-  const bool comp = c < 3, use_part = (MODE != FIN_OPEN) || (S.flags[0] != 0);
-  const bool near = !ALL && !(MODE == FIN_OPEN && use_part);
+  const int tid = threadIdx.x, bi = tid / LPB, sl = tid % LPB, np = S.npad;
+  const int i = blockIdx.x * FIN_BODIES + bi;
+  // this lane's component of the sums, held by the first lane of a quarter
+  const int c = sl / (LPB / 4) < 2 ? sl / (LPB / 4) : 2;
+  const bool own = sl % (LPB / 4) == 0 && sl < 3 * (LPB / 4);
+  const bool use_part = (MODE != FIN_OPEN) || (S.flags[0] != 0);
+  const bool near = !ALL && !(MODE == FIN_OPEN && use_part) && ((S.rowany[i >> 5] >> (i & 31)) & 1u);
   // the loads of the final update first, so that their latency passes under the sums
-  const double a_far = (!use_part && comp) ? S.afar[c * np + i] : 0.0;
-  const double v_old = (MODE != FIN_INIT && comp) ? S.v[c * np + i] : 0.0;
+  const double a_far = !use_part ? S.afar[c * np + i] : 0.0;
+  const double v_old = MODE != FIN_INIT ? S.v[c * np + i] : 0.0;
   const double m_i = S.m[i];
   const bool alive = S.alive[i] != 0;
   double a = a_far;
   if (use_part) {
-    double a0 = 0.0, a1 = 0.0;
-    if (comp) {
-      const double *p = S.part + (size_t)(i >> 5) * nslot * 96 + c * 32 + (i & 31);
-      int s = sl;
+    double f[3] = {0.0, 0.0, 0.0};
+    const double *p = S.part + (size_t)(i >> 5) * nslot * 96 + (i & 31);
 #pragma unroll 4
-      for (; s + 8 < nslot; s += 16) { a0 += p[(size_t)s * 96]; a1 += p[(size_t)(s + 8) * 96]; }
-      if (s < nslot) a0 += p[(size_t)s * 96];
-    }
-    a = a0 + a1;
-#pragma unroll
-    for (int o = 4; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    for (int s = sl; s < nslot; s += LPB)
+      for (int k = 0; k < 3; ++k) f[k] += p[(size_t)s * 96 + 32 * k];
+    a = segment_sum3<LPB>(f[0], f[1], f[2]);
   }
-  if (MODE != FIN_OPEN && !ALL && comp && sl == 0) S.afar[c * np + i] = a;
-  if (near && ((S.rowany[i >> 5] >> (i & 31)) & 1u)) {
+  if (MODE != FIN_OPEN && !ALL && own) S.afar[c * np + i] = a;
+  if (__any_sync(0xffffffffu, near)) {
+    const int wl = (S.W + LPB - 1) / LPB, w0 = sl * wl, w1 = near ? (w0 + wl < S.W ? w0 + wl : S.W) : w0;
+    const unsigned *row = S.cbm + (size_t)i * S.W;
+    int mine = 0;
+    for (int w = w0; w < w1; ++w) mine += __popc(row[w]);
+    int incl = mine;
+#pragma unroll
+    for (int o = 1; o < LPB; o <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, incl, o, LPB);
+      if (sl >= o) incl += t;
+    }
+    const int cnt = __shfl_sync(0xffffffffu, incl, LPB - 1, LPB);
+    if (mine) {
+      int k = incl - mine;
+      for (int w = w0; w < w1; ++w)
+        for (unsigned bits = row[w]; bits; bits &= bits - 1) s_j[bi][k++] = (unsigned short)(w * 32 + __ffs(bits) - 1);
+    }
+    __syncwarp();
     const double xi = S.x[i], yi = S.x[np + i], zi = S.x[2 * np + i], Ai = S.A[i];
     const u64 Qi = S.rcsq[i];
     double nx = 0.0, ny = 0.0, nz = 0.0;
-    for (int w0 = 0; w0 < S.W; w0 += 32) {
-      unsigned bits = w0 + lane < S.W ? S.cbm[(size_t)i * S.W + w0 + lane] : 0u;
-      const int mine = __popc(bits);
-      int incl = mine;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
-      }
-      const int cnt = __shfl_sync(0xffffffffu, incl, 31);
-      for (int k = incl - mine; bits; ++k, bits &= bits - 1) s_j[wi][k] = (unsigned short)((w0 + lane) * 32 + __ffs(bits) - 1);
-      __syncwarp();
-      for (int k = lane; k < cnt; k += 32) {
-        const int j = s_j[wi][k];
-        const double dx = S.x[j] - xi, dy = S.x[np + j] - yi, dz = S.x[2 * np + j] - zi;
-        const double f = near_factor(S, P, Qi, Ai, j, r2_exact(dx, dy, dz));
-        nx = fma(f, dx, nx); ny = fma(f, dy, ny); nz = fma(f, dz, nz);
-      }
-      __syncwarp();
+    for (int k = sl; k < cnt; k += LPB) {
+      const int j = s_j[bi][k];
+      const double dx = S.x[j] - xi, dy = S.x[np + j] - yi, dz = S.x[2 * np + j] - zi;
+      const double f = near_factor(S, P, Qi, Ai, j, r2_exact(dx, dy, dz));
+      nx = fma(f, dx, nx); ny = fma(f, dy, ny); nz = fma(f, dz, nz);
     }
-    a += warp_sum3(nx, ny, nz);
+    a += segment_sum3<LPB>(nx, ny, nz);
   }
-  if (aout && i < S.n && comp && sl == 0) aout[(size_t)c * ald + i] = a;
+  if (aout && i < S.n && own) aout[(size_t)c * ald + i] = a;
   if (MODE == FIN_INIT) return;
-  if (comp && sl == 0) {
+  if (own) {
     double v = v_old;
     if (alive) {
       v = fma(h1, a, v);
       if (h2 != 0.0) v = fma(h2, a, v);
       S.v[c * np + i] = v;
     }
-    s_pm[c][wi] = m_i * v;
+    s_pm[c][bi] = m_i * v;
   }
   __syncthreads();
-  if (wi != 0) return;
-  double pm = comp ? s_pm[c][sl] : 0.0;
+  if (tid >= 32) return;
+  double pm = tid < 3 * FIN_BODIES ? s_pm[tid / FIN_BODIES][tid % FIN_BODIES] : 0.0;
 #pragma unroll
   for (int o = FIN_BODIES / 2; o > 0; o >>= 1) pm += __shfl_xor_sync(0xffffffffu, pm, o);
-  if (comp && sl == 0) S.pfin[blockIdx.x * 3 + c] = pm;
+  if (tid < 3 * FIN_BODIES && tid % FIN_BODIES == 0) S.pfin[blockIdx.x * 3 + tid / FIN_BODIES] = pm;
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -369,14 +371,23 @@ void launch_kick(const Sim &S, const DevParams &P, bool full, bool precise, cuda
   }
 }
 
+// Lanes per body: about 600 sub-partitions, one warp each.
+template <int MODE>
+static void fin_lanes(const Sim &S, const DevParams &P, double h1, double h2, double *aout, int ald, int nslot,
+                      cudaStream_t st) {
+  const int grid = S.nt * FIN_PER_TILE;
+  if (S.npad > 1216) k_fin<MODE, 8><<<grid, 8 * FIN_BODIES, 0, st>>>(S, P, h1, h2, aout, ald, nslot);
+  else if (S.npad > 608) k_fin<MODE, 16><<<grid, 16 * FIN_BODIES, 0, st>>>(S, P, h1, h2, aout, ald, nslot);
+  else k_fin<MODE, 32><<<grid, 32 * FIN_BODIES, 0, st>>>(S, P, h1, h2, aout, ald, nslot);
+}
+
 void launch_fin(const Sim &S, const DevParams &P, FinMode mode, bool precise, double h1, double h2, double *aout,
                 int ald, cudaStream_t st) {
-  const int grid = S.nt * FIN_PER_TILE, block = 32 * FIN_BODIES;
   const int nslot = precise ? 2 * S.nt : S.kch;  // partial-sum slots per tile of the pair kernel used
-  if (mode == FIN_CLOSE) k_fin<FIN_CLOSE><<<grid, block, 0, st>>>(S, P, h1, h2, aout, ald, nslot);
-  else if (mode == FIN_CLOSE_ALL) k_fin<FIN_CLOSE_ALL><<<grid, block, 0, st>>>(S, P, h1, h2, aout, ald, nslot);
-  else if (mode == FIN_OPEN) k_fin<FIN_OPEN><<<grid, block, 0, st>>>(S, P, h1, h2, aout, ald, nslot);
-  else k_fin<FIN_INIT><<<grid, block, 0, st>>>(S, P, h1, h2, aout, ald, nslot);
+  if (mode == FIN_CLOSE) fin_lanes<FIN_CLOSE>(S, P, h1, h2, aout, ald, nslot, st);
+  else if (mode == FIN_CLOSE_ALL) fin_lanes<FIN_CLOSE_ALL>(S, P, h1, h2, aout, ald, nslot, st);
+  else if (mode == FIN_OPEN) fin_lanes<FIN_OPEN>(S, P, h1, h2, aout, ald, nslot, st);
+  else fin_lanes<FIN_INIT>(S, P, h1, h2, aout, ald, nslot, st);
 }
 
 // Second Sun drift after the last substep: x += hcm * P, P the momentum before the closing kick.
@@ -386,7 +397,7 @@ __global__ void k_hc(Sim S, double hcm) {
   double p[3] = {0.0, 0.0, 0.0};
   for (int t = lane; t < S.nt; t += 32)
     for (int c = 0; c < 3; ++c) p[c] += S.pkick[t * 3 + c];
-  const double ps = warp_sum3(p[0], p[1], p[2]);
+  const double ps = segment_sum3<32>(p[0], p[1], p[2]);
 #pragma unroll
   for (int c = 0; c < 3; ++c) p[c] = __shfl_sync(0xffffffffu, ps, 8 * c);
   if (i >= S.npad || !S.alive[i]) return;
