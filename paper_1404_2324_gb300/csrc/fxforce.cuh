@@ -107,6 +107,23 @@ FX_HD double pull_factor(double r2, const Num &pref, const Num &A, bool full, bo
   return to_double(factor(R, rho2, k, pref, A, full, zone), pref.me - 59 - 3 * k);
 }
 
+// r^-3 and r^-5 for r2 > 0 (normal).
+FX_HD void inverse_powers(double r2, double &y3, double &y5) {
+  const u64 b = d2u(r2);
+  const int q = (int)(b >> 52) - 1022, odd = q & 1, k = (q - odd) >> 1;  // r2 = R 4^k, R in [0.5, 2)
+  const u64 R = (((b & 0xfffffffffffffULL) | 0x10000000000000ULL) << 9) << odd;  // 2^-62
+  const float rho2 = i2f(((126 + odd) << 23) | (int)((u32)(b >> 29) & 0x7fffffu));
+  const u32 U = (u32)f2i(frsqrt(rho2) + 2.0f) << 9;             // 2^-31
+  const u64 W = mulu(U, U);                                     // 2^-62
+  const u64 e = (1ULL << 60) - mulhi(R, W);                     // 2^-60, signed
+  const int e1 = (int)((i64)e >> 11);                           // 2^-49
+  const u32 ee = hi32((u64)muls(e1, e1));                       // 2^-66
+  const u64 Y3 = mulhi(mul32(W, U), (1ULL << 63) + 12ULL * e + (ee * 15u >> 6));  // rho^-3, 2^-60
+  const u64 Y2 = mulhi(W, (1ULL << 63) + 8ULL * e + (ee >> 3)); // rho^-2, 2^-61
+  y3 = to_double(Y3, -60 - 3 * k);
+  y5 = to_double(mulhi(Y3 << 1, Y2 << 1), -59 - 5 * k);
+}
+
 }  // namespace fx
 
 #ifdef __CUDACC__

@@ -218,3 +218,22 @@ def test_forward_kick_at_tile_and_chunk_edges(n):
         for got, k in ((xo, 0), (vo, 1)):
             assert _rel(got[b].cpu().numpy(), ref[b][k]) <= max(1e-12, 30 * _rel(alt[b][k], ref[b][k])), (b, k)
     eng.close()
+
+
+@pytest.mark.parametrize("n", [33, 66])
+def test_gradient_of_ragged_tiles_equals_oracle_tangent_map(n):
+    """One step of a ring that fills its last tile with one or two bodies: every pair of tiles of the
+    kick's VJP, the diagonal ones included; the bound of the gradient test above."""
+    rng = np.random.default_rng(n)
+    d = ics._disk(rng, n, 1e-7, 1e-6, 0.95, (0.9025 + 0.00418 * n) ** 0.5, 0.01, 0.005)
+    x, v, m = d["x"], d["v"], d["m"]
+    eng = AdjointEngine(np.ones(1), G, 6.0, 2, ckpt_every=4)
+    eng.forward(_t(x[None]), _t(v[None]), _t(m[None]), 1)
+    ux, uv = rng.standard_normal((n, 3)), rng.standard_normal((n, 3)) * 50.0
+    gx, gv, gm = (t.cpu().numpy()[0] for t in eng.backward(_t(ux[None]), _t(uv[None])))
+    T = TG.TangentSim(O.params(G=G, m0=1.0, dt=6.0, order=2, collisions=0), m, x, v)
+    T.step(1)
+    ref = T.jacobian().T @ np.concatenate([ux.ravel(), uv.ravel()])
+    for got, sl in ((gx, slice(0, 3 * n)), (gv, slice(3 * n, 6 * n)), (gm, slice(6 * n, 7 * n))):
+        assert np.linalg.norm(got.ravel() - ref[sl]) <= 1e-8 * np.linalg.norm(ref[sl]), sl
+    eng.close()
