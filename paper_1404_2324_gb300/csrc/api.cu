@@ -310,8 +310,8 @@ void enqueue_step(genga_ctx *c, cudaStream_t st) {
   const bool tp = c->tpmode;
   const TPSet &T = c->T;
   launch_rcrit(S, P, std::fabs(dt), 1, st);
-  launch_kick(S, P, true, precise, st);  // runs only if the critical radii grew too much
-  launch_fin(S, P, FIN_OPEN, precise, 0.5 * c->w[0] * dt, 0.0, nullptr, 0, st);
+  launch_kick(S, P, true, precise, st, false, true);  // runs only if the critical radii grew too much
+  launch_fin(S, P, FIN_OPEN, precise, 0.5 * c->w[0] * dt, 0.0, nullptr, 0, st, true);
   for (int j = 0; j < c->nsub; ++j) {
     const double tau = c->w[j] * dt;
     const double hcm2 = j > 0 ? 0.5 * c->w[j - 1] * dt * inv_m0 : 0.0;
@@ -319,7 +319,7 @@ void enqueue_step(genga_ctx *c, cudaStream_t st) {
     // kick reads); at the first substep it carries their critical radii and opening kick as well
     if (tp && j == 0) launch_tp_open_drift(S, T, P, std::fabs(dt), 0.5 * c->w[0] * dt, tau, 0.5 * tau * inv_m0, st);
     else if (tp) launch_tp_drift(S, T, P, tau, 0.5 * tau * inv_m0, hcm2, st);
-    launch_drift(S, P, tau, 0.5 * tau * inv_m0, hcm2, j, st);             // clears the reuse flag
+    launch_drift(S, P, tau, 0.5 * tau * inv_m0, hcm2, j, st, true);       // clears the reuse flag
     if (tp) {  // the planets' paths for the particles, on a branch beside the planets' encounters and BS
       cudaEventRecord(c->ev_tab, st);
       cudaStreamWaitEvent(c->side3, c->ev_tab, 0);
@@ -338,7 +338,7 @@ void enqueue_step(genga_ctx *c, cudaStream_t st) {
       cudaStreamWaitEvent(c->side2, c->ev_fork, 0);
       launch_bs_cluster(S, P, tau, c->gsplit, c->cl_grid, c->side);
       launch_bs_grid(S, P, tau, BS_GMAX + 1, c->grid_blocks, c->side2);
-      launch_bs(S, P, tau, c->bs_grid, st, c->gsplit);
+      launch_bs(S, P, tau, c->bs_grid, st, c->gsplit, 1, true);
       cudaEventRecord(c->ev_join, c->side);
       cudaEventRecord(c->ev_join2, c->side2);
       cudaStreamWaitEvent(st, c->ev_join, 0);
@@ -357,7 +357,7 @@ void enqueue_step(genga_ctx *c, cudaStream_t st) {
     launch_kick(S, P, inner, precise, st, inner);
     if (c->profiling) cudaEventRecordWithFlags(c->kev[2 * j + 1], st, cudaEventRecordExternal);
     const double h2 = (j + 1 < c->nsub) ? 0.5 * c->w[j + 1] * dt : 0.0;
-    launch_fin(S, P, inner ? FIN_CLOSE_ALL : FIN_CLOSE, precise, 0.5 * tau, h2, nullptr, 0, st);
+    launch_fin(S, P, inner ? FIN_CLOSE_ALL : FIN_CLOSE, precise, 0.5 * tau, h2, nullptr, 0, st, !c->profiling);
     if (tp) {  // join; the particles' BS and every particle's closing kick (after the last substep
                // with their last Sun drift, from the massive momentum before the closing kick)
       cudaStreamWaitEvent(st, c->ev_join, 0);

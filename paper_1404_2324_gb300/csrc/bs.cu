@@ -35,6 +35,7 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? 1 : 512 / NT)
   __shared__ __align__(16) unsigned char bs_static[GM <= BS_GMAX ? sizeof(BsSharedT<GM>) : 16];
   extern __shared__ __align__(16) unsigned char bs_dyn[];
   BsSharedT<GM> &sh = *reinterpret_cast<BsSharedT<GM> *>(GM <= BS_GMAX ? bs_static : bs_dyn);
+  wait_previous();
   const int tid = threadIdx.x;
   const int ngroups = *S.ngroups;
   for (int it = 0;; ++it) {
@@ -69,9 +70,11 @@ void bs_init_constants() {
   bs_core_set_factors();
 }
 
-void launch_bs(const Sim &S, const DevParams &P, double tau, int max_groups, cudaStream_t st, int gsplit, int gmin) {
+void launch_bs(const Sim &S, const DevParams &P, double tau, int max_groups, cudaStream_t st, int gsplit, int gmin,
+               bool after) {
   const int grid = max_groups < 1 ? 1 : max_groups;
-  k_bs<BS_THREADS, BS_GMAX><<<grid, BS_THREADS, 0, st>>>(S, P, tau, gmin, gsplit, 2, 0);
+  if (after) launch_after(k_bs<BS_THREADS, BS_GMAX>, grid, BS_THREADS, st, S, P, tau, gmin, gsplit, 2, 0);
+  else k_bs<BS_THREADS, BS_GMAX><<<grid, BS_THREADS, 0, st>>>(S, P, tau, gmin, gsplit, 2, 0);
 }
 void launch_bs_small(const Sim &S, const DevParams &P, double tau, int blocks, cudaStream_t st) {
   k_bs<128, BS_GMAX><<<blocks < 1 ? 1 : blocks, 128, 0, st>>>(S, P, tau, 3, BS_SMALL + 1, 1, 0);

@@ -598,6 +598,10 @@ __device__ __forceinline__ void warp_max_to(u64 *dst, u64 v) {
   if ((threadIdx.x & 31) == 0 && v) atomicMax((unsigned long long *)dst, (unsigned long long)v);
 }
 
+// First statement of a kernel launched by launch_after: waits until every kernel before it has finished
+// and its writes are visible.
+__device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Warp reductions (butterfly), fixed order -> deterministic
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll

@@ -196,6 +196,7 @@ __device__ __forceinline__ double kx_near(const Sim &S, const DevParams &P, int 
 
 template <bool FULL, int TW>
 __global__ void __launch_bounds__(32 * KX_WARPS, KX_CTAS) k_kick_fx(Sim S, DevParams P, int force) {
+  wait_previous();
   if (FULL && !force && S.flags[0] == 0) return;
   const bool record = FULL ? (!force && S.flags[3] != 0) : true;
   const int lane = threadIdx.x & 31, np = S.npad, C = S.kch, nt = S.nt;
@@ -203,11 +204,8 @@ __global__ void __launch_bounds__(32 * KX_WARPS, KX_CTAS) k_kick_fx(Sim S, DevPa
   if ((!FULL || force) && gwarp < nt) {  // per-tile momentum before the closing kick (second Sun drift)
     const int i = gwarp * 32 + lane;
     const double mi = S.m[i];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const double p = warp_sum(mi * S.v[c * np + i]);
-      if (lane == 0) S.pkick[gwarp * 3 + c] = p;
-    }
+    const double p = segment_sum3<32>(mi * S.v[i], mi * S.v[np + i], mi * S.v[2 * np + i]);
+    if ((lane & 7) == 0 && lane < 24) S.pkick[gwarp * 3 + (lane >> 3)] = p;
   }
   const int tgroups = (nt + TW - 1) / TW;
   int I, c0;
@@ -237,13 +235,12 @@ void kick_split(int npad, int sms, int *chunks, int *chunk, int systems) {
 }
 
 template <bool FULL>
-static void launch_kick_fx(const Sim &S, const DevParams &P, int force, cudaStream_t st) {
+static void launch_kick_fx(const Sim &S, const DevParams &P, int force, cudaStream_t st, bool after) {
   const int tw = S.nt >= 8 ? 8 : (S.nt >= 4 ? 4 : (S.nt >= 2 ? 2 : 1)), cw = KX_WARPS / tw;
   const int grid = ((S.nt + tw - 1) / tw) * ((S.kch + cw - 1) / cw);
-  if (tw == 8) k_kick_fx<FULL, 8><<<grid, 32 * KX_WARPS, 0, st>>>(S, P, force);
-  else if (tw == 4) k_kick_fx<FULL, 4><<<grid, 32 * KX_WARPS, 0, st>>>(S, P, force);
-  else if (tw == 2) k_kick_fx<FULL, 2><<<grid, 32 * KX_WARPS, 0, st>>>(S, P, force);
-  else k_kick_fx<FULL, 1><<<grid, 32 * KX_WARPS, 0, st>>>(S, P, force);
+  auto *kernel = tw == 8 ? k_kick_fx<FULL, 8> : (tw == 4 ? k_kick_fx<FULL, 4> : (tw == 2 ? k_kick_fx<FULL, 2> : k_kick_fx<FULL, 1>));
+  if (after) launch_after(kernel, grid, 32 * KX_WARPS, st, S, P, force);
+  else kernel<<<grid, 32 * KX_WARPS, 0, st>>>(S, P, force);
 }
 
 // The near-pair pull of partner j on body i, per unit separation, with the current critical radii
@@ -284,6 +281,7 @@ __global__ void __launch_bounds__(FIN_BODIES * LPB) k_fin(Sim S, DevParams P, do
   constexpr bool ALL = MODE == FIN_CLOSE_ALL;  // the pair kernel weighed every pair: no near pass
   __shared__ unsigned short s_j[FIN_BODIES][NMAX];  // near partners
   __shared__ double s_pm[3][FIN_BODIES];
+  wait_previous();
   const int tid = threadIdx.x, bi = tid / LPB, sl = tid % LPB, np = S.npad;
   const int i = blockIdx.x * FIN_BODIES + bi;
   // this lane's component of the sums, held by the first lane of a quarter
@@ -359,39 +357,40 @@ void launch_rcrit(const Sim &S, const DevParams &P, double tau_abs, int check_re
   k_rcrit<<<(S.npad + 127) / 128, 128, 0, st>>>(S, P, tau_abs, check_reuse);
 }
 
-void launch_kick(const Sim &S, const DevParams &P, bool full, bool precise, cudaStream_t st, bool force) {
+void launch_kick(const Sim &S, const DevParams &P, bool full, bool precise, cudaStream_t st, bool force, bool after) {
   const int f = force ? 1 : 0;
   if (precise) {
     const int grid = ((S.nwarps > S.nt ? S.nwarps : S.nt) * 32 + 127) / 128;
     if (full) k_kick_precise<true><<<grid, 128, 0, st>>>(S, P, f);
     else k_kick_precise<false><<<grid, 128, 0, st>>>(S, P, 0);
   } else {
-    if (full) launch_kick_fx<true>(S, P, f, st);
-    else launch_kick_fx<false>(S, P, 0, st);
+    if (full) launch_kick_fx<true>(S, P, f, st, after);
+    else launch_kick_fx<false>(S, P, 0, st, after);
   }
 }
 
 // Lanes per body: about 600 sub-partitions, one warp each.
 template <int MODE>
 static void fin_lanes(const Sim &S, const DevParams &P, double h1, double h2, double *aout, int ald, int nslot,
-                      cudaStream_t st) {
-  const int grid = S.nt * FIN_PER_TILE;
-  if (S.npad > 1216) k_fin<MODE, 8><<<grid, 8 * FIN_BODIES, 0, st>>>(S, P, h1, h2, aout, ald, nslot);
-  else if (S.npad > 608) k_fin<MODE, 16><<<grid, 16 * FIN_BODIES, 0, st>>>(S, P, h1, h2, aout, ald, nslot);
-  else k_fin<MODE, 32><<<grid, 32 * FIN_BODIES, 0, st>>>(S, P, h1, h2, aout, ald, nslot);
+                      cudaStream_t st, bool after) {
+  const int lpb = S.npad > 1216 ? 8 : (S.npad > 608 ? 16 : 32), grid = S.nt * FIN_PER_TILE;
+  auto *kernel = lpb == 8 ? k_fin<MODE, 8> : (lpb == 16 ? k_fin<MODE, 16> : k_fin<MODE, 32>);
+  if (after) launch_after(kernel, grid, lpb * FIN_BODIES, st, S, P, h1, h2, aout, ald, nslot);
+  else kernel<<<grid, lpb * FIN_BODIES, 0, st>>>(S, P, h1, h2, aout, ald, nslot);
 }
 
 void launch_fin(const Sim &S, const DevParams &P, FinMode mode, bool precise, double h1, double h2, double *aout,
-                int ald, cudaStream_t st) {
+                int ald, cudaStream_t st, bool after) {
   const int nslot = precise ? 2 * S.nt : S.kch;  // partial-sum slots per tile of the pair kernel used
-  if (mode == FIN_CLOSE) fin_lanes<FIN_CLOSE>(S, P, h1, h2, aout, ald, nslot, st);
-  else if (mode == FIN_CLOSE_ALL) fin_lanes<FIN_CLOSE_ALL>(S, P, h1, h2, aout, ald, nslot, st);
-  else if (mode == FIN_OPEN) fin_lanes<FIN_OPEN>(S, P, h1, h2, aout, ald, nslot, st);
-  else fin_lanes<FIN_INIT>(S, P, h1, h2, aout, ald, nslot, st);
+  if (mode == FIN_CLOSE) fin_lanes<FIN_CLOSE>(S, P, h1, h2, aout, ald, nslot, st, after);
+  else if (mode == FIN_CLOSE_ALL) fin_lanes<FIN_CLOSE_ALL>(S, P, h1, h2, aout, ald, nslot, st, after);
+  else if (mode == FIN_OPEN) fin_lanes<FIN_OPEN>(S, P, h1, h2, aout, ald, nslot, st, after);
+  else fin_lanes<FIN_INIT>(S, P, h1, h2, aout, ald, nslot, st, after);
 }
 
 // Second Sun drift after the last substep: x += hcm * P, P the momentum before the closing kick.
 __global__ void k_hc(Sim S, double hcm) {
+  wait_previous();
   const int lane = threadIdx.x & 31;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   double p[3] = {0.0, 0.0, 0.0};
@@ -406,7 +405,7 @@ __global__ void k_hc(Sim S, double hcm) {
 }
 
 void launch_hc(const Sim &S, double hcm, cudaStream_t st) {
-  k_hc<<<(S.npad + 63) / 64, 64, 0, st>>>(S, hcm);
+  launch_after(k_hc, (S.npad + 63) / 64, 64, st, S, hcm);
 }
 
 }  // namespace genga

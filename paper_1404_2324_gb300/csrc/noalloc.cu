@@ -168,8 +168,8 @@ extern "C" int genga_kick_noalloc(int n, double G, double pc, int kmode, int pre
   if (precise_div) k_items<<<1, 32, 0, st>>>(S.items, S.nt);
   // 8 threads a body: the bitmap's words, up to 32 a body, are most of what there is to clear
   k_kick_setup<<<(8 * S.npad + 127) / 128, 128, 0, st>>>(S, G, pc, m, alive, x, rc, n);
-  launch_kick(S, P, false, precise_div != 0, st);
-  launch_fin(S, P, FIN_INIT, precise_div != 0, 0.0, 0.0, a, n, st);
-  launch_bitmap_pairs(S.cbm, S.rowany, S.npad, S.W, cand, cap, ncand, st);
+  launch_kick(S, P, false, precise_div != 0, st, false, true);
+  launch_fin(S, P, FIN_INIT, precise_div != 0, 0.0, 0.0, a, n, st, true);
+  launch_bitmap_pairs(S.cbm, S.rowany, S.npad, S.W, cand, cap, ncand, st, true);
   return cudaGetLastError() == cudaSuccess ? GENGA_OK : GENGA_ECUDA;
 }

@@ -11,6 +11,7 @@ namespace genga {
 // warp sums the per-tile momentum partials itself (no extra launch).
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(32) k_drift(Sim S, DevParams P, double tau, double hcm1, double hcm2, int substep) {
+  wait_previous();
   const int lane = threadIdx.x;
   const int i = blockIdx.x * 32 + lane;
   const int np = S.npad;
@@ -336,6 +337,7 @@ __global__ void __launch_bounds__(GROUP_THREADS) k_encounter_group(Sim S, double
   __shared__ int s_i[EG_CAP], s_j[EG_CAP];
   __shared__ int s_n, s_found, s_last;
   __shared__ GroupShared sm;
+  wait_previous();
   encounter_body<GROUP_THREADS, EG_BODIES, EG_CAP>(S, tau, ebm, keep, s_i, s_j, s_n, s_found);
   if (threadIdx.x == 0) {
     __threadfence();  // this CTA's edges before its count
@@ -379,6 +381,7 @@ __global__ void __launch_bounds__(1024) k_bitmap_pairs(const unsigned *bm, const
                                                        int cap, int *count) {
   __shared__ int wtot[32];
   __shared__ int s_base;
+  wait_previous();
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   if (tid == 0) s_base = 0;
   __syncthreads();
@@ -449,15 +452,16 @@ __global__ void k_copy_edges(Sim S, const int *pairs, int npairs) {
 
 // ---------------------------------------------------------------------------------------------
 void launch_drift(const Sim &S, const DevParams &P, double tau, double hcm1, double hcm2,
-                  int substep, cudaStream_t st) {
-  k_drift<<<S.npad / 32, 32, 0, st>>>(S, P, tau, hcm1, hcm2, substep);
+                  int substep, cudaStream_t st, bool after) {
+  if (after) launch_after(k_drift, S.npad / 32, 32, st, S, P, tau, hcm1, hcm2, substep);
+  else k_drift<<<S.npad / 32, 32, 0, st>>>(S, P, tau, hcm1, hcm2, substep);
 }
 void launch_encounter(const Sim &S, double tau, unsigned *ebm, cudaStream_t st, bool keep) {
   k_encounter<<<(S.npad + ENC_BODIES - 1) / ENC_BODIES, ENC_THREADS, 0, st>>>(S, tau, ebm, keep ? 1 : 0);
 }
 void launch_group(const Sim &S, cudaStream_t st, int gbig) { k_group<<<1, GROUP_THREADS, 0, st>>>(S, gbig); }
 void launch_encounter_group(const Sim &S, double tau, unsigned *ebm, cudaStream_t st, bool keep, int gbig) {
-  k_encounter_group<<<(S.npad + EG_BODIES - 1) / EG_BODIES, GROUP_THREADS, 0, st>>>(S, tau, ebm, keep ? 1 : 0, gbig);
+  launch_after(k_encounter_group, (S.npad + EG_BODIES - 1) / EG_BODIES, GROUP_THREADS, st, S, tau, ebm, keep ? 1 : 0, gbig);
 }
 void launch_kepler_phase(int n, double mu, double dt, int maxit, const int *alive, double *x, double *v,
                          int *fail, cudaStream_t st) {
@@ -467,8 +471,9 @@ void launch_pairs_to_bitmap(const Sim &S, const int *pairs, int npairs, cudaStre
   if (npairs > 0) k_pairs_to_bitmap<<<(npairs + 127) / 128, 128, 0, st>>>(S, pairs, npairs);
 }
 void launch_bitmap_pairs(const unsigned *bm, const unsigned *rows, int npad, int W, int *out, int cap, int *count,
-                         cudaStream_t st) {
-  k_bitmap_pairs<<<1, 1024, 0, st>>>(bm, rows, npad, W, out, cap, count);
+                         cudaStream_t st, bool after) {
+  if (after) launch_after(k_bitmap_pairs, 1, 1024, st, bm, rows, npad, W, out, cap, count);
+  else k_bitmap_pairs<<<1, 1024, 0, st>>>(bm, rows, npad, W, out, cap, count);
 }
 void launch_single_to_fail(const Sim &S, const int *single, cudaStream_t st) {
   k_single_to_fail<<<(S.n + 127) / 128, 128, 0, st>>>(S, single);
