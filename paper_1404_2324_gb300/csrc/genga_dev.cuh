@@ -147,6 +147,8 @@ struct TPSet {
   unsigned *pairs, *npairs;      // candidate (TP, planet) pairs of the last closing kick: i * 32 + j
   double *ptab;                  // planets' Kepler paths at the BS midpoint times [TP_MAXPL * TP_TAB * 6]
   double *ppoly;                 // planets' paths over the substep, polynomials in s = 2t/tau - 1 [TP_MAXPL * 6 * TP_CHEB]
+  long long *pfix;               // the position polynomials in fixed point, unit 2^(pexp - 62) [TP_MAXPL * 3 * TP_CHEB]
+  int *pexp;
   int *pcok;                     // 1: planet j's series is exact to rounding; 0: solve Kepler instead
   long long *counters;           // candidates, encounters, BS steps, removed, ejected
 };

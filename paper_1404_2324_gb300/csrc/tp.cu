@@ -476,7 +476,17 @@ __global__ void __launch_bounds__(128) k_planet_table(Sim S, TPSet T, DevParams 
     // NaN (a failed node) fails every comparison
     if (!(decay <= lim * scale) || !(tail <= 2.0 * lim * scale) || !(sum <= 2.0 * scale)) ok = 0;
   }
+  // the position polynomial in fixed point (poly3_fx); a path whose size has no exponent to spare, or
+  // whose velocity bound fails, keeps the Kepler solve
+  const double r2 = fma(z0, z0, fma(y0, y0, x0 * x0));
+  const int ex = fx::expo(r2);  // r < 2^((ex - 1022) / 2 rounded up)
+  if (ex < 400 || ex > 1600) ok = 0;
   ok = __syncthreads_and(ok);
+  if (ok && e < 3 * TP_CHEB) {
+    const int E = ((ex - 1021) >> 1) + 2;  // 2 r < 2^(E - 1)
+    T.pfix[((size_t)j * 3) * TP_CHEB + e] = fx::fixed(mono[e / TP_CHEB][e % TP_CHEB], E);
+    if (e == 0) T.pexp[j] = E;
+  }
   if (e == 0) T.pcok[j] = ok;
 }
 
@@ -519,6 +529,32 @@ __global__ void __launch_bounds__(256) k_tp_encounter(Sim S, TPSet T, double tau
   if (s_last && threadIdx.x == 0) { *T.npairs = 0u; T.bsnext[2] = 0u; }
 }
 
+// The position of a planet's path polynomial at s in [-1, 1], |s| <= 1, from its fixed-point
+// coefficients cf (2^(62 - E), their magnitudes' sum below 2^61), Horner on the integer pipe: a step is
+// three wide multiply-adds and some 7 more instructions of 2-4 cycles where FP64 takes 64, and rounds
+// at 2^-60 of the path's size.
+__device__ __forceinline__ long long horner_fx(const long long *cf, int sh, int sl) {
+  long long a = cf[TP_CHEB - 1];
+#pragma unroll
+  for (int k = TP_CHEB - 2; k >= 0; --k) {
+    const int ah = fx::hi_s((u64)a), al = (int)fx::lo32((u64)a);
+    const long long c = fx::mads(al, sh, fx::muls(ah, sl));
+    const u64 r = (u64)fx::mads(ah, sh, c >> 32);
+    a = (long long)fx::pair64(__funnelshift_l(fx::lo32((u64)c), fx::lo32(r), 2), __funnelshift_l(fx::lo32(r), fx::hi32(r), 2)) + cf[k];
+  }
+  return a;
+}
+__device__ __forceinline__ double scale2(double x, int k) {  // x 2^k; the result normal or zero
+  return x == 0.0 ? 0.0 : fx::u2d(fx::d2u(x) + ((u64)(long long)k << 52));
+}
+__device__ __forceinline__ void poly3_fx(const long long *cf, int E, double s, double &a, double &b, double &c) {
+  const u64 S = (u64)(s >= 1.0 ? 1LL << 62 : (s <= -1.0 ? -(1LL << 62) : fx::fixed(s, 0)));
+  const int sh = fx::hi_s(S), sl = (int)fx::lo32(S);
+  a = scale2((double)horner_fx(cf, sh, sl), E - 62);
+  b = scale2((double)horner_fx(cf + TP_CHEB, sh, sl), E - 62);
+  c = scale2((double)horner_fx(cf + 2 * TP_CHEB, sh, sl), E - 62);
+}
+
 // A planet's path polynomial (components c0 .. c0 + 2, powers of s) at s in [-1, 1] (Horner).
 __device__ __forceinline__ void poly3(const double *cf, double s, double &a, double &b, double &c) {
   a = cf[TP_CHEB - 1]; b = cf[2 * TP_CHEB - 1]; c = cf[3 * TP_CHEB - 1];
@@ -544,7 +580,7 @@ __device__ __forceinline__ void planet_at(const Sim &S, const TPSet &T, const De
     return;
   }
   if (T.pcok[j]) {
-    poly3(T.ppoly + (size_t)j * 6 * TP_CHEB, fma(t, i2tau, -1.0), px, py, pz);
+    poly3_fx(T.pfix + (size_t)j * 3 * TP_CHEB, T.pexp[j], fma(t, i2tau, -1.0), px, py, pz);
     return;
   }
   const int pp = S.npad;
@@ -575,28 +611,73 @@ constexpr int TP_PRE = 2;  // encountered planets whose positions a BS attempt e
 
 __constant__ double c_tp_facinv[BS_LEVELS + 1][BS_LEVELS];  // 1 / ((L / (L - j))^2 - 1)
 
-// Acceleration of a TP at state y (level k, midpoint m of an attempt of length H from t0): the
-// Sun, and each encountered planet weighted by 1 - W_B inside the pair's critical radius. Lanes
-// pair up: level lane l (l16 < 8) evaluates the Sun's pull at its own state while lane l + 8
-// evaluates the first planet's at the same state (passed over) with the same instructions, and
-// hands back g and the separation; further planets follow on the upper lane. The level lane
-// accumulates Sun, planet 1, planet 2, ... exactly as a serial evaluation would. `act` holds the
-// participating lanes (whole pairs); planet positions come from the prepared list (wpos) for the
-// first TP_PRE planets of a shorter attempt, otherwise from the table or the path polynomial.
+// The body whose pull a lane evaluates first: the Sun on the level lanes (l16 < 8), the first
+// encountered planet on the upper ones. Constant over a particle's attempts.
+struct TpBody {
+  fx::Num gm_n, A_n;  // G m and 1/(0.9 rc) for the fixed-point factor
+  double gm, A;
+  u64 cut;            // r^2 below it: inside the critical radius
+  bool live;
+};
+__device__ __forceinline__ TpBody tp_body(const Sim &S, const TPSet &T, const DevParams &P, int i, unsigned em, bool up) {
+  TpBody b;
+  b.gm = P.Gm0; b.A = 0.0; b.cut = 0ULL; b.live = !up || em != 0u;
+  if (up && em) {
+    const int j = __ffs(em) - 1;
+    b.gm = S.gm[j];
+    b.A = pmin(T.A[i], S.A[j]);
+    b.cut = umax64(T.rcsq[i], S.rcsq[j]);
+  }
+  b.gm_n = fx::num(b.gm);
+  b.A_n = fx::num(b.A);
+  return b;
+}
+
+// Acceleration of a TP whose position is p (level k, midpoint m of an attempt of length H from t0): the
+// Sun, and each encountered planet weighted by 1 - W_B inside the pair's critical radius. Lanes pair up
+// on a level: the level lane (l16 < 8) holds components x and y of its chain and evaluates the Sun's
+// pull, lane l + 8 holds z and evaluates the first planet's with the same instructions; they exchange
+// positions and what the other's components need, 15 FP64 instructions a step of the chain where a
+// lane with all components and a passive partner took 21. Further planets follow on the upper lane.
+// Each component accumulates Sun, planet 1, planet 2, ... as a serial evaluation would. `act` holds the
+// participating lanes (whole pairs); pq: the first planet's position (prepared list or table); further
+// planets' come from the prepared list (wpos) for the first TP_PRE planets of a shorter attempt,
+// otherwise from the table or the path polynomial. The pass lasts as long as its deepest particle's chain of
+// evaluations, 3400 cycles each before; with poly3_fx's positions 10^5 particles x 4 steps 1507 -> 1298 us,
+// 2^20 particles x 2 fourth-order steps 5.54 -> 4.87 ms.
 __device__ __forceinline__ void tp_force(const Sim &S, const TPSet &T, const DevParams &P, int i, unsigned em, bool table,
                                          int k, int m, double t0, double h, double H, double i2tau, const double *wpos,
-                                         const double *y, double &ax, double &ay, double &az, unsigned act) {
-  const int lane = threadIdx.x & 31;
-  const bool up = (lane & 8) != 0;
-  const double sx = __shfl_sync(act, y[0], lane & ~8), sy = __shfl_sync(act, y[1], lane & ~8),
-               sz = __shfl_sync(act, y[2], lane & ~8);
-  unsigned bits = em;
-  for (int p = 0;; ++p) {
-    // this lane's body: the Sun (level lane, first round) or planet p (upper lane)
-    double bx = 0.0, by = 0.0, bz = 0.0, gm = P.Gm0, A = 0.0;
-    u64 cut = 0ULL;
-    const bool body = up && bits;
-    if (body) {
+                                         const TpBody &B, const double *pq, double p0, double p1, double &a0, double &a1,
+                                         unsigned act) {
+  const bool up = (threadIdx.x & 8) != 0;
+  const double e0 = __shfl_xor_sync(act, p0, 8), e1 = __shfl_xor_sync(act, p1, 8);
+  const double sx = up ? e0 : p0, sy = up ? e1 : p1, sz = up ? p0 : e0;
+  double bx = 0.0, by = 0.0, bz = 0.0;
+  if (up && em) { bx = pq[0]; by = pq[1]; bz = pq[2]; }
+  double dx = bx - sx, dy = by - sy, dz = bz - sz;
+  double r2 = fma(dz, dz, fma(dy, dy, dx * dx)), g = 0.0;
+  const bool inside = up && B.live && dbits(r2) < B.cut;
+  if (!up || inside) {
+    if (P.kmode == 0) {
+      const double f = fx::pull_factor(r2, B.gm_n, B.A_n, !up, inside);
+      g = __longlong_as_double(__double_as_longlong(f) | (__double_as_longlong(B.gm) & (long long)0x8000000000000000ULL));
+    } else {
+      g = bs_factor_gradient(r2, B.gm, B.A, !up);
+    }
+  }
+  const double tx = g * dx, ty = g * dy, tz = g * dz;  // the Sun's: -G m0 y / |y|^3
+  double x0 = __shfl_xor_sync(act, up ? g : tz, 8), x1 = __shfl_xor_sync(act, dx, 8), x2 = __shfl_xor_sync(act, dy, 8);
+  if (em) {
+    a0 = up ? fma(g, dz, x0) : fma(x0, x1, tx);
+    a1 = fma(x0, x2, ty);
+  } else {
+    a0 = up ? x0 : tx;
+    a1 = ty;
+  }
+  int p = 1;
+  for (unsigned bits = em & (em - 1u); bits; bits &= bits - 1, ++p) {
+    g = dx = dy = dz = 0.0;
+    if (up) {
       const int j = __ffs(bits) - 1;
       if (!table && p < TP_PRE) {
         const double *q = wpos + (p * TP_TAB + tab_index(k, m)) * 3;
@@ -605,23 +686,13 @@ __device__ __forceinline__ void tp_force(const Sim &S, const TPSet &T, const Dev
         const double t = (m == 2 * k) ? t0 + H : t0 + m * h;
         planet_at(S, T, P, j, table, k, m, t, i2tau, bx, by, bz);
       }
-      gm = S.gm[j];
-      A = pmin(T.A[i], S.A[j]);
-      cut = umax64(T.rcsq[i], S.rcsq[j]);
-    }
-    double g = 0.0, dx = 0.0, dy = 0.0, dz = 0.0;
-    if (body || (!up && p == 0)) {
       dx = bx - sx; dy = by - sy; dz = bz - sz;
-      const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-      g = bs_factor(r2, gm, A, !up, dbits(r2) < cut, P.kmode);
+      r2 = fma(dz, dz, fma(dy, dy, dx * dx));
+      g = bs_factor(r2, S.gm[j], pmin(T.A[i], S.A[j]), false, dbits(r2) < umax64(T.rcsq[i], S.rcsq[j]), P.kmode);
     }
-    if (p == 0 && !up) { ax = g * dx; ay = g * dy; az = g * dz; }  // the Sun: -G m0 y / |y|^3
-    const double gp = __shfl_xor_sync(act, g, 8), px = __shfl_xor_sync(act, dx, 8),
-                 py = __shfl_xor_sync(act, dy, 8), pz = __shfl_xor_sync(act, dz, 8);
-    if (!bits) break;
-    if (!up) { ax = fma(gp, px, ax); ay = fma(gp, py, ay); az = fma(gp, pz, az); }
-    bits &= bits - 1;
-    if (!bits) break;
+    x0 = __shfl_xor_sync(act, g, 8); x1 = __shfl_xor_sync(act, dx, 8); x2 = __shfl_xor_sync(act, dy, 8);
+    if (up) a0 = fma(g, dz, a0);
+    else { a0 = fma(x0, x1, a0); a1 = fma(x0, x2, a1); }
   }
 }
 
@@ -715,6 +786,10 @@ __global__ void __launch_bounds__(32 * TPB_WARPS, 1) k_tp_bs(Sim S, TPSet T, Dev
     const unsigned em = T.emask[i];
     static_assert(BS_LEVELS == 8, "lanes l16 and l16 + 8 pair up on level (l16 & 7) + 1");
     const int L = (l16 & 7) + 1, nk = 2 * L;
+    const bool up = (lane & 8) != 0;
+    const int oc = up ? 2 : 0, on = up ? 1 : 2;  // this lane's components of its level's chain
+    const TpBody body = tp_body(S, T, P, i, em, up);
+    const double *ptab0 = T.ptab + ((size_t)(em ? __ffs(em) - 1 : 0) * TP_TAB + tab_index(L, 0)) * 6;
     double y[6];
     for (int c = 0; c < 3; ++c) { y[c] = T.x0[c * np + i]; y[3 + c] = T.v0[c * np + i]; }
     double t0 = 0.0, rem = tau, H = tau;
@@ -756,11 +831,13 @@ __global__ void __launch_bounds__(32 * TPB_WARPS, 1) k_tp_bs(Sim S, TPSet T, Dev
         }
         __syncwarp();
       }
-      double za[6], zb[6], ax, ay, az;
-      for (int c = 0; c < 6; ++c) za[c] = y[c];
-      tp_force(S, T, P, i, em, use_tab, L, 0, t0, h, Hl, i2tau, wpos, y, ax, ay, az, 0xffffffffu);
-      zb[0] = fma(h, y[3], y[0]); zb[1] = fma(h, y[4], y[1]); zb[2] = fma(h, y[5], y[2]);
-      zb[3] = fma(h, ax, y[3]); zb[4] = fma(h, ay, y[4]); zb[5] = fma(h, az, y[5]);
+      // the first planet's positions at this lane's midpoints
+      const double *pq = use_tab ? ptab0 : wpos + tab_index(L, 0) * 3;
+      const int pstride = use_tab ? 6 : 3;
+      double xA[2] = {up ? y[2] : y[0], y[1]}, vA[2] = {up ? y[5] : y[3], y[4]}, xB[2], vB[2], ac[2];
+      tp_force(S, T, P, i, em, use_tab, L, 0, t0, h, Hl, i2tau, wpos, body, pq, xA[0], xA[1], ac[0], ac[1], 0xffffffffu);
+#pragma unroll
+      for (int c = 0; c < 2; ++c) { xB[c] = fma(h, vA[c], xA[c]); vB[c] = fma(h, ac[c], vA[c]); }
       // Level L (lane L - 1 of each half) finishes at evaluation 2L; the half's lanes 8..13 then
       // extend its tableau by that row, component c on lane 8 + c (polynomial extrapolation in h^2,
       // Neville), and the first converged level ends that half's attempt: the same decision as
@@ -780,22 +857,30 @@ __global__ void __launch_bounds__(32 * TPB_WARPS, 1) k_tp_bs(Sim S, TPSet T, Dev
       for (int m = 1; m <= 2 * lmax; ++m) {
         const unsigned act = __ballot_sync(0xffffffffu, m <= nk);
         if (m <= nk) {
-          tp_force(S, T, P, i, em, use_tab, L, m, t0, h, Hl, i2tau, wpos, zb, ax, ay, az, act);
+          tp_force(S, T, P, i, em, use_tab, L, m, t0, h, Hl, i2tau, wpos, body, pq + m * pstride, xB[0], xB[1], ac[0], ac[1],
+                   act);
           if (m < nk) {
-            double zn[6];
-            zn[0] = fma(h2, zb[3], za[0]); zn[1] = fma(h2, zb[4], za[1]); zn[2] = fma(h2, zb[5], za[2]);
-            zn[3] = fma(h2, ax, za[3]); zn[4] = fma(h2, ay, za[4]); zn[5] = fma(h2, az, za[5]);
-            for (int c = 0; c < 6; ++c) { za[c] = zb[c]; zb[c] = zn[c]; }
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+              const double xn = fma(h2, vB[c], xA[c]), vn = fma(h2, ac[c], vA[c]);
+              xA[c] = xB[c]; vA[c] = vB[c];
+              xB[c] = xn; vB[c] = vn;
+            }
           }
         }
         if (m & 1) continue;
         const int Lc = m >> 1;
-        // level Lc's lane hands its last midpoint state to the tableau lanes, which form
+        // level Lc's lanes hand their last midpoint state to the tableau lanes, which form
         // T_{Lc,1} = (z_{n-1} + z_n + h z'_n) / 2 one component each
         double *zt = s_zt[half];
-        if (l16 == Lc - 1) {
-          for (int c = 0; c < 6; ++c) { zt[c] = za[c]; zt[6 + c] = zb[c]; }
-          zt[12] = ax; zt[13] = ay; zt[14] = az; zt[15] = h;
+        if ((l16 & 7) == Lc - 1) {
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {
+            if (c >= on) continue;
+            zt[oc + c] = xA[c]; zt[3 + oc + c] = vA[c]; zt[6 + oc + c] = xB[c]; zt[9 + oc + c] = vB[c];
+            zt[12 + oc + c] = ac[c];
+          }
+          if (!up) zt[15] = h;
         }
         __syncwarp();
         double t1 = 0.0;
