@@ -428,58 +428,44 @@ __device__ __forceinline__ void k_and_dk(double r, double A, double &K, double &
   const double y = fma(r, A, -1.0 / 9.0);
   if (is_neg_or_zero(y)) { K = 0.0; dK = 0.0; return; }
   if (dbits(y) >= dbits(1.0)) { K = 1.0; dK = 0.0; return; }
-  const double omy = 1.0 - y, y2 = y * y, o2 = omy * omy, Dn = y2 + o2;
-  K = y2 / Dn;
-  dK = 2.0 * y * omy / (Dn * Dn);
+  const double omy = 1.0 - y, y2 = y * y, iD = rcp_refined(fma(omy, omy, y2));
+  K = y2 * iD;
+  dK = 2.0 * (y * omy) * (iD * iD);
 }
 
-// Adjoint of one pair term of an acceleration field: the pair (i, j) adds m_j g(d) to a_i and
-// -m_i g(d) to a_j, g(d) = G W(r) d/r^3, d = x_j - x_i, W = K (kick, SIGN = +1) or 1 - K (BS,
-// SIGN = -1, only inside rc). Given u_i, u_j (adjoints of a_i, a_j), returns the contribution to
-// xbar_i (xbar_j gets the negative), to mbar_i (from a_j), and to rcbar of the pair.
-template <int SIGN>
-__device__ __forceinline__ void pair_vjp(double dx, double dy, double dz, double gmi, double gmj, double G,
-                                         const double *ui, const double *uj, double Apair, double rcpair,
-                                         bool inside, double *xb, double &mb, double &rcb) {
-  const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-  const double yr = rsqrt_refined(r2), yr2 = yr * yr, yr3 = yr2 * yr;
-  double W, Wr = 0.0, Wrc = 0.0;
-  if (inside) {
-    const double r = r2 * yr;
-    double K, dK;
-    k_and_dk(r, Apair, K, dK);
-    if (SIGN > 0) { W = K; Wr = dK * Apair; Wrc = -dK * (r * Apair) / rcpair; }
-    else { W = 1.0 - K; Wr = -dK * Apair; Wrc = dK * (r * Apair) / rcpair; }
+// r^-3 and r^-5 from r^2, on the integer pipes where r^2 is normal.
+__device__ __forceinline__ void inverse_35(double r2, double &y3, double &y5) {
+  const int ex = (int)(dbits(r2) >> 52);
+  if (ex > 0 && ex < 0x7ff) {
+    fx::inverse_powers(r2, y3, y5);
   } else {
-    W = SIGN > 0 ? 1.0 : 0.0;
+    const double yr = rsqrt_refined(r2);
+    y3 = yr * yr * yr;
+    y5 = y3 * yr * yr;
   }
-  if (dbits(W) == 0ULL && dbits(Wr) == 0ULL) return;
-  const double w0 = gmj * ui[0] - gmi * uj[0], w1 = gmj * ui[1] - gmi * uj[1], w2 = gmj * ui[2] - gmi * uj[2];
-  const double dw = fma(dz, w2, fma(dy, w1, dx * w0));
-  const double c1 = W * yr3, c2 = dw * (Wr * yr2 * yr2 - 3.0 * W * yr3 * yr2);
-  xb[0] -= fma(c1, w0, c2 * dx); xb[1] -= fma(c1, w1, c2 * dy); xb[2] -= fma(c1, w2, c2 * dz);
-  mb -= G * c1 * fma(dz, uj[2], fma(dy, uj[1], dx * uj[0]));
-  rcb += Wrc * yr3 * dw;
 }
 
-// Both sides of one changeover-zone pair of the kick (weight W = K): Jw (xbar_i -= Jw, xbar_j += Jw),
-// the mbar contributions of i (from a_j) and of j (from a_i), and the pair's rcbar.
-__device__ __forceinline__ void pair_vjp_zone(double dx, double dy, double dz, double gmi, double gmj, double G,
-                                              const double *ui, const double *uj, double Apair, double rcpair,
-                                              double *Jw, double &mbi, double &mbj, double &rcbp) {
-  const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-  const double yr = rsqrt_refined(r2), yr2 = yr * yr, yr3 = yr2 * yr;
-  const double r = r2 * yr;
+// Adjoint of one pair term of an acceleration field inside the pair's critical radius: the pair (i, j)
+// adds m_j g(d) to a_i and -m_i g(d) to a_j, g(d) = G W(r) d/r^3, d = x_j - x_i, W = K (kick, SIGN = +1) or
+// 1 - K (BS, SIGN = -1); A = 1/(0.9 rc). Given u_i, u_j (adjoints of a_i, a_j): Jw (xbar_i -= Jw, xbar_j += Jw),
+// c1 = W/r^3 (mbar_i from a_j: -G c1 d.u_j, mbar_j: G c1 d.u_i) and the pair's rcbar. False: nothing.
+template <int SIGN>
+__device__ __forceinline__ bool pair_vjp(double dx, double dy, double dz, double r2, double gmi, double gmj,
+                                         const double *ui, const double *uj, double A, double *Jw, double &c1, double &rcb) {
+  double y3, y5;
+  inverse_35(r2, y3, y5);
+  const double r = r2 * r2 * y3;
   double K, dK;
-  k_and_dk(r, Apair, K, dK);
-  const double W = K, Wr = dK * Apair, Wrc = -dK * (r * Apair) / rcpair;
-  const double w0 = gmj * ui[0] - gmi * uj[0], w1 = gmj * ui[1] - gmi * uj[1], w2 = gmj * ui[2] - gmi * uj[2];
-  const double dw = fma(dz, w2, fma(dy, w1, dx * w0));
-  const double c1 = W * yr3, c2 = dw * (Wr * yr2 * yr2 - 3.0 * W * yr3 * yr2);
+  k_and_dk(r, A, K, dK);
+  const double W = SIGN > 0 ? K : 1.0 - K, Wr = SIGN > 0 ? dK * A : -dK * A;  // dW/dr; dW/drc = -Wr r/rc
+  if (dbits(W) == 0ULL && dbits(Wr) << 1 == 0ULL) return false;
+  const double w0 = fma(gmj, ui[0], -gmi * uj[0]), w1 = fma(gmj, ui[1], -gmi * uj[1]), w2 = fma(gmj, ui[2], -gmi * uj[2]);
+  const double dw = fma(dz, w2, fma(dy, w1, dx * w0)), Wrr = Wr * r;
+  c1 = W * y3;
+  const double c2 = dw * y5 * fma(-3.0, W, Wrr);
   Jw[0] = fma(c1, w0, c2 * dx); Jw[1] = fma(c1, w1, c2 * dy); Jw[2] = fma(c1, w2, c2 * dz);
-  mbi = -G * c1 * fma(dz, uj[2], fma(dy, uj[1], dx * uj[0]));
-  mbj = G * c1 * fma(dz, ui[2], fma(dy, ui[1], dx * ui[0]));
-  rcbp = Wrc * yr3 * dw;
+  rcb = -Wrr * (0.9 * A) * y3 * dw;
+  return true;
 }
 
 // Kick VJP, Newton's third law: every unordered pair once, on 32x32 tile pairs of one system with a
@@ -525,7 +511,7 @@ __device__ __forceinline__ void vjp_acc_shfl(VjpAcc &a, int src) {
 
 // The pair (a, b) with d = x_b - x_a, both sides. The kernel is bound by FP64 issue, 64-76 cycles a warp
 // instruction: r^-3 and r^-5 on the integer pipes (fxforce.cuh) leave 31 of its 41 to
-// a pair. Measured at 64 systems x 256 bodies: 201 -> 159.5 us a kick.
+// a pair. Measured at 64 systems x 256 bodies: 201 -> 159.5 us a kick, 144 with the zone's pairs.
 __device__ __forceinline__ void vjp_pair(const VjpBody &Pa, const VjpBody &Pb, int ia, int ib, double G, bool act,
                                          VjpAcc &aa, VjpAcc &ab) {
   if (!act || !Pa.al || !Pb.al) return;
@@ -533,23 +519,16 @@ __device__ __forceinline__ void vjp_pair(const VjpBody &Pa, const VjpBody &Pb, i
   const double r2 = r2_exact(dx, dy, dz);
   const double ua[3] = {Pa.u0, Pa.u1, Pa.u2}, ub[3] = {Pb.u0, Pb.u1, Pb.u2};
   if (dbits(r2) < umax64(Pa.Q, Pb.Q)) {  // changeover zone (rare): general form
-    double Jw[3], mba, mbb, rcbp;
-    pair_vjp_zone(dx, dy, dz, Pa.gm, Pb.gm, G, ua, ub, pmin(Pa.A, Pb.A), pmax(Pa.rc, Pb.rc), Jw, mba, mbb, rcbp);
-    aa.e0 -= Jw[0]; aa.e1 -= Jw[1]; aa.e2 -= Jw[2]; aa.me += mba;
-    ab.e0 += Jw[0]; ab.e1 += Jw[1]; ab.e2 += Jw[2]; ab.me += mbb;
+    double Jw[3], c1, rcbp;
+    if (!pair_vjp<1>(dx, dy, dz, r2, Pa.gm, Pb.gm, ua, ub, pmin(Pa.A, Pb.A), Jw, c1, rcbp)) return;
+    aa.e0 -= Jw[0]; aa.e1 -= Jw[1]; aa.e2 -= Jw[2]; aa.me -= G * c1 * fma(dz, ub[2], fma(dy, ub[1], dx * ub[0]));
+    ab.e0 += Jw[0]; ab.e1 += Jw[1]; ab.e2 += Jw[2]; ab.me += G * c1 * fma(dz, ua[2], fma(dy, ua[1], dx * ua[0]));
     const bool own_a = dbits(Pa.rc) > dbits(Pb.rc) || (dbits(Pa.rc) == dbits(Pb.rc) && ia < ib);
     if (own_a) aa.rcb += rcbp; else ab.rcb += rcbp;
     return;
   }
   double yr3, yr5;
-  const int ex = (int)(dbits(r2) >> 52);
-  if (ex > 0 && ex < 0x7ff) {
-    fx::inverse_powers(r2, yr3, yr5);
-  } else {
-    const double yr = rsqrt_refined(r2);
-    yr3 = yr * yr * yr;
-    yr5 = yr3 * yr * yr;
-  }
+  inverse_35(r2, yr3, yr5);
   const double dua = fma(dz, ua[2], fma(dy, ua[1], dx * ua[0]));
   const double dub = fma(dz, ub[2], fma(dy, ub[1], dx * ub[0]));
   const double dw = fma(Pb.gm, dua, -Pa.gm * dub);  // d.w with w = Gm_b u_a - Gm_a u_b
@@ -774,22 +753,23 @@ struct LevShared {  // per level (warp)
   double mb[BS_GMAX], rcb[BS_GMAX];           // the level's mbar / rcbar contributions
 };
 
+// The factors of the pulls come from the integer pipes as in the forward BS kernels (fxforce.cuh): the
+// VJP kernels are bound by FP64 issue, 64-76 cycles a warp instruction. With inverse_35 and without
+// divisions in the adjoint of a pair, an evaluation and its adjoint in a group of two take about 90 FP64
+// instructions where they took 180. Measured at 64 systems x 256 bodies: small groups
+// 199 -> 150 us a substep, the kick (whose pairs inside the zone share it) 159.5 -> 144 us.
 __device__ void grp_accel(const GrpShared &G, const double (*cur)[3], int g, int q, double Gm0, double *a) {
   a[0] = a[1] = a[2] = 0.0;
   if (q >= g) return;
   const double xq = cur[q][0], yq = cur[q][1], zq = cur[q][2];
-  const double r2 = fma(zq, zq, fma(yq, yq, xq * xq));
-  const double f = -Gm0 * rcube_refined(r2);
+  const double f = -bs_factor(fma(zq, zq, fma(yq, yq, xq * xq)), Gm0, 0.0, true, false, 0);
   a[0] = f * xq; a[1] = f * yq; a[2] = f * zq;
   for (int p = 0; p < g; ++p) {
     if (p == q) continue;
     const double dx = cur[p][0] - xq, dy = cur[p][1] - yq, dz = cur[p][2] - zq;
     const double pr2 = fma(dz, dz, fma(dy, dy, dx * dx));
     if (dbits(pr2) >= umax64(G.rcsq[q], G.rcsq[p])) continue;
-    const double yr = rsqrt_refined(pr2);
-    double wB, wA;
-    changeover_w(pr2 * yr, pmin(G.A[q], G.A[p]), 0, wB, wA);
-    const double ff = G.gm[p] * wA * (yr * yr * yr);
+    const double ff = bs_factor(pr2, G.gm[p], pmin(G.A[q], G.A[p]), false, true, 0);
     a[0] = fma(ff, dx, a[0]); a[1] = fma(ff, dy, a[1]); a[2] = fma(ff, dz, a[2]);
   }
 }
@@ -803,12 +783,10 @@ __device__ void grp_accel_vjp(const GrpShared &G, const double (*cur)[3], const 
   const double xq = cur[q][0], yq = cur[q][1], zq = cur[q][2];
   const double uq[3] = {fv[q][0], fv[q][1], fv[q][2]};
   {  // central: a = -G m0 x / |x|^3, J = -G m0 (I/r^3 - 3 x x^T / r^5)
-    const double r2 = fma(zq, zq, fma(yq, yq, xq * xq));
-    const double yr = rsqrt_refined(r2), yr3 = yr * yr * yr, yr5 = yr3 * yr * yr;
-    const double xu = fma(zq, uq[2], fma(yq, uq[1], xq * uq[0]));
-    xb[0] -= Gm0 * (uq[0] * yr3 - 3.0 * xq * xu * yr5);
-    xb[1] -= Gm0 * (uq[1] * yr3 - 3.0 * yq * xu * yr5);
-    xb[2] -= Gm0 * (uq[2] * yr3 - 3.0 * zq * xu * yr5);
+    double y3, y5;
+    inverse_35(fma(zq, zq, fma(yq, yq, xq * xq)), y3, y5);
+    const double c1 = Gm0 * y3, c2 = 3.0 * Gm0 * y5 * fma(zq, uq[2], fma(yq, uq[1], xq * uq[0]));
+    xb[0] = fma(c2, xq, -c1 * uq[0]); xb[1] = fma(c2, yq, -c1 * uq[1]); xb[2] = fma(c2, zq, -c1 * uq[2]);
   }
   for (int p = 0; p < g; ++p) {
     if (p == q) continue;
@@ -816,9 +794,10 @@ __device__ void grp_accel_vjp(const GrpShared &G, const double (*cur)[3], const 
     const double pr2 = fma(dz, dz, fma(dy, dy, dx * dx));
     if (dbits(pr2) >= umax64(G.rcsq[q], G.rcsq[p])) continue;
     const double up[3] = {fv[p][0], fv[p][1], fv[p][2]};
-    double rcb_pair = 0.0;
-    pair_vjp<-1>(dx, dy, dz, G.gm[q], G.gm[p], Gc, uq, up, pmin(G.A[q], G.A[p]), pmax(G.rc[q], G.rc[p]), true, xb,
-                 mb, rcb_pair);
+    double Jw[3], c1, rcb_pair;
+    if (!pair_vjp<-1>(dx, dy, dz, pr2, G.gm[q], G.gm[p], uq, up, pmin(G.A[q], G.A[p]), Jw, c1, rcb_pair)) continue;
+    xb[0] -= Jw[0]; xb[1] -= Jw[1]; xb[2] -= Jw[2];
+    mb -= Gc * c1 * fma(dz, up[2], fma(dy, up[1], dx * up[0]));
     const bool own = dbits(G.rc[q]) > dbits(G.rc[p]) || (dbits(G.rc[q]) == dbits(G.rc[p]) && q < p);
     if (own) rcb += rcb_pair;
   }
