@@ -105,7 +105,6 @@ struct BsPairShared {
   double yn[2][2][6];                 // [warp] result of the warp's attempt
   double pos[2][2][BS_LEVELS][2][3];  // [warp][buffer][level][member]
   double zt[2][BS_LEVELS][2][16];     // [warp] a level's last midpoint state: z_{n-1}, z_n, a(z_n), h
-  u64 err[2][BS_LEVELS];              // [warp]
   int acc[2];
   int gidx;
   double U;
@@ -138,10 +137,10 @@ __device__ int pair_attempt(BsPairShared &sh, int w, const DevParams &P, double 
     const double s2 = fma(yq[2], yq[2], fma(yq[1], yq[1], yq[0] * yq[0]));
     scale = dbits(s2) == 0ULL ? 4.49423283715579e307 : rsqrt_refined(s2);
   }
-  if (lane < BS_LEVELS) sh.err[w][lane] = 0ULL;
   __syncwarp();
   double ac[3];
-  bs_accel(sh, P, Gm0, g, qq, sub, 2, sh.pos[w][0][lev], qa, ac);
+  const BsTerm t0 = bs_term(sh, Gm0, g, qq, sub);
+  bs_accel(sh, P, t0, Gm0, g, qq, sub, 2, sh.pos[w][0][lev], qa, ac);
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
     xB[k] = qa ? fma(h, vA[k], xA[k]) : xA[k];
@@ -159,7 +158,7 @@ __device__ int pair_attempt(BsPairShared &sh, int w, const DevParams &P, double 
         if (k < on) sh.pos[w][b][lev][q][oc + k] = xB[k];
     }
     __syncwarp();
-    bs_accel(sh, P, Gm0, g, qq, sub, 2, sh.pos[w][b][lev], qa && e <= nk, ac);
+    bs_accel(sh, P, t0, Gm0, g, qq, sub, 2, sh.pos[w][b][lev], qa && e <= nk, ac);
     if (lv) {
       // the level's chain is done: its tableau lanes form T_{L,1} = (z_{n-1} + z_n + h z'_n) / 2,
       // one component each, so the warp issues that arithmetic once instead of per level lane
@@ -186,16 +185,16 @@ __device__ int pair_attempt(BsPairShared &sh, int w, const DevParams &P, double 
     if (e & 1) continue;
     const int Lc = e >> 1;  // level Lc is complete: its tableau row (Neville, in h^2)
     __syncwarp();
+    bool bad = false;
     if (rowth) {
       const double *z = sh.zt[w][Lc - 1][qc];
       const double dz = cc < 3 ? z[9 + cc] : z[12 + cc - 3];  // derivative of component cc at z_n
       const double t1 = sh.alive[qc] ? 0.5 * fma(z[15], dz, z[6 + cc] + z[cc]) : z[cc];
       double before;
       tlast = neville_row(t1, Lc, [&](int j) { return c_facinv[Lc][j]; }, prev, before);
-      if (Lc >= 2 && sh.alive[qc]) atomicMax(&sh.err[w][Lc - 1], absbits((tlast - before) * scale));
+      bad = sh.alive[qc] && absbits((tlast - before) * scale) > eps;
     }
-    __syncwarp();
-    if (Lc >= 2 && sh.err[w][Lc - 1] <= eps) { acc = Lc; break; }
+    if (!__any_sync(0xffffffffu, bad) && Lc >= 2) { acc = Lc; break; }
   }
   if (acc && rowth) sh.yn[w][qc][cc] = tlast;  // the accepted row is the last one built
   __syncwarp();

@@ -46,7 +46,7 @@ struct BsClShared {
   int cnt[2];                            // pairs listed, by evaluation
   unsigned short pair[CL_PAIRS];         // the listed pairs i << 8 | j, i < j
   double T1[2][BS_GMAX][6];              // this level's result, double-buffered by attempt
-  u64 err[BS_LEVELS];
+  unsigned bad;                          // bit r - 1: level r has not converged
   unsigned char cont[BS_GMAX * (BS_GMAX - 1) / 2];
   double H, rem, U;
   int accept, nseq;
@@ -190,7 +190,7 @@ __global__ void __cluster_dims__(CL_SIZE, 1, 1) __launch_bounds__(CL_THREADS, 2)
       if (act) { sh.pos[0][q][c] = xA; sh.fp[0][q][c] = cl_float(xA); }
       const int qc = tid / 6, cc = tid % 6;
       const bool rowth = qc < g;
-      if (tid < BS_LEVELS) sh.err[tid] = 0ULL;
+      if (tid == 0) sh.bad = 0u;
       __syncthreads();
       double acc_c = cl_eval(sh, P, Gm0, g, sh.pos[0], sh.fp[0], par, q, c);
       if (qa) {
@@ -232,19 +232,19 @@ __global__ void __cluster_dims__(CL_SIZE, 1, 1) __launch_bounds__(CL_THREADS, 2)
 #pragma unroll
         for (int r = 1; r <= BS_LEVELS; ++r) {
           if (r < r0 || r > Lc) continue;  // uniform
-          u64 ev = 0ULL;
+          bool bad = false;
           if (rowth) {
             const double *rt = cluster.map_shared_rank(&sh.T1[buf][0][0], (unsigned)(r - 1));
             double before;
             tlast = neville_row(rt[qc * 6 + cc], r, [&](int j) { return c_facinv_cl[r][j]; }, prev, before);
-            if (r >= 2 && sh.alive[qc]) ev = absbits((tlast - before) * scale);
+            if (r >= 2 && sh.alive[qc]) bad = absbits((tlast - before) * scale) > eps;
             if (r <= CL_FIRST_CHECK) tk[r] = tlast;
           }
-          if (r >= 2) warp_max_to(&sh.err[r - 1], ev);
+          if (r >= 2) warp_flag(&sh.bad, 1u << (r - 1), bad);
         }
         __syncthreads();
-        for (int r = r0 < 2 ? 2 : r0; r <= Lc; ++r)  // uniform: every thread reads the same errors
-          if (sh.err[r - 1] <= eps) { acc = r; break; }
+        for (int r = r0 < 2 ? 2 : r0; r <= Lc; ++r)  // uniform: every thread reads the same bits
+          if (!((sh.bad >> (r - 1)) & 1u)) { acc = r; break; }
         if (acc) {
           if (acc < Lc && rowth) tlast = tk[acc];
           break;

@@ -31,7 +31,7 @@ struct BsSharedT {
   double y[GM][6], yn[GM][6];
   double pos[2][BS_LEVELS][GM][3];
   double tab[BS_LEVELS][GM][6];
-  u64 err[BS_LEVELS], err2[BS_LEVELS];  // per level: the attempt at H, the speculative one at H/2
+  unsigned bad;                         // not converged: bit r - 1 level r of the attempt at H, 7 + r of that at H/2
   unsigned char cont[GM * (GM - 1) / 2];
   double H, rem, U;
   int accept, next;
@@ -51,9 +51,29 @@ using BsShared = BsSharedT<BS_GMAX>;
 // instruction costs its sub-partition 64 cycles whatever its active lanes. The threads exchange what
 // they do not own, so a slot of 4 issues 3 additions for the sum and 4 instructions for its chain
 // step, where every thread holding every component took 6 and 6.
+//
+// What a term of member q and partner p (p == q: the central mass) takes besides their positions; the
+// thread's first one is formed once an attempt.
+struct BsTerm {
+  fx::Num gm, A;  // G m and 1/(0.9 rc) for the fixed-point factor
+  u64 cut;        // r^2 below it: inside the critical radius
+  int sign;       // the sign bit of G m
+};
 template <class SH>
-__device__ __forceinline__ void bs_accel(const SH &sh, const DevParams &P, double Gm0, int g, int q, int tsub, int ttps,
-                                         const double (*pos)[3], bool q_alive, double (&acc)[3]) {
+__device__ __forceinline__ BsTerm bs_term(const SH &sh, double Gm0, int g, int q, int p) {
+  BsTerm t;
+  p = p < g ? p : q;
+  const bool cen = p == q;
+  const double gm = cen ? Gm0 : sh.gm[p];
+  t.gm = fx::num(gm);
+  t.A = fx::num(pmin(sh.A[q], sh.A[p]));
+  t.cut = !cen && sh.alive[p] ? umax64(sh.rcsq[q], sh.rcsq[p]) : 0ULL;
+  t.sign = __double2hiint(gm) & 0x80000000;
+  return t;
+}
+template <class SH>
+__device__ __forceinline__ void bs_accel(const SH &sh, const DevParams &P, const BsTerm &t0, double Gm0, int g, int q, int tsub,
+                                         int ttps, const double (*pos)[3], bool q_alive, double (&acc)[3]) {
   double a0 = 0.0, a1 = 0.0, a2 = 0.0;
   if (q_alive) {
     const double xq = pos[q][0], yq = pos[q][1], zq = pos[q][2];
@@ -62,8 +82,18 @@ __device__ __forceinline__ void bs_accel(const SH &sh, const DevParams &P, doubl
       const double dx = (cen ? 0.0 : pos[p][0]) - xq, dy = (cen ? 0.0 : pos[p][1]) - yq,
                    dz = (cen ? 0.0 : pos[p][2]) - zq;
       const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
-      const bool inside = sh.alive[p] && dbits(r2) < umax64(sh.rcsq[q], sh.rcsq[p]);
-      const double f = bs_factor(r2, cen ? Gm0 : sh.gm[p], pmin(sh.A[q], sh.A[p]), cen, inside, P.kmode);
+      BsTerm t = t0;
+      if (p != tsub) t = bs_term(sh, Gm0, g, q, p);
+      const bool inside = dbits(r2) < t.cut;
+      double f = 0.0;
+      if (cen || inside) {
+        if (P.kmode == 0) {
+          f = fx::pull_factor(r2, t.gm, t.A, cen, inside);
+          f = __hiloint2double(__double2hiint(f) | t.sign, __double2loint(f));
+        } else {
+          f = bs_factor_gradient(r2, cen ? Gm0 : sh.gm[p], pmin(sh.A[q], sh.A[p]), cen);
+        }
+      }
       a0 = fma(f, dx, a0); a1 = fma(f, dy, a1); a2 = fma(f, dz, a2);
     }
   }
@@ -164,12 +194,13 @@ __device__ void bs_group(BsSharedT<GM> &sh, const Sim &S, const DevParams &P, do
       const double s2 = fma(yq[2], yq[2], fma(yq[1], yq[1], yq[0] * yq[0]));
       scale = dbits(s2) == 0ULL ? 4.49423283715579e307 : rsqrt_refined(s2);
     }
-    if (tid < BS_LEVELS) { sh.err[tid] = 0ULL; sh.err2[tid] = 0ULL; }
+    if (tid == 0) sh.bad = 0u;
     __syncthreads();
     double ac[3] = {0.0, 0.0, 0.0};
+    const BsTerm t0 = bs_term(sh, Gm0, g, q, tsub);
     // every lane of a warp that holds any active slot takes part (the sums shuffle across lanes);
     // warps without active slots stay off the pipes
-    if (__any_sync(0xffffffffu, acta)) bs_accel(sh, P, Gm0, g, q, tsub, ttps, sh.pos[0][lev] + 16 * half, qa, ac);
+    if (__any_sync(0xffffffffu, acta)) bs_accel(sh, P, t0, Gm0, g, q, tsub, ttps, sh.pos[0][lev] + 16 * half, qa, ac);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       if (k >= on) continue;
@@ -189,7 +220,7 @@ __device__ void bs_group(BsSharedT<GM> &sh, const Sim &S, const DevParams &P, do
           if (k < on) sh.pos[b][lev][qm][oc + k] = xB[k];
       }
       __syncthreads();
-      if (__any_sync(0xffffffffu, lv)) bs_accel(sh, P, Gm0, g, q, tsub, ttps, sh.pos[b][lev] + 16 * half, qa, ac);
+      if (__any_sync(0xffffffffu, lv)) bs_accel(sh, P, t0, Gm0, g, q, tsub, ttps, sh.pos[b][lev] + 16 * half, qa, ac);
       if (lv) {
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
@@ -211,19 +242,19 @@ __device__ void bs_group(BsSharedT<GM> &sh, const Sim &S, const DevParams &P, do
       // level Lc = e/2 is complete: its tableau row (polynomial extrapolation in h^2, Neville)
       const int Lc = e >> 1;
       __syncthreads();
-      u64 ev = 0ULL;
+      bool bad = false;
       if (rowth) {
         double before;
         tlast = neville_row(sh.tab[Lc - 1][qc + 16 * thalf][cc], Lc, [&](int j) { return c_facinv[Lc][j]; }, prev, before);
-        if (Lc >= 2 && sh.alive[qc]) ev = absbits((tlast - before) * scale);
+        if (Lc >= 2 && sh.alive[qc]) bad = absbits((tlast - before) * scale) > eps;
       }
-      if (Lc >= 2) warp_max_to(thalf ? &sh.err2[Lc - 1] : &sh.err[Lc - 1], ev);  // thalf is uniform per warp
+      if (Lc >= 2) warp_flag(&sh.bad, 1u << (Lc - 1 + 8 * thalf), bad);  // thalf is uniform per warp
       __syncthreads();
-      if (specn && !accB && Lc >= 2 && sh.err2[Lc - 1] <= eps) {  // the attempt at H/2 converged (uniform)
+      if (specn && !accB && Lc >= 2 && !((sh.bad >> (Lc + 7)) & 1u)) {  // the attempt at H/2 converged (uniform)
         accB = Lc;
         if (thalf && rowth) sh.yn[qc + 16][cc] = tlast;
       }
-      if (Lc >= 2 && sh.err[Lc - 1] <= eps) { acc = Lc; break; }  // uniform: every thread reads the same error
+      if (Lc >= 2 && !((sh.bad >> (Lc - 1)) & 1u)) { acc = Lc; break; }  // uniform: every thread reads the same bits
     }
     if (acc && rowth && !thalf) sh.yn[qc][cc] = tlast;  // the accepted row is the last one built
     double Hs = H;  // length of the accepted substep

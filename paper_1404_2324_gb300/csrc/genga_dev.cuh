@@ -589,15 +589,11 @@ __device__ __forceinline__ void merger_report(const Sim &S, int ia, int ib, cons
   }
 }
 
-// Largest v over the warp into *dst (shared memory; one atomic per warp instead of one per thread,
-// which serialised on the single address). All 32 lanes call it; v = 0 adds nothing.
-__device__ __forceinline__ void warp_max_to(u64 *dst, u64 v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const u64 t = __shfl_xor_sync(0xffffffffu, v, o);
-    v = t > v ? t : v;
-  }
-  if ((threadIdx.x & 31) == 0 && v) atomicMax((unsigned long long *)dst, (unsigned long long)v);
+// Sets bits of *dst (shared) where f holds on any lane. The convergence test of the BS kernels: one bit
+// per level says that an error exceeds the tolerance (a maximum of the errors takes ten shuffles and a
+// 64-bit atomic).
+__device__ __forceinline__ void warp_flag(unsigned *dst, unsigned bits, bool f) {
+  if (__any_sync(0xffffffffu, f) && (threadIdx.x & 31) == 0) atomicOr(dst, bits);
 }
 
 // First statement of a kernel launched by launch_after: waits until every kernel before it has finished
