@@ -163,6 +163,7 @@ struct genga_ctx {
   cudaStream_t side = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   int gsplit = BS_GMAX + 1, cl_grid = 0, pair_grid = 0;
+  bool roomy = false;  // the BS kernels may take an SM per CTA (bs.cu)
   // a further branch: groups above BS_GMAX members (main mode; the larger batched groups too)
   cudaStream_t side2 = nullptr;
   cudaEvent_t ev_join2 = nullptr;
@@ -282,10 +283,10 @@ void enqueue_step_batch(genga_ctx *c, cudaStream_t st) {
       cudaEventRecord(c->ev_fork, st);
       cudaStreamWaitEvent(c->side, c->ev_fork, 0);
       cudaStreamWaitEvent(c->side2, c->ev_fork, 0);
-      launch_bs_pair(S, P, tau, c->pair_grid, c->side);
-      launch_bs(S, P, tau, c->bs_grid, c->side2, BS_GMAX + 1, 3);  // and the groups of 3..BS_SMALL expected to be long
+      launch_bs_pair(S, P, tau, c->pair_grid, c->side, c->roomy);
+      launch_bs(S, P, tau, c->bs_grid, c->side2, BS_GMAX + 1, 3, false, c->roomy);  // and the groups of 3..BS_SMALL expected to be long
       launch_bs_wide(S, P, tau, c->wide_grid, c->side2);  // queue 3: groups above BS_GMAX members
-      launch_bs_small(S, P, tau, c->small_grid, st);
+      launch_bs_small(S, P, tau, c->small_grid, st, c->roomy);
       cudaEventRecord(c->ev_join, c->side);
       cudaEventRecord(c->ev_join2, c->side2);
       cudaStreamWaitEvent(st, c->ev_join, 0);
@@ -338,7 +339,7 @@ void enqueue_step(genga_ctx *c, cudaStream_t st) {
       cudaStreamWaitEvent(c->side2, c->ev_fork, 0);
       launch_bs_cluster(S, P, tau, c->gsplit, c->cl_grid, c->side);
       launch_bs_grid(S, P, tau, BS_GMAX + 1, c->grid_blocks, c->side2);
-      launch_bs(S, P, tau, c->bs_grid, st, c->gsplit, 1, true);
+      launch_bs(S, P, tau, c->bs_grid, st, c->gsplit, 1, true, c->roomy);
       cudaEventRecord(c->ev_join, c->side);
       cudaEventRecord(c->ev_join2, c->side2);
       cudaStreamWaitEvent(st, c->ev_join, 0);
@@ -498,6 +499,7 @@ int genga_init(genga_ctx **out, int n, const double *masses, const double *radii
     genga_free(c);
     return GENGA_ECUDA;
   }
+  c->roomy = c->n <= 608;
   c->gsplit = 5;  // measured: from 5 members on, a cluster per group beats one CTA per group
   c->cl_grid = bs_cluster_grid();
   bs_grid_init_constants();
@@ -702,6 +704,7 @@ static int init_batch_one(genga_ctx **out, int n_sys, const int *offsets, const 
   // the pair kernel (4 groups per CTA) takes one CTA per SM, which leaves the other register half of
   // every SM to k_bs from the start: at two per SM it held the whole GPU and k_bs, the longer branch,
   // began 0.5 ms later (measured: 3.06M -> 3.15M system-steps/s)
+  c->roomy = true;
   c->pair_grid = num_sms();
   // groups of 3..BS_SMALL members (most of those above pairs) on 128-thread CTAs: two fit beside a
   // pair CTA in the register file where one 256-thread CTA did; the few larger groups take a half grid
@@ -889,6 +892,7 @@ int genga_init_batch(genga_ctx **out, int n_sys, const int *offsets, const doubl
   if (e1) cudaEventDestroy(e1);
   for (genga_ctx *p : c->parts) {
     // the parts' BS kernels run side by side: each part a share of the grids one batch would use
+    p->roomy = false;
     p->pair_grid = std::max(8, 2 * p->pair_grid / K);
     p->small_grid = std::max(16, 2 * p->small_grid / K);
     p->bs_grid = std::max(8, 2 * p->bs_grid / K);

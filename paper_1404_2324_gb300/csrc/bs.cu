@@ -29,8 +29,13 @@ __device__ __forceinline__ int batch_group(const Sim &S, int qi, int q) {
 // shared memory). The kernel integrates the groups of gmin .. gsplit - 1 members that it meets and
 // reports larger ones than GM; it takes its groups from batched queue qi, else from the
 // large-group list (from_big), else every group with a fixed stride.
-template <int NT, int GM>
-__global__ void __launch_bounds__(NT, NT >= 512 ? 1 : 512 / NT)
+// MINB: CTAs per SM that the registers are shared out for. Two 256-thread CTAs (128 registers a
+// thread) spill some 60 bytes in the chain of evaluations; where every group finds an SM of its own
+// (`roomy`: one system of at most 608 bodies, a batch in one part) one CTA per SM without spills is
+// faster: 10 steps of 500 bodies 884 -> 858 us, 300 systems x 4 steps 2149 -> 2071 us; not beyond (2048
+// bodies at fourth order 1677 -> 1856 us, 8192 systems 6.78 -> 7.19 ms).
+template <int NT, int GM, int MINB>
+__global__ void __launch_bounds__(NT, MINB)
     k_bs(Sim S, DevParams P, double tau, int gmin, int gsplit, int qi, int from_big) {
   __shared__ __align__(16) unsigned char bs_static[GM <= BS_GMAX ? sizeof(BsSharedT<GM>) : 16];
   extern __shared__ __align__(16) unsigned char bs_dyn[];
@@ -65,22 +70,24 @@ __global__ void __launch_bounds__(NT, NT >= 512 ? 1 : 512 / NT)
 static_assert(BS_WIDE_THREADS == BS_LEVELS * BS_GWIDE, "one thread per (level, member) slot");
 
 void bs_init_constants() {
-  cudaFuncSetAttribute(k_bs<BS_WIDE_THREADS, BS_GWIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaFuncSetAttribute(k_bs<BS_WIDE_THREADS, BS_GWIDE, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (int)sizeof(BsSharedT<BS_GWIDE>));
   bs_core_set_factors();
 }
 
 void launch_bs(const Sim &S, const DevParams &P, double tau, int max_groups, cudaStream_t st, int gsplit, int gmin,
-               bool after) {
+               bool after, bool roomy) {
   const int grid = max_groups < 1 ? 1 : max_groups;
-  if (after) launch_after(k_bs<BS_THREADS, BS_GMAX>, grid, BS_THREADS, st, S, P, tau, gmin, gsplit, 2, 0);
-  else k_bs<BS_THREADS, BS_GMAX><<<grid, BS_THREADS, 0, st>>>(S, P, tau, gmin, gsplit, 2, 0);
+  auto *kernel = roomy ? k_bs<BS_THREADS, BS_GMAX, 1> : k_bs<BS_THREADS, BS_GMAX, 2>;
+  if (after) launch_after(kernel, grid, BS_THREADS, st, S, P, tau, gmin, gsplit, 2, 0);
+  else kernel<<<grid, BS_THREADS, 0, st>>>(S, P, tau, gmin, gsplit, 2, 0);
 }
-void launch_bs_small(const Sim &S, const DevParams &P, double tau, int blocks, cudaStream_t st) {
-  k_bs<128, BS_GMAX><<<blocks < 1 ? 1 : blocks, 128, 0, st>>>(S, P, tau, 3, BS_SMALL + 1, 1, 0);
+void launch_bs_small(const Sim &S, const DevParams &P, double tau, int blocks, cudaStream_t st, bool roomy) {
+  auto *kernel = roomy ? k_bs<128, BS_GMAX, 3> : k_bs<128, BS_GMAX, 4>;
+  kernel<<<blocks < 1 ? 1 : blocks, 128, 0, st>>>(S, P, tau, 3, BS_SMALL + 1, 1, 0);
 }
 void launch_bs_wide(const Sim &S, const DevParams &P, double tau, int blocks, cudaStream_t st) {
-  k_bs<BS_WIDE_THREADS, BS_GWIDE><<<blocks < 1 ? 1 : blocks, BS_WIDE_THREADS, sizeof(BsSharedT<BS_GWIDE>), st>>>(
+  k_bs<BS_WIDE_THREADS, BS_GWIDE, 1><<<blocks < 1 ? 1 : blocks, BS_WIDE_THREADS, sizeof(BsSharedT<BS_GWIDE>), st>>>(
       S, P, tau, BS_GMAX + 1, 0x7fffffff, 3, 1);
 }
 
@@ -201,7 +208,8 @@ __device__ int pair_attempt(BsPairShared &sh, int w, const DevParams &P, double 
   return acc;
 }
 
-__global__ void __launch_bounds__(64 * BSP_UNITS, 2) k_bs_pair(Sim S, DevParams P, double tau) {
+template <int MINB>  // as k_bs
+__global__ void __launch_bounds__(64 * BSP_UNITS, MINB) k_bs_pair(Sim S, DevParams P, double tau) {
   __shared__ BsPairShared shu[BSP_UNITS];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, unit = wid >> 1, spec = wid & 1;
   const int bar = 1 + unit;
@@ -317,8 +325,9 @@ __global__ void __launch_bounds__(64 * BSP_UNITS, 2) k_bs_pair(Sim S, DevParams 
   }
 }
 
-void launch_bs_pair(const Sim &S, const DevParams &P, double tau, int blocks, cudaStream_t st) {
-  k_bs_pair<<<blocks, 64 * BSP_UNITS, 0, st>>>(S, P, tau);
+void launch_bs_pair(const Sim &S, const DevParams &P, double tau, int blocks, cudaStream_t st, bool roomy) {
+  auto *kernel = roomy ? k_bs_pair<1> : k_bs_pair<2>;
+  kernel<<<blocks, 64 * BSP_UNITS, 0, st>>>(S, P, tau);
 }
 
 }  // namespace genga
