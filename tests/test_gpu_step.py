@@ -220,3 +220,18 @@ def test_profiling_events_and_launch_count():
         assert n == nsub and 0.0 < ms < 50.0
         genga.genga_set_profiling(s.ctx, False)
         s.close()
+
+
+@pytest.mark.parametrize("n", [20, 60, 100, 200, 250, 300])
+def test_grouping_by_one_warp_and_by_the_cta(n):
+    """A step of ever denser rings, from no encounter pair over 53 and 78 (one warp groups up to 64) to
+    103: pairs, groups and BS substeps are the oracle's, and the state within the one-step bound."""
+    d = ics._disk(np.random.default_rng(n), n, 1e-9, 1e-8, 0.95, 1.25, 0.01, 0.002)
+    g, o = pair_sims(dict(d, dt=6.0), 2, steps=1)
+    err, same = rel_state_error(g, o)
+    assert same and err <= 1e-12, err
+    np.testing.assert_array_equal(g.encounters(0), o.encounters(0) + 1)
+    _, cnt = g.status()
+    st = o.stats()
+    assert (cnt["encounters"], cnt["groups"], cnt["bs_steps"]) == (st["encounters"], st["groups"], st["bs_steps"])
+    g.close()
