@@ -18,7 +18,7 @@ OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT, "libgenga.so")
 SOURCES = ["kick.cu", "step.cu", "bs.cu", "bs_cluster.cu", "bs_grid.cu", "io.cu", "batch.cu", "batch_persist.cu", "tp.cu", "eject.cu", "adjoint.cu", "api.cu",
            "noalloc.cu"]
-HEADERS = ["genga_dev.cuh", "genga_launch.h", "bs_core.cuh", "fxpair.cuh", "fxforce.cuh", "kick_fx.cuh"]
+HEADERS = ["genga_dev.cuh", "genga_launch.h", "bs_core.cuh", "fxpair.cuh", "fxforce.cuh", "fxmath.cuh", "kick_fx.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ARCH + ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xptxas", "-v"]
 

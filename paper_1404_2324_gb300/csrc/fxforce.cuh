@@ -15,35 +15,13 @@
 //   y = r A - 1/9 clamped to [0, 1], W_A = (1 - y)^2 / (y^2 + (1 - y)^2) with the reciprocal from its
 //   single-precision seed s: s (1 + e' + e'^2), e' = 1 - s (y^2 + (1 - y)^2)
 #pragma once
-#include "fxpair.cuh"
+#include "fxmath.cuh"
 #ifdef __CUDACC__
 #include "genga_dev.cuh"
 #endif
 
 namespace genga {
 namespace fx {
-
-// upper half of the product of two 64-bit numbers, to one unit; the cross products must not carry
-// out of 64 bits together (one factor below 2^63 suffices when the other is, too, and one high word
-// is below 2^31)
-FX_HD u64 mulhi(u64 a, u64 b) {
-  const u64 c = madu(hi32(a), lo32(b), mulu(lo32(a), hi32(b)));
-  return madu(hi32(a), hi32(b), pair64(hi32(c), 0u));
-}
-FX_HD u64 mul32(u64 a, u32 b) {  // (a b) >> 32
-  return madu(hi32(a), b, pair64(hi32(mulu(lo32(a), b)), 0u));
-}
-FX_HD u64 sqrhi(u64 a) {  // (a^2) >> 64, a <= 2^63
-  const u64 c = mulu(hi32(a), lo32(a));
-  return madu(hi32(a), hi32(a), c >> 31);
-}
-FX_HD int clz64(u64 a) {
-#ifdef __CUDA_ARCH__
-  return __clzll((i64)a);
-#else
-  return a ? __builtin_clzll(a) : 64;
-#endif
-}
 
 // A positive double's mantissa in [2^62, 2^63) and exponent: x = M 2^(me - 63); zero: M = 0.
 struct Num {
@@ -85,17 +63,6 @@ FX_HD u64 factor(u64 R, float rho2, int k, const Num &pref, const Num &A, bool f
     w = mulhi(mul32(oo, S), H) << 4;
   }
   return mulhi(mulhi(Y3 << 1, w), pref.M);
-}
-
-// z 2^ex as a double (round to nearest; z > 0 or 0).
-FX_HD double to_double(u64 z, int ex) {
-  if (z == 0ULL) return 0.0;
-  const int lz = clz64(z);
-  z <<= lz;
-  const u64 m = (z + 0x400ULL) >> 11;                           // 53 bits (2^53 carries into the exponent)
-  const int be = 1023 + 63 - lz + ex;
-  if (be <= 0 || be >= 0x7fe || z + 0x400ULL < z) return be <= 0 ? 0.0 : scalbn((double)(z >> 1), ex - lz + 1);
-  return u2d(m + ((u64)(be - 1) << 52));
 }
 
 // pref w / r^3 for r2 > 0 (normal); full, zone as in factor.

@@ -9,6 +9,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "fxmath.cuh"
+
 namespace genga {
 
 typedef unsigned long long u64;
@@ -438,9 +440,10 @@ __device__ __forceinline__ void stumpff_d(double z, double &c0, double &c1, doub
 // reaches its root to (1e-6)^3. The U_k at s + delta follow from dU0/ds = -beta U1, dU_k/ds = U_(k-1)
 // by their Taylor series to second order (the third is below 1e-19 of them), with the second-order
 // terms and the Halley factor in single precision (they are below 1e-11 and 1e-6 of what they correct).
-// One FP64 evaluation of the Stumpff series instead of two or three: about 85 FP64 instructions a
-// drift against 135 (an FP64 instruction holds the sub-partition 64-76 cycles, and the drift kernels
-// are bound by their number). Measured for 200003 bodies: 73.8 -> 53.7 us a call of the phase entry.
+// One evaluation of the Stumpff series instead of two or three, in fixed point on the integer pipes
+// (fxmath.cuh), as 1/r0: about 68 FP64 instructions a drift (an FP64 instruction holds the sub-partition
+// 64-76 cycles, and the drift kernels are bound by their number) where Newton's iteration took 135. Measured for
+// 200003 bodies: 73.8 -> 53.7 us a call of the phase entry with the series in FP64, 45.9 us now.
 // A solution that the single-precision solve does not reach, or a step above 10^-6 of s, takes the
 // iteration in double precision: Newton steps until |ds| <= 4 ulp |s| or a tiny step stops shrinking
 // (rounding floor). Returns 0 on success, 1 when no convergence (state untouched).
@@ -473,8 +476,14 @@ static __device__ int kepler_drift_dev(double mu, double mu2, double &x, double 
                                 double &vy, double &vz, double dt, int maxit, int *iters_out,
                                 double *s_out = nullptr) {
   const double r0sq = fma(z, z, fma(y, y, x * x));
-  const double ir0 = rsqrt_refined(r0sq);
-  const double r0 = r0sq * ir0;
+  double ir0, r0;
+  const int ex = (int)(dbits(r0sq) >> 52);
+  if (ex > 0 && ex < 0x7ff) {
+    fx::inverse_root(r0sq, ir0, r0);
+  } else {
+    ir0 = rsqrt_refined(r0sq);
+    r0 = r0sq * ir0;
+  }
   const double v2 = fma(vz, vz, fma(vy, vy, vx * vx));
   const double u = fma(z, vz, fma(y, vy, x * vx));
   const double beta = fma(mu2, ir0, -v2);
@@ -500,7 +509,9 @@ static __device__ int kepler_drift_dev(double mu, double mu2, double &x, double 
     const double sd = f2d_exact(s);
     const double s2 = sd * sd;
     double c0, c1, c2, c3;
-    stumpff_d(beta * s2, c0, c1, c2, c3);
+    const double z = beta * s2;
+    if (absbits(z) <= dbits(0.4)) fx::stumpff(z, c0, c1, c2, c3);
+    else stumpff_d(z, c0, c1, c2, c3);
     U0 = c0; U1 = sd * c1; U2 = s2 * c2; U3 = s2 * (sd * c3);
     const double F = fma(r0, U1, fma(u, U2, fma(mu, U3, -dt)));
     const double Fp = fma(r0, U0, fma(u, U1, mu * U2));

@@ -313,3 +313,28 @@ def test_energy_matches_oracle():
     ref = O.energy(p, d["m"], alive, d["x"], d["v"])
     E = genga.genga_phase_energy(n, d["G"], d["m0"], dev(d["m"]), dev(alive), soa(d["x"]), soa(d["v"]))
     assert E == pytest.approx(ref, rel=1e-13)
+
+
+@pytest.mark.parametrize("dt", [6.0, -6.0])
+def test_kepler_drift_around_the_limit_of_its_series(dt):
+    """Orbits whose universal argument z = beta s^2 crosses 0.4 (the fixed-point Stumpff series below,
+    the reduced one above), on the bound and the unbound side, through z = 0 (parabolic): the drift
+    test's bound."""
+    G, n = 0.01720209895 ** 2, 400
+    a = np.cbrt(G * dt ** 2 / np.linspace(0.36, 0.44, 160))             # circular: z = (dt n)^2
+    r = np.concatenate([a, np.full(240, 0.25)])
+    vc = np.sqrt(G / r)
+    v = np.where(np.arange(n) < 160, vc, vc * np.sqrt(2.0) * np.linspace(0.9, 2.2, n))  # to hyperbolic
+    v[300] = vc[300] * np.sqrt(2.0)
+    ph = np.linspace(0, 6, n)
+    x = np.stack([r * np.cos(ph), r * np.sin(ph), 0.02 * r], 1)
+    w = np.stack([-v * np.sin(ph), v * np.cos(ph), 0.01 * v], 1)
+    X, V, fail = soa(x), soa(w), dev(np.zeros(n, np.int32))
+    genga.genga_phase_kepler(n, G, dt, 30, dev(np.ones(n, np.int32)), X, V, fail)
+    assert fail.cpu().numpy().sum() == 0
+    gx, gv = aos(X), aos(V)
+    for i in range(n):
+        rx, rv, st, _ = O.kepler_drift(G, x[i], w[i], dt)
+        assert st == 0
+        assert np.linalg.norm(gx[i] - rx) <= 1e-13 * np.linalg.norm(rx), i
+        assert np.linalg.norm(gv[i] - rv) <= 1e-13 * np.linalg.norm(rv), i
