@@ -8,8 +8,8 @@
 // (distributed shared memory), extends its own copy of the Neville tableau and tests level Lc, with
 // the same arithmetic and order in every CTA. Each pair is evaluated once (Newton's third law); of
 // large groups only the pairs that may be inside their critical radius. All CTAs therefore take the
-// same decision and follow the same control flow: every cluster barrier is reached by all 8 CTAs the same number
-// of times. Level results are double-buffered by attempt parity. Cluster k takes the k-th entry of
+// same decision and follow the same control flow: every cluster barrier is reached by all 8 CTAs the
+// same number of times. Level results are double-buffered by attempt parity. Cluster k takes the k-th entry of
 // the large-group list that the grouping kernel writes.
 #include <cooperative_groups.h>
 

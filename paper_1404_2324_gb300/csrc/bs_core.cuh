@@ -42,16 +42,6 @@ struct BsSharedT {
 };
 using BsShared = BsSharedT<BS_GMAX>;
 
-// Acceleration of member q at positions pos by the slot's ttps threads (4, 2 or 1): thread tsub sums
-// the terms p = tsub, tsub + ttps, ... (p == q: the central mass; any other p the (1 - K)-weighted pull
-// of partner p, H_A, Eq. Ha) and is given the components it owns: thread c of 4 component c, threads 0
-// and 1 of 2 the components 0, 1 and 2, one thread all three. Every lane runs the same straight-line
-// code (the central mass is a partner at the origin with G m0 and weight 1; a partner outside rc gets
-// weight 0): lanes of one warp that took different branches would each pay for both, and an FP64 warp
-// instruction costs its sub-partition 64 cycles whatever its active lanes. The threads exchange what
-// they do not own, so a slot of 4 issues 3 additions for the sum and 4 instructions for its chain
-// step, where every thread holding every component took 6 and 6.
-//
 // What a term of member q and partner p (p == q: the central mass) takes besides their positions; the
 // thread's first one is formed once an attempt.
 struct BsTerm {
@@ -71,6 +61,16 @@ __device__ __forceinline__ BsTerm bs_term(const SH &sh, double Gm0, int g, int q
   t.sign = __double2hiint(gm) & 0x80000000;
   return t;
 }
+
+// Acceleration of member q at positions pos by the slot's ttps threads (4, 2 or 1): thread tsub sums
+// the terms p = tsub, tsub + ttps, ... (p == q: the central mass; any other p the (1 - K)-weighted pull
+// of partner p, H_A, Eq. Ha) and is given the components it owns: thread c of 4 component c, threads 0
+// and 1 of 2 the components 0, 1 and 2, one thread all three. Every lane runs the same straight-line
+// code (the central mass is a partner at the origin with G m0 and weight 1; a partner outside rc gets
+// weight 0): lanes of one warp that took different branches would each pay for both, and an FP64 warp
+// instruction costs its sub-partition 64 cycles whatever its active lanes. The threads exchange what
+// they do not own, so a slot of 4 issues 3 additions for the sum and 4 instructions for its chain
+// step, where every thread holding every component took 6 and 6.
 template <class SH>
 __device__ __forceinline__ void bs_accel(const SH &sh, const DevParams &P, const BsTerm &t0, double Gm0, int g, int q, int tsub,
                                          int ttps, const double (*pos)[3], bool q_alive, double (&acc)[3]) {

@@ -752,9 +752,9 @@ __device__ __noinline__ unsigned tp_bs_close(const TPSet &T, const DevParams &P,
 
 // The BS pass of a substep and the closing kick of every TP. Warps take the listed TPs first (the
 // front entries first, each alone on its sub-partition), integrate each over the substep and give
-// it its closing kick; then they take the other TPs, 32 at a time, for their closing kick. The
-// closing kick has the arithmetic of the first kick and reads the planets at the end of the
-// substep; h1 + h2 as in tp_close_update, hcm_last != 0 adds the step's last Sun drift.
+// it its closing kick (in FP64, as the first kick); then they take the other TPs, 64 at a time, for
+// their closing kick in fixed point. The closing kick reads the planets at the end of the substep;
+// h1 + h2 as in tp_close_update, hcm_last != 0 adds the step's last Sun drift.
 __global__ void __launch_bounds__(32 * TPB_WARPS, 1) k_tp_bs(Sim S, TPSet T, DevParams P, double tau, double h1,
                                                            double h2, double hcm_last) {
   constexpr int WPOS = TPB_WPOS;
