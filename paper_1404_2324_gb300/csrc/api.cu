@@ -61,7 +61,7 @@ bool alloc_sim(Sim &S, DevMem &mem, int n, int nsub) {
   S.afar = mem.get<double>(3 * np);
   kick_split(S.npad, num_sms(), &S.kch, &S.kchunk);
   S.part = mem.get<double>(nt * std::max(2 * nt, (size_t)S.kch) * 96);
-  S.pkick = mem.get<double>(nt * 3); S.pfin = mem.get<double>(nt * FIN_PER_TILE * 3);
+  S.pkick = mem.get<double>(nt * FIN_PER_TILE * 3); S.pfin = mem.get<double>(nt * FIN_PER_TILE * 3);
   S.cbm = mem.get<unsigned>(np * W); S.rowany = mem.get<unsigned>(W);
   S.ccnt = mem.get<int>(np); S.clist = mem.get<int>(np * CCAP);
   S.ebm = mem.get<unsigned>((size_t)nsub * np * W);
@@ -1503,8 +1503,7 @@ int genga_phase_kick(int n, double G, double pc, int kmode, int precise_div, con
   int *tmp = mem.get<int>(2 * ((size_t)S.npad * (S.npad - 1) / 2 + 1));
   if (mem.err != cudaSuccess) { mem.release(); return GENGA_ENOMEM; }
   launch_soa_setup(S, P, m, alive, x, nullptr, rc, n, st);
-  launch_kick(S, P, false, precise_div != 0, st);
-  launch_fin(S, P, FIN_INIT, precise_div != 0, 0.0, 0.0, a, n, st);
+  launch_kick_init(S, P, precise_div != 0, a, n, st);
   launch_bitmap_pairs(S.cbm, S.rowany, S.npad, S.W, tmp, S.npad * (S.npad - 1) / 2 + 1, dcnt, st);
   int cnt = 0;
   cudaMemcpyAsync(&cnt, dcnt, sizeof(int), cudaMemcpyDeviceToHost, st);

@@ -84,7 +84,7 @@ struct Sim {
   u64 *T, *rcsq;                 // [npad]; bits of (pc rc)^2 and rc^2
   double *afar;                  // [3 npad] far-field accelerations of the last kick
   double *part;                  // [nt * max(2 nt, kch) * 3 * 32] kick partial sums
-  double *pkick, *pfin;          // momentum partials [nt * 3] per tile, [nt * FIN_PER_TILE * 3] per k_fin CTA
+  double *pkick, *pfin;          // momentum partials before and after a kick [nt * FIN_PER_TILE * 3]
   unsigned *cbm, *rowany;        // candidate bitmap [npad * W], row-nonempty bits [W]
   int *ccnt, *clist;             // per-body candidate count [npad] and partners [npad * CCAP]
   unsigned *ebm;                 // encounter bitmaps [nsub * npad * W] (upper triangle)
@@ -641,7 +641,7 @@ __device__ __forceinline__ void sun_shift(const Sim &S, double h1, double h2, do
 #pragma unroll
     for (int c = 0; c < 3; ++c) a[c] = fma(h1, S.pfin[t * 3 + c], a[c]);
   if (h2 != 0.0)
-    for (int t = lane; t < S.nt; t += 32)
+    for (int t = lane; t < FIN_PER_TILE * S.nt; t += 32)
 #pragma unroll
       for (int c = 0; c < 3; ++c) a[c] = fma(h2, S.pkick[t * 3 + c], a[c]);
   const double s = segment_sum3<32>(a[0], a[1], a[2]);

@@ -38,6 +38,9 @@ void launch_kick(const Sim &S, const DevParams &P, bool full, bool precise, cuda
 // precise: which pair kernel wrote the partial sums
 void launch_fin(const Sim &S, const DevParams &P, FinMode mode, bool precise, double h1, double h2, double *aout,
                 int ald, cudaStream_t st, bool after = false);  // aout: accelerations [3][ald] of the S.n bodies, or null
+// the phase entry points' kick: accelerations aout [3][ald] of the S.n bodies and the candidates; the
+// bitmap, row bits and counts are clear on entry
+void launch_kick_init(const Sim &S, const DevParams &P, bool precise, double *aout, int ald, cudaStream_t st, bool after = false);
 void launch_hc(const Sim &S, double hcm, cudaStream_t st);  // after launch_fin
 // the fixed-point pair kernel's chunks of partners per tile, partners per chunk
 void kick_split(int npad, int sms, int *chunks, int *chunk, int systems = 1);

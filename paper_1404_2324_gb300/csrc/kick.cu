@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(128) k_kick_precise(Sim S, DevParams P, int fo
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       double p = warp_sum(mi * S.v[c * np + i]);
-      if (lane == 0) S.pkick[warp * 3 + c] = p;
+      if (lane < FIN_PER_TILE) S.pkick[(warp * FIN_PER_TILE + lane) * 3 + c] = lane == 0 ? p : 0.0;
     }
   }
   if (warp >= S.nwarps) return;
@@ -205,7 +205,9 @@ __global__ void __launch_bounds__(32 * KX_WARPS, KX_CTAS) k_kick_fx(Sim S, DevPa
     const int i = gwarp * 32 + lane;
     const double mi = S.m[i];
     const double p = segment_sum3<32>(mi * S.v[i], mi * S.v[np + i], mi * S.v[2 * np + i]);
-    if ((lane & 7) == 0 && lane < 24) S.pkick[gwarp * 3 + (lane >> 3)] = p;
+    // the tile's total in the first of its slots (k_kick_small fills them all)
+    if ((lane & 7) < FIN_PER_TILE && lane < 24)
+      S.pkick[(gwarp * FIN_PER_TILE + (lane & 7)) * 3 + (lane >> 3)] = (lane & 7) == 0 ? p : 0.0;
   }
   const int tgroups = (nt + TW - 1) / TW;
   int I, c0;
@@ -353,6 +355,95 @@ __global__ void __launch_bounds__(FIN_BODIES * LPB) k_fin(Sim S, DevParams P, do
 }
 
 // ---------------------------------------------------------------------------------------------
+// The kick of few bodies: one warp per body, a partner a lane, every ordered pair in FP64, so that no
+// sum has to wait for other warps. Bound by latency: at 32 bodies the fixed-point kernel's set-up (grid,
+// chunks, bound pass) is most of its 10 us. Measured against it: 10 steps of 32 bodies 613 -> 570 us, 6 of
+// 64 bodies 399 -> 379, a kick of 64 bodies without allocation, here in one kernel, 21.3 -> 15.8; beyond, the
+// FP64 pairs cost more than the set-up (6 steps of 100 bodies 433 -> 440 us, of 200 bodies 512 -> 548).
+// ---------------------------------------------------------------------------------------------
+constexpr int KS_MAX = 64;
+
+// The far sum of body i (all of it, weighted, if FULL) and, if NEAR, the weighted near sum, on the lanes
+// of segment_sum3; records the candidates (the rows are clear).
+template <bool FULL, bool NEAR>
+__device__ __forceinline__ void small_sums(const Sim &S, const DevParams &P, int i, bool record, double &far, double &near) {
+  const int lane = threadIdx.x & 31, np = S.npad;
+  double fx = 0.0, fy = 0.0, fz = 0.0, nx = 0.0, ny = 0.0, nz = 0.0;
+  if (S.alive[i]) {  // uniform within the warp, as the loop and its votes
+    const double xi = S.x[i], yi = S.x[np + i], zi = S.x[2 * np + i], Ai = S.A[i];
+    const u64 Ti = S.T[i], Qi = S.rcsq[i];
+    int cnt = 0, pairs = 0;
+    for (int w = 0; w < S.W; ++w) {
+      const int j = w * 32 + lane;
+      const bool act = j != i && S.alive[j];
+      const double dx = S.x[j] - xi, dy = S.x[np + j] - yi, dz = S.x[2 * np + j] - zi;
+      const double r2 = r2_exact(dx, dy, dz);
+      const u64 rb = dbits(r2);
+      const bool cand = act && rb < umax64(Ti, S.T[j]);
+      if (act) {
+        const double yr = rsqrt_refined(r2);
+        double g = S.gm[j] * (yr * yr * yr);
+        if ((FULL || (NEAR && cand)) && rb < umax64(Qi, S.rcsq[j])) {
+          double wB, wA;
+          changeover_w(r2 * yr, pmin(Ai, S.A[j]), P.kmode, wB, wA);
+          g *= wB;
+        }
+        if (FULL || !cand) { fx = fma(g, dx, fx); fy = fma(g, dy, fy); fz = fma(g, dz, fz); }
+        else if (NEAR) { nx = fma(g, dx, nx); ny = fma(g, dy, ny); nz = fma(g, dz, nz); }
+      }
+      const unsigned m = record ? __ballot_sync(0xffffffffu, cand) : 0u;
+      if (m) {
+        const int k = cnt + __popc(m & ((1u << lane) - 1u));
+        if (cand && k < CCAP) S.clist[i * CCAP + k] = j;
+        if (lane == 0) S.cbm[(size_t)i * S.W + w] = m;
+        cnt += __popc(m);
+        pairs += __popc(__ballot_sync(0xffffffffu, cand && j > i));
+      }
+    }
+    if (lane == 0 && cnt) {
+      S.ccnt[i] = cnt;
+      atomicOr(&S.rowany[i >> 5], 1u << (i & 31));
+      if (pairs) atomicAdd((unsigned long long *)&S.counters[C_CAND], (unsigned long long)pairs);
+    }
+  }
+  far = segment_sum3<32>(fx, fy, fz);
+  if (NEAR) near = segment_sum3<32>(nx, ny, nz);
+}
+
+// The pair kernel of a step (the arguments and the momentum as k_kick_fx); k_fin reads one sum a body.
+template <bool FULL>
+__global__ void __launch_bounds__(32 * FIN_BODIES) k_kick_small(Sim S, DevParams P, int force) {
+  wait_previous();
+  if (FULL && !force && S.flags[0] == 0) return;
+  __shared__ double s_pm[3][FIN_BODIES];
+  const int wi = threadIdx.x >> 5, lane = threadIdx.x & 31, np = S.npad, i = blockIdx.x * FIN_BODIES + wi;
+  const int c = lane >> 3;  // lanes 0, 8, 16 hold the components of the sums
+  const bool own = (lane & 7) == 0 && c < 3, moment = !FULL || force;
+  if (moment && own) s_pm[c][wi] = S.m[i] * S.v[c * np + i];
+  double far, near;
+  small_sums<FULL, false>(S, P, i, FULL ? (!force && S.flags[3] != 0) : true, far, near);
+  if (own) S.part[(size_t)(i >> 5) * 96 + c * 32 + (i & 31)] = far;
+  if (!moment) return;  // uniform
+  __syncthreads();
+  if (wi != 0) return;
+  double pm = c < 3 ? s_pm[c][lane & 7] : 0.0;
+#pragma unroll
+  for (int o = FIN_BODIES / 2; o > 0; o >>= 1) pm += __shfl_xor_sync(0xffffffffu, pm, o);
+  if (own) S.pkick[blockIdx.x * 3 + c] = pm;
+}
+
+// The whole kick of the phase entry points: accelerations [3][ald] of the S.n bodies and the candidates.
+__global__ void __launch_bounds__(32 * FIN_BODIES) k_kick_once(Sim S, DevParams P, double *aout, int ald) {
+  wait_previous();
+  const int lane = threadIdx.x & 31, i = blockIdx.x * FIN_BODIES + (threadIdx.x >> 5), c = lane >> 3;
+  double far, near;
+  small_sums<false, true>(S, P, i, true, far, near);
+  if ((lane & 7) == 0 && c < 3 && i < S.n) aout[(size_t)c * ald + i] = far + near;
+}
+
+static bool kick_is_small(const Sim &S, bool precise) { return S.npad <= KS_MAX && !precise; }
+
+// ---------------------------------------------------------------------------------------------
 void launch_rcrit(const Sim &S, const DevParams &P, double tau_abs, int check_reuse, cudaStream_t st) {
   k_rcrit<<<(S.npad + 127) / 128, 128, 0, st>>>(S, P, tau_abs, check_reuse);
 }
@@ -363,6 +454,10 @@ void launch_kick(const Sim &S, const DevParams &P, bool full, bool precise, cuda
     const int grid = ((S.nwarps > S.nt ? S.nwarps : S.nt) * 32 + 127) / 128;
     if (full) k_kick_precise<true><<<grid, 128, 0, st>>>(S, P, f);
     else k_kick_precise<false><<<grid, 128, 0, st>>>(S, P, 0);
+  } else if (kick_is_small(S, false)) {
+    auto *kernel = full ? k_kick_small<true> : k_kick_small<false>;
+    if (after) launch_after(kernel, S.nt * FIN_PER_TILE, 32 * FIN_BODIES, st, S, P, full ? f : 0);
+    else kernel<<<S.nt * FIN_PER_TILE, 32 * FIN_BODIES, 0, st>>>(S, P, full ? f : 0);
   } else {
     if (full) launch_kick_fx<true>(S, P, f, st, after);
     else launch_kick_fx<false>(S, P, 0, st, after);
@@ -381,11 +476,22 @@ static void fin_lanes(const Sim &S, const DevParams &P, double h1, double h2, do
 
 void launch_fin(const Sim &S, const DevParams &P, FinMode mode, bool precise, double h1, double h2, double *aout,
                 int ald, cudaStream_t st, bool after) {
-  const int nslot = precise ? 2 * S.nt : S.kch;  // partial-sum slots per tile of the pair kernel used
+  // partial-sum slots per tile of the pair kernel used
+  const int nslot = precise ? 2 * S.nt : (kick_is_small(S, false) ? 1 : S.kch);
   if (mode == FIN_CLOSE) fin_lanes<FIN_CLOSE>(S, P, h1, h2, aout, ald, nslot, st, after);
   else if (mode == FIN_CLOSE_ALL) fin_lanes<FIN_CLOSE_ALL>(S, P, h1, h2, aout, ald, nslot, st, after);
   else if (mode == FIN_OPEN) fin_lanes<FIN_OPEN>(S, P, h1, h2, aout, ald, nslot, st, after);
   else fin_lanes<FIN_INIT>(S, P, h1, h2, aout, ald, nslot, st, after);
+}
+
+void launch_kick_init(const Sim &S, const DevParams &P, bool precise, double *aout, int ald, cudaStream_t st, bool after) {
+  if (kick_is_small(S, precise)) {
+    if (after) launch_after(k_kick_once, S.nt * FIN_PER_TILE, 32 * FIN_BODIES, st, S, P, aout, ald);
+    else k_kick_once<<<S.nt * FIN_PER_TILE, 32 * FIN_BODIES, 0, st>>>(S, P, aout, ald);
+    return;
+  }
+  launch_kick(S, P, false, precise, st, false, after);
+  launch_fin(S, P, FIN_INIT, precise, 0.0, 0.0, aout, ald, st, true);
 }
 
 // Second Sun drift after the last substep: x += hcm * P, P the momentum before the closing kick.
@@ -394,7 +500,7 @@ __global__ void k_hc(Sim S, double hcm) {
   const int lane = threadIdx.x & 31;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   double p[3] = {0.0, 0.0, 0.0};
-  for (int t = lane; t < S.nt; t += 32)
+  for (int t = lane; t < FIN_PER_TILE * S.nt; t += 32)
     for (int c = 0; c < 3; ++c) p[c] += S.pkick[t * 3 + c];
   const double ps = segment_sum3<32>(p[0], p[1], p[2]);
 #pragma unroll

@@ -35,7 +35,7 @@ constexpr size_t O_RCSQ = O_T + align256(NA_NMAX * sizeof(u64));
 constexpr size_t O_AFAR = O_RCSQ + align256(NA_NMAX * sizeof(u64));
 constexpr size_t O_PART = O_AFAR + align256(3 * NA_NMAX * sizeof(double));
 constexpr size_t O_PKICK = O_PART + align256((size_t)NA_NT * NA_NT * 2 * 96 * sizeof(double));
-constexpr size_t O_PFIN = O_PKICK + align256(NA_NT * 3 * sizeof(double));
+constexpr size_t O_PFIN = O_PKICK + align256(NA_NT * FIN_PER_TILE * 3 * sizeof(double));
 constexpr size_t O_CBM = O_PFIN + align256(NA_NT * FIN_PER_TILE * 3 * sizeof(double));
 constexpr size_t O_ROWANY = O_CBM + align256((size_t)NA_NMAX * NA_W * sizeof(unsigned));
 constexpr size_t O_CCNT = O_ROWANY + align256(NA_W * sizeof(unsigned));
@@ -168,8 +168,7 @@ extern "C" int genga_kick_noalloc(int n, double G, double pc, int kmode, int pre
   if (precise_div) k_items<<<1, 32, 0, st>>>(S.items, S.nt);
   // 8 threads a body: the bitmap's words, up to 32 a body, are most of what there is to clear
   k_kick_setup<<<(8 * S.npad + 127) / 128, 128, 0, st>>>(S, G, pc, m, alive, x, rc, n);
-  launch_kick(S, P, false, precise_div != 0, st, false, true);
-  launch_fin(S, P, FIN_INIT, precise_div != 0, 0.0, 0.0, a, n, st, true);
+  launch_kick_init(S, P, precise_div != 0, a, n, st, true);
   launch_bitmap_pairs(S.cbm, S.rowany, S.npad, S.W, cand, cap, ncand, st, true);
   return cudaGetLastError() == cudaSuccess ? GENGA_OK : GENGA_ECUDA;
 }

@@ -281,7 +281,7 @@ __device__ __forceinline__ void warp_load_planets(const Sim &S, double hcm_last,
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       double a = 0.0;
-      for (int t = lane; t < S.nt; t += 32) a += S.pkick[t * 3 + c];
+      for (int t = lane; t < FIN_PER_TILE * S.nt; t += 32) a += S.pkick[t * 3 + c];
       a = warp_sum(a);
       if (lane == 0) shc[c] = hcm_last * a;
     }
