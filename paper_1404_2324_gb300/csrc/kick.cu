@@ -6,6 +6,7 @@
 // root and division) evaluates every unordered pair once in FP64. Both leave partial sums per body
 // tile in a fixed layout that the finalisation sums in a fixed order, so results are bitwise
 // reproducible.
+#include "fxforce.cuh"
 #include "kick_fx.cuh"
 
 namespace genga {
@@ -245,13 +246,25 @@ static void launch_kick_fx(const Sim &S, const DevParams &P, int force, cudaStre
   else kernel<<<grid, 32 * KX_WARPS, 0, st>>>(S, P, force);
 }
 
+// r^-3 from r^2, on the integer pipes where r^2 is normal: rounded once, where the refined inverse root
+// cubed carries four roundings.
+__device__ __forceinline__ double inverse_cube(double r2) {
+  const int ex = (int)(dbits(r2) >> 52);
+  double y3, y5;
+  if (ex > 0 && ex < 0x7ff) fx::inverse_powers(r2, y3, y5);
+  else y3 = rcube_refined(r2);
+  return y3;
+}
+
 // The near-pair pull of partner j on body i, per unit separation, with the current critical radii
-// (refined inverse square root; the changeover weight as in the kick).
+// (the changeover weight as in the kick). ONCE: r^-3 rounded once, for the kick whose accelerations are
+// the result (1000 bodies: error 2.7-3.2e-16 against 3.0-3.7e-16); a step keeps the shorter chain.
+template <bool ONCE>
 __device__ __forceinline__ double near_factor(const Sim &S, const DevParams &P, u64 Qi, double Ai, int j, double r2) {
   const double yr = rsqrt_refined(r2);
   double wB = 1.0, wA;
   if (dbits(r2) < umax64(Qi, S.rcsq[j])) changeover_w(r2 * yr, pmin(Ai, S.A[j]), P.kmode, wB, wA);
-  return S.gm[j] * wB * (yr * yr * yr);
+  return S.gm[j] * wB * (ONCE ? inverse_cube(r2) : yr * yr * yr);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -330,7 +343,7 @@ __global__ void __launch_bounds__(FIN_BODIES * LPB) k_fin(Sim S, DevParams P, do
     for (int k = sl; k < cnt; k += LPB) {
       const int j = s_j[bi][k];
       const double dx = S.x[j] - xi, dy = S.x[np + j] - yi, dz = S.x[2 * np + j] - zi;
-      const double f = near_factor(S, P, Qi, Ai, j, r2_exact(dx, dy, dz));
+      const double f = near_factor<MODE == FIN_INIT>(S, P, Qi, Ai, j, r2_exact(dx, dy, dz));
       nx = fma(f, dx, nx); ny = fma(f, dy, ny); nz = fma(f, dz, nz);
     }
     a += segment_sum3<LPB>(nx, ny, nz);
@@ -358,7 +371,7 @@ __global__ void __launch_bounds__(FIN_BODIES * LPB) k_fin(Sim S, DevParams P, do
 // The kick of few bodies: one warp per body, a partner a lane, every ordered pair in FP64, so that no
 // sum has to wait for other warps. Bound by latency: at 32 bodies the fixed-point kernel's set-up (grid,
 // chunks, bound pass) is most of its 10 us. Measured against it: 10 steps of 32 bodies 613 -> 570 us, 6 of
-// 64 bodies 399 -> 379, a kick of 64 bodies without allocation, here in one kernel, 21.3 -> 15.8; beyond, the
+// 64 bodies 399 -> 379, a kick of 64 bodies without allocation, here in one kernel, 20.0 -> 17-19 (bound by submission); beyond, the
 // FP64 pairs cost more than the set-up (6 steps of 100 bodies 433 -> 440 us, of 200 bodies 512 -> 548).
 // ---------------------------------------------------------------------------------------------
 constexpr int KS_MAX = 64;
@@ -381,11 +394,10 @@ __device__ __forceinline__ void small_sums(const Sim &S, const DevParams &P, int
       const u64 rb = dbits(r2);
       const bool cand = act && rb < umax64(Ti, S.T[j]);
       if (act) {
-        const double yr = rsqrt_refined(r2);
-        double g = S.gm[j] * (yr * yr * yr);
+        double g = S.gm[j] * (NEAR ? inverse_cube(r2) : rcube_refined(r2));
         if ((FULL || (NEAR && cand)) && rb < umax64(Qi, S.rcsq[j])) {
           double wB, wA;
-          changeover_w(r2 * yr, pmin(Ai, S.A[j]), P.kmode, wB, wA);
+          changeover_w(r2 * rsqrt_refined(r2), pmin(Ai, S.A[j]), P.kmode, wB, wA);
           g *= wB;
         }
         if (FULL || !cand) { fx = fma(g, dx, fx); fy = fma(g, dy, fy); fz = fma(g, dz, fz); }
