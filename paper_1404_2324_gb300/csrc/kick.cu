@@ -370,9 +370,10 @@ __global__ void __launch_bounds__(FIN_BODIES * LPB) k_fin(Sim S, DevParams P, do
 // ---------------------------------------------------------------------------------------------
 // The kick of few bodies: one warp per body, a partner a lane, every ordered pair in FP64, so that no
 // sum has to wait for other warps. Bound by latency: at 32 bodies the fixed-point kernel's set-up (grid,
-// chunks, bound pass) is most of its 10 us. Measured against it: 10 steps of 32 bodies 613 -> 570 us, 6 of
-// 64 bodies 399 -> 379, a kick of 64 bodies without allocation, here in one kernel, 20.0 -> 17-19 (bound by submission); beyond, the
-// FP64 pairs cost more than the set-up (6 steps of 100 bodies 433 -> 440 us, of 200 bodies 512 -> 548).
+// chunks, bound pass) is most of its 10 us. Measured against it: 10 steps of 32 bodies 613 -> 570 us, 6
+// of 64 bodies 399 -> 379; a kick of 64 bodies without allocation, here in one kernel, 20.0 -> 17-19 us
+// (bound by submission). Beyond, the FP64 pairs cost more than the set-up (6 steps of 100 bodies 433 ->
+// 440 us, of 200 bodies 512 -> 548).
 // ---------------------------------------------------------------------------------------------
 constexpr int KS_MAX = 64;
 

@@ -78,7 +78,8 @@ int scratch_address(unsigned char **out) {
 // call's contents): the candidate bitmap, row bits and counts, flags, status and counters. One launch
 // for what six fills, a copy and a set-up kernel took: the call was bound by the gaps between its
 // launches (n = 64: 32.6 -> 23.6 us; n = 1000: 62.5 -> 41.0 us, also from the pair list reading only
-// rows that have candidates).
+// rows that have candidates; 17-19 and 32.8 us with dependent launches and the one-kernel kick of few
+// bodies).
 __global__ void k_kick_setup(Sim S, double G, double pc, const double *m, const int *alive, const double *x,
                              const double *rc, int n) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x, nthr = gridDim.x * blockDim.x, np = S.npad;
