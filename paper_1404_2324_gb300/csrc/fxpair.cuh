@@ -223,9 +223,10 @@ FX_HD float mass_f(u64 M, int me, int me_max) {
 }
 
 // The units exponent A of a body's sums, from the single-precision bound B of its chunk (sum of
-// mass_f / r^2); the sum of the factors is then below 2^61.
+// mass_f / r^2 with the rough r^2, within 2^-12, so rounded up by 2^-10); the sum of the factors is then
+// below 2^61.
 FX_HD int units(float B, int me_max) {
-  int ex = ((f2i(B) >> 23) & 0xff) - 127;  // B in [2^ex, 2^(ex+1))
+  int ex = ((f2i(B * 1.001f) >> 23) & 0xff) - 127;  // the bound in [2^ex, 2^(ex+1))
   if (ex < -120) ex = -120;
   return ex + 1 + me_max - 120;
 }
@@ -296,8 +297,10 @@ FX_HD void pull(const Pos &i, const Pos &j, u64 M, int me, int A, bool use, Acc 
   const u64 Q = madu(hi32(M), hi32(W), pair64(hi32(cq), 0u));
   const u64 cf = madu(hi32(Q), lo32(F), mulu(lo32(Q), hi32(F)));
   const u64 C = madu(hi32(Q), hi32(F), pair64(hi32(cf), 0u));
-  const int sh = use ? A - me - 63 + 2 * kk : 64;
-  const u64 g = shr_clamp(C << 3, sh);
+  // C = M / (8 rho^2), in [2^58, 2^61] up to the error of U: the largest M at rho^2 = 0.5 passes 2^61, so
+  // the product keeps a spare bit on top; the smallest C with a factor below 2^61 leaves the shift at 0
+  const int sh = use ? A - me - 64 + 2 * kk : 64;
+  const u64 g = shr_clamp(C << 2, sh);
   const int gh = hi_s(g), gl = (int)lo32(g);
   acc.h[0] = mads(ax, gh, acc.h[0]); acc.h[1] = mads(ay, gh, acc.h[1]); acc.h[2] = mads(az, gh, acc.h[2]);
   acc.l[0] = mads(ax, gl, mads(bx, gh, acc.l[0]));
