@@ -87,11 +87,11 @@ __device__ __forceinline__ void bs_accel(const SH &sh, const DevParams &P, const
       const bool inside = dbits(r2) < t.cut;
       double f = 0.0;
       if (cen || inside) {
-        if (P.kmode == 0) {
+        if (bs_factor_is_fixed(r2, P.kmode)) {
           f = fx::pull_factor(r2, t.gm, t.A, cen, inside);
           f = __hiloint2double(__double2hiint(f) | t.sign, __double2loint(f));
         } else {
-          f = bs_factor_gradient(r2, cen ? Gm0 : sh.gm[p], pmin(sh.A[q], sh.A[p]), cen);
+          f = bs_factor_fp64(r2, cen ? Gm0 : sh.gm[p], pmin(sh.A[q], sh.A[p]), cen, P.kmode);
         }
       }
       a0 = fma(f, dx, a0); a1 = fma(f, dy, a1); a2 = fma(f, dz, a2);

@@ -96,19 +96,23 @@ FX_HD void inverse_powers(double r2, double &y3, double &y5) {
 #ifdef __CUDACC__
 // The factor of one Bulirsch-Stoer term from its r^2: the whole pull (central mass), the pull weighted
 // by W_A (inside the pair's critical radius), else 0 without evaluating anything. kmode 1 (the exact
-// gradient of H_B) keeps the FP64 form.
-static __device__ __noinline__ double bs_factor_gradient(double r2, double pref, double A, bool full) {
+// gradient of H_B) keeps the FP64 form, and so does an r^2 that has no normalised mantissa: for members
+// at one position it gives a finite factor, which their separation of zero then annuls.
+__device__ __forceinline__ bool bs_factor_is_fixed(double r2, int kmode) {
+  return kmode == 0 && (unsigned)__double2hiint(r2) >= 0x00100000u;
+}
+static __device__ __noinline__ double bs_factor_fp64(double r2, double pref, double A, bool full, int kmode) {
   const double yr = rsqrt_refined(r2);
-  const double w = full ? 1.0 : changeover_wA_clamped(r2 * yr, A, 1);
+  const double w = full ? 1.0 : changeover_wA_clamped(r2 * yr, A, kmode);
   return pref * w * (yr * yr * yr);
 }
 __device__ __forceinline__ double bs_factor(double r2, double pref, double A, bool full, bool inside, int kmode) {
   if (!full && !inside) return 0.0;
-  if (kmode == 0) {
+  if (bs_factor_is_fixed(r2, kmode)) {
     const double f = fx::pull_factor(r2, fx::num(pref), fx::num(A), full, inside);
     return __longlong_as_double(__double_as_longlong(f) | (__double_as_longlong(pref) & (long long)0x8000000000000000ULL));
   }
-  return bs_factor_gradient(r2, pref, A, full);
+  return bs_factor_fp64(r2, pref, A, full, kmode);
 }
 #endif
 }  // namespace genga

@@ -658,11 +658,11 @@ __device__ __forceinline__ void tp_force(const Sim &S, const TPSet &T, const Dev
   double r2 = fma(dz, dz, fma(dy, dy, dx * dx)), g = 0.0;
   const bool inside = up && B.live && dbits(r2) < B.cut;
   if (!up || inside) {
-    if (P.kmode == 0) {
+    if (bs_factor_is_fixed(r2, P.kmode)) {
       const double f = fx::pull_factor(r2, B.gm_n, B.A_n, !up, inside);
       g = __longlong_as_double(__double_as_longlong(f) | (__double_as_longlong(B.gm) & (long long)0x8000000000000000ULL));
     } else {
-      g = bs_factor_gradient(r2, B.gm, B.A, !up);
+      g = bs_factor_fp64(r2, B.gm, B.A, !up, P.kmode);
     }
   }
   const double tx = g * dx, ty = g * dy, tz = g * dz;  // the Sun's: -G m0 y / |y|^3
