@@ -265,17 +265,17 @@ FX_HD u64 unit(i64 d, u32 U, int s) {
 #endif
 }
 
-// One partner: adds M_j's pull at (dX, dY, dZ) to the sums. use: false leaves the partner out.
-FX_HD void pull(const Pos &i, const Pos &j, u64 M, int me, int A, bool use, Acc &acc) {
+// One partner: adds the pull of M_j to the sums, from the separation (dX, dY, dZ) and the same in single
+// precision (fx, fy, fz; units of 2^32). use: false leaves the partner out.
+FX_HD void pull(float fx, float fy, float fz, i64 dX, i64 dY, i64 dZ, u64 M, int me, int A, bool use, Acc &acc) {
   // single precision: r^2 in units of 2^64, its exponent, the inverse square root
-  const float fx = (j.hx - i.hx) + (j.mx - i.mx), fy = (j.hy - i.hy) + (j.my - i.my), fz = (j.hz - i.hz) + (j.mz - i.mz);
   const float r2 = ffma(fz, fz, ffma(fy, fy, fx * fx));
   const int eb = f2i(r2), kk = eb >> 24;                      // r = rho 2^(kk - 63)
   const float rho2 = i2f(eb - (kk << 24) + (126 << 23));      // in [0.5, 2)
   const float u2 = frsqrt(rho2) + 2.0f;
   const u32 U2 = (u32)f2i(u2) << 9, U = U2 >> 2;              // 2^31 / rho, 2^29 / rho: 23 bits
   // unit vector, |v| = 2^61: the 96-bit products d U, shifted down by their exponent (21 .. 31)
-  const u64 vx = unit(j.X - i.X, U, kk - 63), vy = unit(j.Y - i.Y, U, kk - 63), vz = unit(j.Z - i.Z, U, kk - 63);
+  const u64 vx = unit(dX, U, kk - 63), vy = unit(dY, U, kk - 63), vz = unit(dZ, U, kk - 63);
   const int ax = hi_s(vx), ay = hi_s(vy), az = hi_s(vz);
   const int bx = (int)lo32(vx), by = (int)lo32(vy), bz = (int)lo32(vz);
   // e = 1 - |v|^2, in 2^-58
@@ -306,6 +306,11 @@ FX_HD void pull(const Pos &i, const Pos &j, u64 M, int me, int A, bool use, Acc 
   acc.l[0] = mads(ax, gl, mads(bx, gh, acc.l[0]));
   acc.l[1] = mads(ay, gl, mads(by, gh, acc.l[1]));
   acc.l[2] = mads(az, gl, mads(bz, gh, acc.l[2]));
+}
+
+FX_HD void pull(const Pos &i, const Pos &j, u64 M, int me, int A, bool use, Acc &acc) {
+  pull((j.hx - i.hx) + (j.mx - i.mx), (j.hy - i.hy) + (j.my - i.my), (j.hz - i.hz) + (j.mz - i.mz), j.X - i.X, j.Y - i.Y,
+       j.Z - i.Z, M, me, A, use, acc);
 }
 
 // Rough r^2 (units of 2^64) of the first pass.

@@ -214,7 +214,7 @@ __global__ void __launch_bounds__(32 * KX_WARPS, KX_CTAS) k_kick_fx(Sim S, DevPa
   int I, c0;
   bool ali;
   double ax, ay, az;
-  const bool on = kx_block<TW>(
+  const bool on = kx_block<TW, true>(
       S.x, np, S.gm, S.alive, S.T, 0, np, nt, C, S.kchunk, blockIdx.x % tgroups, blockIdx.x / tgroups,
       [&](int i, int j, double &dx, double &dy, double &dz) { return kx_near<FULL>(S, P, i, j, record, dx, dy, dz); }, I, c0,
       ali, ax, ay, az);
