@@ -445,10 +445,11 @@ __device__ __forceinline__ void stumpff_d(double z, double &c0, double &c1, doub
 // 64-76 cycles, and the drift kernels are bound by their number) where Newton's iteration took 135. Measured for
 // 200003 bodies: 73.8 -> 53.7 us a call of the phase entry with the series in FP64, 45.9 us now.
 // A solution that the single-precision solve does not reach, or a step above 10^-6 of s, takes the
-// iteration in double precision: Newton steps until |ds| <= 4 ulp |s| or a tiny step stops shrinking
-// (rounding floor). Returns 0 on success, 1 when no convergence (state untouched).
+// iteration in double precision: one Halley step from the float root (if it was reached), then Newton
+// steps until |ds| <= 4 ulp |s| or a tiny step stops shrinking (rounding floor). Returns 0 on success, 1
+// when no convergence (state untouched).
 static __device__ __noinline__ int kepler_iterate(double mu, double r0, double u, double beta, double dt, double sd,
-                                                  int maxit, double *s_out, double *U) {
+                                                  bool halley, int maxit, double *s_out, double *U) {
   double c0, c1, c2, c3;
   float ds_prev = 3.0e38f;
   for (int it = 1; it <= maxit; ++it) {
@@ -456,7 +457,14 @@ static __device__ __noinline__ int kepler_iterate(double mu, double r0, double u
     const double s2 = sd * sd, mus2 = mu * s2;
     const double F = fma(r0 * sd, c1, fma(u * s2, c2, fma(mus2 * sd, c3, -dt)));
     const double Fp = fma(r0, c0, fma(u * sd, c1, mus2 * c2));
-    const double ds = F * rcp_refined(Fp);
+    double ds;
+    if (halley) {  // ds = 2 F F' / (2 F'^2 - F F''), F'' = (mu - beta r0) s c1 + u c0
+      const double Fpp = fma(fma(-beta, r0, mu) * sd, c1, u * c0);
+      ds = (2.0 * F * Fp) * rcp_refined(fma(2.0 * Fp, Fp, -F * Fpp));
+      halley = false;
+    } else {
+      ds = F * rcp_refined(Fp);
+    }
     const double snew = sd - ds;
     if (((dbits(snew) >> 52) & 0x7ffu) == 0x7ffu) return 1;  // not finite
     const float fa = fabsf(d2f_safe(ds)), fs = fabsf(d2f_safe(snew));
@@ -538,7 +546,7 @@ static __device__ int kepler_drift_dev(double mu, double mu2, double &x, double 
   }
   if (!done) {
     double Uk[4];
-    if (kepler_iterate(mu, r0, u, beta, dt, (fok && s != 0.0f) ? f2d_exact(s) : dt * ir0, maxit, &s1, Uk)) return 1;
+    if (kepler_iterate(mu, r0, u, beta, dt, (fok && s != 0.0f) ? f2d_exact(s) : dt * ir0, fok, maxit, &s1, Uk)) return 1;
     U0 = Uk[0]; U1 = Uk[1]; U2 = Uk[2]; U3 = Uk[3];
   }
   if (s_out) *s_out = s1;
