@@ -199,10 +199,16 @@ __device__ __forceinline__ double f2d_exact(float f) {
   return __hiloint2double((int)hi, (int)lo);
 }
 
-// float -> double, a zero or subnormal float to zero (corrections whose size it bounds)
+// float -> double, a zero or subnormal float to zero (corrections whose size it bounds); times 2^k
 __device__ __forceinline__ double f2d_flush(float f) {
   return (__float_as_uint(f) & 0x7f800000u) ? f2d_exact(f) : 0.0;
 }
+__device__ __forceinline__ double f2d_scaled(float f, int k) {
+  const u64 b = dbits(f2d_exact(f)) + ((u64)(unsigned)(k << 20) << 32);
+  return (__float_as_uint(f) & 0x7f800000u) ? __longlong_as_double((long long)b) : 0.0;
+}
+// 2^k, -126 <= k <= 126
+__device__ __forceinline__ float exp2_float(int k) { return __uint_as_float((unsigned)(127 + k) << 23); }
 
 // ---------------------------------------------------------------------------------------------
 // Refined reciprocal and inverse square roots (Householder iterations of order 3, i.e. the
@@ -533,8 +539,12 @@ static __device__ int kepler_drift_dev(double mu, double mu2, double &x, double 
     const double dn = -F * iq;
     const double dl = fma(dn, f2d_flush(hal), dn);
     if (fabsf(fdn) <= 1.0e-6f * fabsf(s) && fabsf(hal) <= 4.0e-6f) {
-      const float h2 = 0.5f * fdn * fdn, fb1 = fb * fU1;
-      const double q3 = f2d_flush(h2 * fU1), q2 = f2d_flush(h2 * fU0), q1 = f2d_flush(-h2 * fb1), q0 = f2d_flush(-h2 * fb * fU0);
+      // in units where s is of order 1 (a power of two, exact): their squares would leave the range of
+      // single precision where s is small (lengths in cm and times in days)
+      const int k = (int)((__float_as_uint(s) >> 23) & 0xffu) - 127;
+      const float up = exp2_float(k), dn1 = exp2_float(-k), d = fdn * dn1, h2 = 0.5f * d * d, u1 = fU1 * dn1, b = fb * up * up;
+      const double q3 = f2d_scaled(h2 * u1, 3 * k), q2 = f2d_scaled(h2 * fU0, 2 * k), q1 = f2d_scaled(-h2 * (b * u1), k),
+                   q0 = f2d_flush(-h2 * b * fU0);
       const double bU1 = beta * U1;
       U3 = U3 + fma(dl, U2, q3);
       U2 = U2 + fma(dl, U1, q2);

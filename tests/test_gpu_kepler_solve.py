@@ -1,4 +1,5 @@
-"""The Kepler solve where its shortened form hands over to the iteration."""
+"""The Kepler solve where its shortened form hands over or runs out of range: units in which the universal
+variable is tiny, and callers that allow few iterations."""
 import numpy as np
 import pytest
 import torch
@@ -29,6 +30,19 @@ def _drift(mu, dt, maxit, x, v):
     genga.genga_phase_kepler(n, mu, dt, maxit, dev(np.ones(n, np.int32)), X, V, fail)
     torch.cuda.synchronize()
     return aos(X), aos(V), fail.cpu().numpy()
+
+
+@pytest.mark.parametrize("p", [10, 30, 38, 42, -30])
+@pytest.mark.parametrize("dt", [6.0, -20.0])
+def test_drift_is_the_same_in_other_units_of_length(p, dt):
+    """Lengths 2^p times as large in number (p = 42: AU to 0.03 m; the universal variable goes to 10^-13):
+    every operation scales by a power of two, so the results are the same to the last bit."""
+    x, v, _ = _orbits(20000, 0.3)
+    x0, v0, f0 = _drift(G, dt, 30, x, v)
+    x1, v1, f1 = _drift(np.ldexp(G, 3 * p), dt, 30, np.ldexp(x, p), np.ldexp(v, p))
+    assert not f0.any() and not f1.any()
+    np.testing.assert_array_equal(np.ldexp(x1, -p), x0)
+    np.testing.assert_array_equal(np.ldexp(v1, -p), v0)
 
 
 def _stumpff(z):
