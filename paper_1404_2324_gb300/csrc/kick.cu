@@ -1,11 +1,12 @@
 // kick.cu -- critical radii (Eq. rcrit), the K-weighted pairwise kick with the prechecker
 // (Eq. Hb, Sect. 2.2 and 3.2 "Kick"), and its per-body finalisation (KickA/KickB reuse).
 //
-// Two pair kernels. k_kick_fx (the default) evaluates each body's pull from every partner in 64-bit
-// fixed point on the integer and FP32 pipes (fxpair.cuh). k_kick_precise (precise_div = 1: IEEE square
-// root and division) evaluates every unordered pair once in FP64. Both leave partial sums per body
-// tile in a fixed layout that the finalisation sums in a fixed order, so results are bitwise
-// reproducible.
+// Pair kernels. k_kick_fx (more than 64 bodies) evaluates each body's pull from every partner in 64-bit
+// fixed point on the integer and FP32 pipes (fxpair.cuh). k_kick_small (up to 64 bodies) and k_kick_once
+// (the same for the phase entry points, in one kernel with what follows) evaluate it in FP64, one warp
+// per body. k_kick_precise (precise_div = 1: IEEE square root and division; any size) evaluates every
+// unordered pair once in FP64. They leave partial sums per body tile in a fixed layout that the
+// finalisation sums in a fixed order, so results are bitwise reproducible.
 #include "fxforce.cuh"
 #include "kick_fx.cuh"
 
@@ -239,9 +240,9 @@ void kick_split(int npad, int sms, int *chunks, int *chunk, int systems) {
 
 template <bool FULL>
 static void launch_kick_fx(const Sim &S, const DevParams &P, int force, cudaStream_t st, bool after) {
-  const int tw = S.nt >= 8 ? 8 : (S.nt >= 4 ? 4 : (S.nt >= 2 ? 2 : 1)), cw = KX_WARPS / tw;
+  const int tw = S.nt >= 8 ? 8 : (S.nt >= 4 ? 4 : 2), cw = KX_WARPS / tw;  // at least three tiles
   const int grid = ((S.nt + tw - 1) / tw) * ((S.kch + cw - 1) / cw);
-  auto *kernel = tw == 8 ? k_kick_fx<FULL, 8> : (tw == 4 ? k_kick_fx<FULL, 4> : (tw == 2 ? k_kick_fx<FULL, 2> : k_kick_fx<FULL, 1>));
+  auto *kernel = tw == 8 ? k_kick_fx<FULL, 8> : (tw == 4 ? k_kick_fx<FULL, 4> : k_kick_fx<FULL, 2>);
   if (after) launch_after(kernel, grid, 32 * KX_WARPS, st, S, P, force);
   else kernel<<<grid, 32 * KX_WARPS, 0, st>>>(S, P, force);
 }
