@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(32 * KX_WARPS, KX_CTAS) k_ad_kick_fx(Sim S, Ad
   int I, c0;
   bool ali;
   double ax, ay, az;
-  if (!kx_block<TW, false>(S.x, NB, S.gm, S.alive, MODE == 1 ? S.T : S.rcsq, base, D.Np, T, C, kchunk, k % tgroups, k / tgroups,
+  if (!kx_block<TW, (TW < 8)>(S.x, NB, S.gm, S.alive, MODE == 1 ? S.T : S.rcsq, base, D.Np, T, C, kchunk, k % tgroups, k / tgroups,
                     near_pair, I, c0, ali, ax, ay, az))
     return;
   double *p = part + (((size_t)b * T + I) * C + c0) * 96 + lane;

@@ -141,8 +141,9 @@ __device__ __noinline__ void kx_far_wide(const KxShared<CAP> &sm, int cnt, const
 // with leading dimension ld. lim: squared limit radii (bits); a pair inside max(lim_i, lim_j), or
 // closer than the grid resolves, is near(i, j, dx, dy, dz)'s, which returns the pull's factor.
 // Returns false for a warp without a tile and chunk. All threads of the CTA call it.
-// OUT: the rare kx_far<true> as a call, otherwise in line: in line it cost 10 steps of 500 bodies 1.2%, as a
-// call the gradient over 20 steps of 64 systems of 256 bodies 0.3%.
+// OUT: the rare kx_far<true> as a call, otherwise in line. In line the kernel's code is longer, which short
+// launches pay for: 10 steps of 500 bodies +1.2%, gradients of systems of up to seven tiles +1.6%; as a
+// call the gradient of 64 systems of eight tiles +0.3%.
 template <int TW, bool OUT, class Near>
 __device__ __forceinline__ bool kx_block(const double *__restrict__ X, int ld, const double *__restrict__ gm,
                                          const int *__restrict__ alive, const u64 *__restrict__ lim, int base, int np,
