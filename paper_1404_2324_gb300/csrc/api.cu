@@ -163,7 +163,7 @@ struct genga_ctx {
   cudaStream_t side = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   int gsplit = BS_GMAX + 1, cl_grid = 0, pair_grid = 0;
-  bool roomy = false;  // the BS kernels may take an SM per CTA (bs.cu)
+  bool roomy = false;  // few enough groups that the BS kernels may take an SM per CTA (bs.cu)
   // a further branch: groups above BS_GMAX members (main mode; the larger batched groups too)
   cudaStream_t side2 = nullptr;
   cudaEvent_t ev_join2 = nullptr;
@@ -222,6 +222,12 @@ void drop_graph(genga_ctx *c) {
 
 // The first kick (Sect. 2.2): critical radii, far-field accelerations and candidates of the
 // current state, with no velocity change. Also run after set_state / set_params.
+// One system's number of groups grows with its bodies and with their critical radii: k_bs<256, 32, 1> (an SM
+// a group) against k_bs<256, 32, 2>, 10 steps: 600 bodies 827 against 844 us at n2 = 0.4, 1033 against
+// 1041 at 1.0, 608 bodies 1683 against 1597 at 1.5, 1000 bodies 1.008 times as fast at 0.4, 2048 bodies
+// slower (bs.cu).
+bool few_groups(const genga_ctx *c) { return c->n <= 608 && c->prm.n2 <= 1.0; }
+
 int first_kick(genga_ctx *c) {
   Sim &S = c->S;
   cudaStream_t st = c->stream;
@@ -499,7 +505,7 @@ int genga_init(genga_ctx **out, int n, const double *masses, const double *radii
     genga_free(c);
     return GENGA_ECUDA;
   }
-  c->roomy = c->n <= 608;
+  c->roomy = few_groups(c);
   c->gsplit = 5;  // measured: from 5 members on, a cluster per group beats one CTA per group
   c->cl_grid = bs_cluster_grid();
   bs_grid_init_constants();
@@ -704,7 +710,7 @@ static int init_batch_one(genga_ctx **out, int n_sys, const int *offsets, const 
   // the pair kernel (4 groups per CTA) takes one CTA per SM, which leaves the other register half of
   // every SM to k_bs from the start: at two per SM it held the whole GPU and k_bs, the longer branch,
   // began 0.5 ms later (measured: 3.06M -> 3.15M system-steps/s)
-  c->roomy = true;
+  c->roomy = true;  // up to 1023 systems: 4 steps of 300 systems 2221 against 2367 us, 1023 systems 3122 against 3325
   c->pair_grid = num_sms();
   // groups of 3..BS_SMALL members (most of those above pairs) on 128-thread CTAs: two fit beside a
   // pair CTA in the register file where one 256-thread CTA did; the few larger groups take a half grid
@@ -1044,6 +1050,7 @@ int genga_set_params(genga_ctx *c, const genga_params *p) {
     return rc == GENGA_OK ? parts_join(c) : rc;
   }
   c->prm = *p;
+  if (!c->batched) c->roomy = few_groups(c);
   c->P = make_params(c->G, c->m0, c->prm);
   drop_graph(c);
   return c->batched ? first_kick_batch(c) : first_kick(c);

@@ -30,10 +30,11 @@ __device__ __forceinline__ int batch_group(const Sim &S, int qi, int q) {
 // reports larger ones than GM; it takes its groups from batched queue qi, else from the
 // large-group list (from_big), else every group with a fixed stride.
 // MINB: CTAs per SM that the registers are shared out for. Two 256-thread CTAs (128 registers a
-// thread) spill some 60 bytes in the chain of evaluations; where every group finds an SM of its own
-// (`roomy`: one system of at most 608 bodies, a batch in one part) one CTA per SM without spills is
-// faster: 10 steps of 500 bodies 884 -> 858 us, 300 systems x 4 steps 2149 -> 2071 us; not beyond (2048
-// bodies at fourth order 1677 -> 1856 us, 8192 systems 6.78 -> 7.19 ms).
+// thread) spill some 60 bytes in the chain of evaluations; where there are few enough groups (`roomy`:
+// few_groups and init_batch_one in api.cu, with figures at the limits) one CTA per SM without spills (the
+// 128-thread form at three per SM: 24 bytes) is faster: 10 steps of 500 bodies 884 -> 858 us, 300 systems
+// x 4 steps 2149 -> 2071 us; not with more (2048 bodies at fourth order 1677 -> 1856 us, 8192 systems
+// 6.78 -> 7.19 ms).
 template <int NT, int GM, int MINB>
 __global__ void __launch_bounds__(NT, MINB)
     k_bs(Sim S, DevParams P, double tau, int gmin, int gsplit, int qi, int from_big) {

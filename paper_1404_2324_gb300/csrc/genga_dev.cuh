@@ -449,7 +449,8 @@ __device__ __forceinline__ void stumpff_d(double z, double &c0, double &c1, doub
 // One evaluation of the Stumpff series instead of two or three, in fixed point on the integer pipes
 // (fxmath.cuh), as 1/r0: about 68 FP64 instructions a drift (an FP64 instruction holds the sub-partition
 // 64-76 cycles, and the drift kernels are bound by their number) where Newton's iteration took 135. Measured for
-// 200003 bodies: 73.8 -> 53.7 us a call of the phase entry with the series in FP64, 45.9 us now.
+// 200003 bodies: 73.8 -> 53.7 us a call of the phase entry with the series in FP64, 46-49 us now (at 76
+// cycles an instruction 26 us would be FP64 issue alone).
 // A solution that the single-precision solve does not reach, or a step above 10^-6 of s, takes the
 // iteration in double precision: one Halley step from the float root (if it was reached), then Newton
 // steps until |ds| <= 4 ulp |s| or a tiny step stops shrinking (rounding floor). Returns 0 on success, 1
