@@ -93,3 +93,34 @@ def test_groups_of_three_and_four_with_failed_attempts_match_the_oracle(seed, sp
         steps += want["bs_steps"]
         coll += len(want["collisions"])
     assert steps > len(groups) and (coll > 0) == (R is not None)
+
+
+@pytest.mark.parametrize("seed", [4, 6, 9, 13])
+def test_mergers_of_groups_of_three_and_four_book_energy_mass_and_radius(seed):
+    """The inputs above whose members merge: per group the same mergers as the oracle, the survivors'
+    masses and radii, and the internal energy to ten times the oracle's own sensitivity (1e-9 at least,
+    the bound of the other groups' mergers)."""
+    x, v, m, Rr, groups = _clumps((3, 4) * 4, seed=seed, spread=0.0003, R=2e-5)
+    n = len(m)
+    alive, rc = np.ones(n, np.int32), np.full(n, 0.02)
+    p = O.params(G=ics.G_GAUSS, m0=1.0)
+    coll = 0
+    for g in groups:
+        g = np.asarray(g, np.int32)
+        want = O.bs_group(p, g, 6.0, m, Rr, alive, x, v, rc)
+        if not len(want["collisions"]):
+            continue
+        sens = 0.0
+        for k in range(4):
+            x2 = x * (1 + 1.1e-16 * np.random.default_rng(k).integers(-1, 2, x.shape))
+            sens = max(sens, abs(O.bs_group(p, g, 6.0, m, Rr, alive, x2, v, rc)["U"] - want["U"]))
+        X, V, M, RR, AL = soa(x), soa(v), dev(m), dev(Rr), dev(alive)
+        st, U = genga.genga_phase_bs(n, ics.G_GAUSS, 1.0, 6.0, 1e-12, 8, 30, 0, 1, 1, dev(np.array([0, len(g)], np.int32)),
+                                     dev(g), dev(rc), M, RR, AL, X, V)
+        assert st == 0
+        np.testing.assert_array_equal(AL.cpu().numpy(), want["alive"])
+        np.testing.assert_allclose(M.cpu().numpy(), want["m"], rtol=1e-15)
+        np.testing.assert_allclose(RR.cpu().numpy(), want["R"], rtol=1e-14)
+        assert abs(U - want["U"]) <= max(1e-9 * abs(want["U"]), 10 * sens), (U, want["U"], sens)
+        coll += len(want["collisions"])
+    assert coll > 0
