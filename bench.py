@@ -49,7 +49,8 @@ SEED = 2
 FMA_LANES_PER_SM_CLK = 2  # FP64 FMA lanes per SM per clock on GB300 (measured: 1.9-2.0 at load clocks)
 FLOPS_PER_PAIR = 20       # algorithmic flops per ordered pair of the kick (sqrt and division count 1)
 PROFILE_SUMMARY = os.path.join(ROOT, "profiles", "kick_disk2048_ncu.md")
-KICK_SOURCES = [os.path.join(ROOT, "paper_1404_2324_gb300", "csrc", f) for f in ("kick.cu", "kick_fx.cuh", "fxpair.cuh", "genga_dev.cuh")]
+KICK_SOURCES = [os.path.join(ROOT, "paper_1404_2324_gb300", "csrc", f)
+                for f in ("kick.cu", "kick_fx.cuh", "fxpair.cuh", "fxforce.cuh", "fxmath.cuh", "genga_dev.cuh")]
 
 
 def workload_config():

@@ -71,8 +71,8 @@ typedef struct genga_params {
   int kepler_maxit;     /* iteration cap of the universal Kepler solve (30) */
   int kmode;            /* 0: K multiplies the Newtonian pair force; 1: exact gradient of H_B */
   int collisions;       /* 1: perfect merging on contact (Sect. 3.2, Collisions) */
-  int precise_div;      /* 1: kick uses IEEE sqrt and division; 0: 64-bit fixed point, near pairs a
-                         * refined reciprocal square root */
+  int precise_div;      /* 1: kick uses IEEE sqrt and division; 0: 64-bit fixed point, and a refined
+                         * reciprocal square root for near pairs and for systems of up to 64 bodies */
   /* Ejections (Sect. 3.2): at the end of every step a body farther than rcut from its central mass
    * or closer than rcut_sun is removed (a ghost, as after a merger), its heliocentric state
    * recorded (genga_ejections) and the energy it takes away booked into U; test particles are
