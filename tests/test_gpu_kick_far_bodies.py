@@ -4,10 +4,12 @@ nor turn every pair into a near one. Bound and oracle as in test_gpu_kick_fixed.
 run here at the sizes of two to seven tiles, too (its n = 40 is the FP64 kernel's)."""
 import numpy as np
 import pytest
+import torch
 
 import oracle as O
 from paper_1404_2324_gb300 import genga, ics
-from tests.gpu_util import with_central
+from paper_1404_2324_gb300.adjoint import AdjointEngine
+from tests.gpu_util import pair_sims, rel_state_error, with_central
 from tests.test_gpu_kick_fixed import _case, _disk, _run
 
 pytestmark = pytest.mark.gpu
@@ -26,11 +28,18 @@ def _spread(kind, n):
     elif kind == "octaves":             # one body an octave outwards, to 2^30 times the disk
         k = np.arange(0, n, max(1, n // 30))[:30]
         x[k] *= (2.0 ** np.arange(len(k)))[:, None]
+    elif kind == "mixed":               # half of them spread, with ghosts, massless bodies and masses over decades
+        k = rng.choice(n, n // 2, replace=False)
+        x[k] *= np.exp(rng.uniform(0.0, np.log(1e4), len(k)))[:, None]
+        m *= 10.0 ** rng.uniform(-12, 0, n)
+        m[1::5] = 0.0
     elif kind == "inner":               # one body an octave inwards, to the central mass
         k = np.arange(0, n, max(1, n // 30))[:30]
         x[k] *= (0.5 ** np.arange(len(k)))[:, None]
         x[-1] = 0.0
     alive = np.ones(n, np.int32)
+    if kind == "mixed":
+        alive[::4] = 0
     return G, m, alive, x, np.full(n, 0.02)
 
 
@@ -49,7 +58,7 @@ def _check(G, m, alive, x, rc, kmode=0):
 
 
 @pytest.mark.parametrize("n", [70, 97, 200, 257, 1100, 2048])
-@pytest.mark.parametrize("kind", ["far1", "far3", "far40", "share10", "share50", "share100", "octaves", "inner"])
+@pytest.mark.parametrize("kind", ["far1", "far3", "far40", "share10", "share50", "share100", "octaves", "inner", "mixed"])
 def test_kick_of_radii_over_many_octaves(kind, n):
     _check(*_spread(kind, n))
 
@@ -58,6 +67,33 @@ def test_kick_of_radii_over_many_octaves(kind, n):
 @pytest.mark.parametrize("kind", ["decades", "giant", "outlier", "ghosts", "massless"])
 def test_kick_of_a_few_tiles(kind, n):
     _check(*_case(kind, n))
+
+
+@pytest.mark.parametrize("n", [100, 300])
+def test_steps_of_a_scattered_disk_match_the_oracle(n):
+    """A third of the bodies out to 4000 AU on the orbits of their new distance: one step of the main mode
+    (its opening kick weighs every pair) and of the differentiable engine."""
+    d = ics.disk2048(9, n=n, total_mass=2 * ics.M_EARTH * n / 2048)
+    rng = np.random.default_rng(n)
+    k = rng.choice(n, n // 3, replace=False)
+    f = np.exp(rng.uniform(0.0, np.log(1e3), len(k)))[:, None]
+    d["x"][k] *= f
+    d["v"][k] /= np.sqrt(f)
+    g, o = pair_sims(d, 4, steps=1)
+    err, same = rel_state_error(g, o)
+    g.close()
+    o.close()
+    assert same and err <= 1e-12
+    o = O.Sim(O.params(G=d["G"], m0=1.0, dt=d["dt"], order=2, collisions=0), d["m"], np.zeros(n), d["x"], d["v"])
+    o.step(1)
+    want = o.state()
+    o.close()
+    eng = AdjointEngine(np.ones(1), d["G"], d["dt"], 2, ckpt_every=1)
+    t = lambda q: torch.tensor(q[None], dtype=torch.float64, device="cuda")  # noqa: E731
+    xo, vo = eng.forward(t(d["x"]), t(d["v"]), t(d["m"]), 1)
+    eng.close()
+    for got, ref in ((xo, want["x"]), (vo, want["v"])):
+        assert np.max(np.linalg.norm(got[0].cpu().numpy() - ref, axis=1) / np.linalg.norm(ref, axis=1)) <= 1e-12
 
 
 def _kick_us(x, d):
